@@ -49,11 +49,9 @@
 // Drawing. x_n = 0 when u_n < q0 = max(p0, 0) / (max(p0, 0) + max(p1, 0))
 // (1/2 if both are <= 0); P[n] keeps the chosen branch unclipped.
 //
-// Layout. Every per-sample array is [entry][S] (sample index fastest), so a warp
-// always touches consecutive samples of one entry: 32 with one sample per lane,
-// 128 in the FP32 table updates, whose lanes hold 4 samples each (16-byte loads)
-// and whose warps take one entry of one 128-sample group, the groups along the
-// slow grid axis (all entries of a group in flight together share its rows in L2).
+// Layout. The samples form groups of SG; every per-sample table of a group is
+// [entry][SG] (sample fastest, see SG), so a warp always touches consecutive
+// samples of one entry: 32 VW of them, VW per lane.
 #include <cstdint>
 #include <cstdio>
 #include <cstdlib>
@@ -79,14 +77,27 @@ __host__ __device__ __forceinline__ uint64_t i_z5(int t, int i, int m) {        
     return cb(m - 1, 3) + cb(i - 1, 2) + (uint64_t)(t - 1);
 }
 
+// Samples per group. The per-sample tables of one group of SG consecutive samples
+// form one block ([entry][SG], sample fastest; Args::tab, gs elements per block),
+// so an entry's row is 512 bytes in FP32 and consecutive entries are neighbours
+// in memory. (With one row of all S samples per entry, neighbouring entries lay
+// 4 S bytes apart: at S = 8192 every warp's load opened another DRAM page.)
+constexpr int SG = 128;
+
+// First entry of each table inside a group's block.
+struct Tabs {
+    size_t chi, P, Pp, P1, P2, Z, Z5, G, Y, X, CA, CB, CC, T, entries;
+};
+
 template <class R>
 struct Args {
     const R *kap;          // spin cumulants, orders 1..K, gbs.h layout
     uint64_t off[6];       // order offsets of the cumulant table
     int M, K, S, opp, op1, op2;
-    R *chi, *P, *Pp, *P1, *P2, *Z, *Z5, *G, *Y, *X, *W;
-    R *CA, *CB, *CC;       // per-step coefficients [i][S]: chi_i Pp~[n-1][i+1], kappa(i,n) chi_i, kappa(i,n) chi_i Pp~[n-1][i+1]
-    R *T;                  // [C(M,2)][2][S] per-pair parts of the p1 order-3 term (see p2_kernel)
+    R *tab;                // the groups' tables
+    size_t gs;             // elements per group block (Tabs::entries x SG)
+    Tabs o;
+    R *W;
     float *At;             // tensor-core product: the step's rows, split and tiled (atc_kernel)
     const R *hs;           // per-variable half scale s_v / 2, hs[v], v = 1..M
     const R *lead;         // per-variable pairs (kappa'({v}), hs[v]) at lead[2v], lead[2v+1]
@@ -103,22 +114,29 @@ struct Args {
     int n_valid;           // samples of this chunk that are real
 };
 
+// The tables of one group, each shifted to the calling thread's (first) sample.
 template <class R>
-__device__ __forceinline__ R pp(const Args<R> &a, int x, int b, int s) {
-    return b > x ? R(1) : a.Pp[i_pp(x, b) * a.S + s];
-}
-template <class R>
-__device__ __forceinline__ R p1(const Args<R> &a, int x, int e, int s) {
-    return e == x ? a.P[(size_t)(x - 1) * a.S + s] : a.P1[i_p1(x, e) * a.S + s];
-}
-template <class R>
-__device__ __forceinline__ R p2(const Args<R> &a, int x, int e, int d, int s) {
-    return e == x ? p1(a, x - 1, d, s) : a.P2[i_p2(x, e, d) * a.S + s];
-}
-template <class R>
-__device__ __forceinline__ R chi(const Args<R> &a, int v, int s) {
-    return a.chi[(size_t)v * a.S + s];
-}
+struct Grp {
+    R *chi, *P, *Pp, *P1, *P2, *Z, *Z5, *G, *Y, *X, *CA, *CB, *CC, *T;
+    __device__ __forceinline__ Grp(const Args<R> &a, int s) {
+        R *b = a.tab + (size_t)(s / SG) * a.gs + (s % SG);
+        chi = b + a.o.chi * SG;
+        P = b + a.o.P * SG;
+        Pp = b + a.o.Pp * SG;
+        P1 = b + a.o.P1 * SG;
+        P2 = b + a.o.P2 * SG;
+        Z = b + a.o.Z * SG;
+        Z5 = b + a.o.Z5 * SG;
+        G = b + a.o.G * SG;
+        Y = b + a.o.Y * SG;
+        X = b + a.o.X * SG;
+        CA = b + a.o.CA * SG;
+        CB = b + a.o.CB * SG;
+        CC = b + a.o.CC * SG;
+        T = b + a.o.T * SG;
+    }
+};
+
 // Spins of one sample read from its packed bits; the current 32-bit word is
 // cached, so a loop over ascending variables loads one word per 32 of them.
 template <class R>
@@ -163,14 +181,6 @@ __device__ __forceinline__ R k3(const Args<R> &a, int j, int i, int n) {
     return a.kap[a.off[3] + cb(n - 1, 3) + cb(i - 1, 2) + (j - 1)];
 }
 
-// (x, y, z) -> decreasing order
-__device__ __forceinline__ void ord3(int x, int y, int z, int &p, int &q, int &r) {
-    if (x < y) { int t = x; x = y; y = t; }
-    if (y < z) { int t = y; y = z; z = t; }
-    if (x < y) { int t = x; x = y; y = t; }
-    p = x; q = y; r = z;
-}
-
 // Pair rank -> (hi, lo), hi > lo >= 0 (colex: rank = C(hi, 2) + lo). The root
 // estimate is taken in FP32 (GB300's FP64 pipe is narrow and every lane of the
 // table kernels decodes its pair) and corrected exactly by the loops.
@@ -185,45 +195,39 @@ __device__ __forceinline__ void pair_of(uint64_t r, int &hi, int &lo) {
 
 // ---------------------------------------------------------------- step t: Z rows
 
-// Rows of the product at step t and where each result goes. kbase = offset of the
-// row's segment in the cumulant table; dst = its output entry (or -1 for G).
-__device__ __forceinline__ void zrow(int K, int M, int t, uint64_t q, const uint64_t *off, uint64_t &kbase,
-                                     int &kind, uint64_t &dst) {
+// Row q of the product at step t: kbase = offset of its segment in the cumulant
+// table, dst = the entry of the group's block its result goes to.
+__device__ __forceinline__ void zrow(int K, int M, int t, uint64_t q, const uint64_t *off, const Tabs &o,
+                                     uint64_t &kbase, uint64_t &dst) {
     if (K == 3) {
         if (q == 0) {
             kbase = off[2] + cb(t - 1, 2);
-            kind = 0;
-            dst = 0;
+            dst = o.G;
         } else {
             const int n = t + (int)q;
             kbase = off[3] + cb(n - 1, 3) + cb(t - 1, 2);
-            kind = 1;
-            dst = i_z(t, n);
+            dst = o.Z + i_z(t, n);
         }
         return;
     }
     if (q == 0) {
         kbase = off[3] + cb(t - 1, 3);
-        kind = 0;
-        dst = 0;
+        dst = o.G;
     } else if (q <= (uint64_t)(M - t)) {
         const int n = t + (int)q;
         kbase = off[4] + cb(n - 1, 4) + cb(t - 1, 3);
-        kind = 1;
-        dst = i_z(t, n);
+        dst = o.Z + i_z(t, n);
     } else if (q <= 2 * (uint64_t)(M - t)) {
         // the pairs below t of the order-3 set {., ., n}: X_t(n) for the p1 update
         const int n = t + (int)(q - (uint64_t)(M - t));
         kbase = off[3] + cb(n - 1, 3);
-        kind = 3;
-        dst = i_z(t, n);
+        dst = o.X + i_z(t, n);
     } else {  // K = 5 only
         int hi, lo;
         pair_of(q - 1 - 2 * (uint64_t)(M - t), hi, lo);
         const int i = t + 1 + lo, m = t + 1 + hi;
         kbase = off[5] + cb(m - 1, 5) + cb(i - 1, 4) + cb(t - 1, 3);
-        kind = 2;
-        dst = i_z5(t, i, m);
+        dst = o.Z5 + i_z5(t, i, m);
     }
 }
 
@@ -241,13 +245,14 @@ __global__ void __launch_bounds__(ETB) w_kernel(Args<R> a, int t, int D) {
     const int r0 = blockIdx.y * per, r1 = r0 + per < D ? r0 + per : D;
     if (r0 >= r1) return;
     Spins<R> sp(a, s);
+    const Grp<R> tb(a, s);
     R *W = a.W + s;
     if (K == 3) {
         // W_t(d) = chi_d P1~[t-1][d], d = r + 1; d = t - 1 -> P~[t-2]
-        const R *q = a.P1 + (t >= 3 ? i_p1(t - 1, 1) : 0) * S + s;
+        const R *q = tb.P1 + (t >= 3 ? i_p1(t - 1, 1) : 0) * SG;
         for (int r = r0; r < r1; ++r) {
             const int d = r + 1;
-            const R v = d == t - 1 ? a.P[(size_t)(t - 2) * S + s] : q[(size_t)r * S];
+            const R v = d == t - 1 ? tb.P[(size_t)(t - 2) * SG] : q[(size_t)r * SG];
             W[(size_t)r * S] = v * sp(d);
         }
         return;
@@ -260,11 +265,11 @@ __global__ void __launch_bounds__(ETB) w_kernel(Args<R> a, int t, int D) {
     int e = hi + 1, d = lo + 1;
     Spins<R> sd(a, s);
     const uint64_t rowlen = cb(t - 2, 2);
-    const R *q2 = a.P2 + (t >= 4 ? cb(t - 2, 3) : 0) * S + s;
+    const R *q2 = tb.P2 + (t >= 4 ? cb(t - 2, 3) : 0) * SG;
     for (int r = r0; r < r1; ++r) {
         R v;
-        if ((uint64_t)r < rowlen) v = q2[(size_t)r * S];
-        else v = d == t - 2 ? a.P[(size_t)(t - 3) * S + s] : a.P1[i_p1(t - 2, d) * S + s];
+        if ((uint64_t)r < rowlen) v = q2[(size_t)r * SG];
+        else v = d == t - 2 ? tb.P[(size_t)(t - 3) * SG] : tb.P1[i_p1(t - 2, d) * SG];
         W[(size_t)r * S] = v * sp(e) * sd(d);
         if (++d == e) {
             ++e;
@@ -285,14 +290,13 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
     __shared__ __align__(16) R Bs[2][BKt][BNt];
     __shared__ uint64_t kb[BMt];
     __shared__ uint64_t dst[BMt];
-    __shared__ int kind[BMt];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const uint64_t m0 = (uint64_t)blockIdx.x * BMt;
     const int s0 = blockIdx.y * BNt;
     for (int m = tid; m < BMt; m += 256) {
         const uint64_t q = m0 + m;
-        if (q < rows) zrow(K, a.M, t, q, a.off, kb[m], kind[m], dst[m]);
-        else kind[m] = -1;
+        if (q < rows) zrow(K, a.M, t, q, a.off, a.o, kb[m], dst[m]);
+        else kb[m] = ~0ull;
     }
     __syncthreads();
     // stage loaders: A element e = tid + 256 q -> (row e / 8, inner e % 8);
@@ -303,7 +307,7 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
 #pragma unroll
         for (int q = 0; q < AE; ++q) {
             const int e = tid + 256 * q, m = e / BKt, k = e % BKt;
-            ra[q] = (kind[m] >= 0 && k0 + k < D) ? a.kap[kb[m] + k0 + k] : R(0);
+            ra[q] = (kb[m] != ~0ull && k0 + k < D) ? a.kap[kb[m] + k0 + k] : R(0);
         }
         const R *w = a.W + (size_t)(k0 + bk) * a.S + s0 + bs;
 #pragma unroll
@@ -351,13 +355,10 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const int m = (i < 4 ? 0 : BMt / 2) + ty * 4 + (i & 3);
-        if (kind[m] < 0) continue;
-        R *out = kind[m] == 0 ? a.G
-               : kind[m] == 1 ? a.Z + dst[m] * a.S
-               : kind[m] == 2 ? a.Z5 + dst[m] * a.S
-                              : a.X + dst[m] * a.S;
+        if (kb[m] == ~0ull) continue;
+        R *out = a.tab + (size_t)(s0 / SG) * a.gs + dst[m] * SG + s0 % SG;  // the tile lies in one group
 #pragma unroll
-        for (int j = 0; j < TN; ++j) out[s0 + (j < 4 ? 0 : BNt / 2) + tx * 4 + (j & 3)] = acc[i][j];
+        for (int j = 0; j < TN; ++j) out[(j < 4 ? 0 : BNt / 2) + tx * 4 + (j & 3)] = acc[i][j];
     }
 }
 
@@ -482,9 +483,9 @@ __global__ void __launch_bounds__(ETB) wtc_kernel(Args<float> a, int t, int D) {
     Spins<float> sp(a, s), sd(a, s);
     // K = 4, 5: pair r = (e, d) with e < t - 1 is entry C(t-2, 3) + r of the p2
     // table (row t - 1 lists its pairs in colex order); e = t - 1 reads P1~[t-2][d]
-    const size_t S = (size_t)a.S;
+    const Grp<float> tb(a, s);
     const uint64_t rowlen = K == 3 ? 0 : cb(t - 2, 2);
-    const float *q2 = a.P2 + (K != 3 && t >= 4 ? cb(t - 2, 3) : 0) * S + s;
+    const float *q2 = tb.P2 + (K != 3 && t >= 4 ? cb(t - 2, 3) : 0) * SG;
     for (int qd = blockIdx.y; qd < Dp / 4; qd += gridDim.y) {
         const int r0 = 4 * qd;
         float v[4];
@@ -501,11 +502,11 @@ __global__ void __launch_bounds__(ETB) wtc_kernel(Args<float> a, int t, int D) {
             v[j] = 0.f;
             if (r < D) {
                 if (K == 3) {
-                    v[j] = p1(a, t - 1, r + 1, s) * sp(r + 1);
+                    v[j] = (r + 1 == t - 1 ? tb.P[(size_t)(t - 2) * SG] : tb.P1[i_p1(t - 1, r + 1) * SG]) * sp(r + 1);
                 } else {
-                    const float p = (uint64_t)r < rowlen ? q2[(size_t)r * S]
-                                    : d == t - 2         ? a.P[(size_t)(t - 3) * S + s]
-                                                         : a.P1[i_p1(t - 2, d) * S + s];
+                    const float p = (uint64_t)r < rowlen ? q2[(size_t)r * SG]
+                                    : d == t - 2         ? tb.P[(size_t)(t - 3) * SG]
+                                                         : tb.P1[i_p1(t - 2, d) * SG];
                     v[j] = p * sp(e) * sd(d);
                     if (++d == e) {  // next pair in colex order
                         ++e;
@@ -536,8 +537,7 @@ __global__ void __launch_bounds__(128) atc_kernel(Args<float> a, int t, uint64_t
     const int tid = threadIdx.x, rt = blockIdx.x, c = blockIdx.y, nk = gridDim.y;
     const uint64_t q = (uint64_t)rt * TC_M + tid;
     uint64_t kb = 0, dst = 0;
-    int kind = -1;
-    if (q < rows) zrow(K, a.M, t, q, a.off, kb, kind, dst);
+    if (q < rows) zrow(K, a.M, t, q, a.off, a.o, kb, dst);
     float *blk = a.At + ((size_t)rt * nk + c) * 2 * TC_ACH;
     const float *kp = a.kap + kb;
 #pragma unroll 2
@@ -545,7 +545,7 @@ __global__ void __launch_bounds__(128) atc_kernel(Args<float> a, int t, uint64_t
         const int k = c * TC_KC + j;
         float v[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = (kind >= 0 && k + i < D) ? kp[k + i] : 0.f;
+        for (int i = 0; i < 4; ++i) v[i] = (q < rows && k + i < D) ? kp[k + i] : 0.f;
         float4 h, l;
         h.x = to_tf32(v[0]); l.x = to_tf32(v[0] - h.x);
         h.y = to_tf32(v[1]); l.y = to_tf32(v[1] - h.y);
@@ -666,13 +666,11 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
     tc_fence_after();
     if (*flag) {
         uint64_t kb = 0, dst = 0;
-        int kind = -1;
-        if (m0 + tid < rows) zrow(K, a.M, t, m0 + tid, a.off, kb, kind, dst);
-        float *out = kind < 0    ? nullptr
-                   : kind == 0 ? a.G
-                   : kind == 1 ? a.Z + dst * a.S
-                   : kind == 2 ? a.Z5 + dst * a.S
-                               : a.X + dst * a.S;
+        float *out = nullptr;
+        if (m0 + tid < rows) {
+            zrow(K, a.M, t, m0 + tid, a.off, a.o, kb, dst);
+            out = a.tab + dst * SG;
+        }
         // The warp's 32 rows leave through shared memory (the ring is idle now):
         // a lane holds 32 columns of its own row after tcgen05.ld; the warp
         // writes them to a 32 x 36-float tile and reads them back as 8 lanes per
@@ -689,6 +687,8 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
         for (int cc = 0; cc < TC_N / 32; ++cc) {
+            const int sc = s0 + cc * 32;
+            const size_t col = (size_t)(sc / SG) * a.gs + sc % SG + c4;  // group block and sample within it
             uint32_t v[32];
             tc_ld32(lane_base + (uint32_t)(cc * 32), v);
             float4 *row = reinterpret_cast<float4 *>(tile + lane * 36);
@@ -700,7 +700,7 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const float4 w = *reinterpret_cast<const float4 *>(tile + (4 * i + rsub) * 36 + c4);
-                if (optr[i]) *reinterpret_cast<float4 *>(optr[i] + s0 + cc * 32 + c4) = w;
+                if (optr[i]) *reinterpret_cast<float4 *>(optr[i] + col) = w;
             }
             __syncwarp();
         }
@@ -710,144 +710,13 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_N) : "memory");
 }
 
-// ---------------------------------------------------------------- step n: bias and draw
-
-// K = 5: Y[i][s] = Z3_i(n) + sum_{3 <= j < i} chi_j Pp~[i-1][j+1] Z5_j(i, n), 3 <= i < n.
-template <class R>
-__global__ void __launch_bounds__(ETB) y_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
-    for (int i = 3 + blockIdx.y; i < n; i += gridDim.y) {
-        Spins<R> sp(a, s);
-        R y = a.Z[i_z(i, n) * a.S + s];
-        for (int j = 3; j < i; ++j) y = fma(sp(j) * pp(a, i - 1, j + 1, s), a.Z5[i_z5(j, i, n) * a.S + s], y);
-        a.Y[(size_t)i * a.S + s] = y;
-    }
-}
-
-template <class R, int K>
-__global__ void bias_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= a.S) return;
-    Spins<R> sp(a, s);
-    const R Pm = a.P[(size_t)(n - 1) * a.S + s];
-    R B = k1(a, n) * Pm;
-    if (K == 3) {
-        if (n >= 2) B += a.G[s];
-        for (int i = 2; i < n; ++i) B = fma(sp(i) * pp(a, n - 1, i + 1, s), a.Z[i_z(i, n) * a.S + s], B);
-    } else {
-        for (int i = 1; i < n; ++i) B = fma(k2(a, i, n) * sp(i), p1(a, n - 1, i, s), B);
-        if (n >= 3) B += a.G[s];
-        // K = 5: Y = Z3 + the order-5 part (y_kernel); K = 4: Z3 alone
-        const R *Yv = K == 5 ? a.Y : nullptr;
-        for (int i = 3; i < n; ++i)
-            B = fma(sp(i) * pp(a, n - 1, i + 1, s), K == 5 ? Yv[(size_t)i * a.S + s] : a.Z[i_z(i, n) * a.S + s], B);
-    }
-    const R hn = lead(a, n).y;
-    const R p0 = fma(hn, Pm, B), p1v = fma(hn, Pm, -B);
-    const R c0 = p0 > R(0) ? p0 : R(0), c1 = p1v > R(0) ? p1v : R(0);
-    const R q = (c0 + c1 > R(0)) ? c0 / (c0 + c1) : R(0.5);
-    int x = 0;
-    const bool real = s < a.n_valid;
-    if (real) {
-        const size_t o = (size_t)s * a.M + (n - 1);
-        if (a.force) x = a.force[o] ? 1 : 0;
-        else x = (a.u[o] < (double)q) ? 0 : 1;
-        a.bits[o] = (uint8_t)x;
-        if (a.q0) a.q0[o] = (double)q;
-    }
-    a.chi[(size_t)n * a.S + s] = x ? R(-1) : R(1);
-    if (x) a.bw[(size_t)(n >> 5) * a.S + s] |= 1u << (n & 31);
-    a.P[(size_t)n * a.S + s] = x ? p1v : p0;
-}
-
-// ---------------------------------------------------------------- step n: table rows
-// Thread per (entry, sample); the entry comes from blockIdx.y, so every index
-// below is uniform across a warp. These grids serve the FP64 calls (a few
-// hundred samples); FP32 runs the grouped forms further down (p2_kernel for
-// both, ppv/pvv/yv/p1v for FP32).
-
-// Order-3 part of the p+ update, factored: the term
-//   sum_{i > j >= l} kappa(j,i,n) chi_i chi_j chi_n Pp~[n-1][i+1] Pp~[i-1][j+1] Pp~[j-1][l]
-// equals chi_n sum_{j >= l} Pp~[j-1][l] v(j) with
-//   v(j) = chi_j sum_{i > j} kappa(j,i,n) chi_i Pp~[n-1][i+1] Pp~[i-1][j+1],
-// which does not depend on l. v goes to Y (free after the bias).
-template <class R>
-__global__ void __launch_bounds__(ETB) pv_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
-    for (int j = 1 + blockIdx.y; j < n; j += gridDim.y) {
-        Spins<R> sp(a, s);
-        R v = R(0);
-        for (int i = j + 1; i < n; ++i)
-            v = fma(k3(a, j, i, n) * sp(i) * pp(a, n - 1, i + 1, s), pp(a, i - 1, j + 1, s), v);
-        a.Y[(size_t)j * a.S + s] = v * sp(j);
-    }
-}
-
-// Pp~[n][l], l = 1..n (Eq. a / Eq. probpartialade).
-template <class R>
-__global__ void __launch_bounds__(ETB) pp_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
-    for (int l = 1 + blockIdx.y; l <= n; l += gridDim.y) {
-        Spins<R> sp(a, s);
-        const R cn = sp(n);
-        R acc = R(0);
-        if (a.opp >= 2)
-            for (int i = l; i < n; ++i)
-                acc = fma(k2(a, i, n) * sp(i) * pp(a, n - 1, i + 1, s), pp(a, i - 1, l, s), acc);
-        if (a.opp >= 3)
-            for (int j = l; j < n - 1; ++j) acc = fma(a.Y[(size_t)j * a.S + s], pp(a, j - 1, l, s), acc);
-        const auto ld = lead(a, n);
-        a.Pp[i_pp(n, l) * a.S + s] = fma(cn, acc, fma(ld.x, cn, ld.y) * pp(a, n - 1, l, s));
-    }
-}
-
-// Per-step coefficients of the table updates, one per (i < n, sample):
-//   CA = chi_i Pp~[n-1][i+1],  CB = kappa(i,n) chi_i,  CC = kappa(i,n) chi_i Pp~[n-1][i+1].
-template <class R>
-__global__ void __launch_bounds__(ETB) coef_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
-    for (int i = 1 + blockIdx.y; i < n; i += gridDim.y) {
-        Spins<R> sp(a, s);
-        const R ppv = pp(a, n - 1, i + 1, s), cbv = k2(a, i, n) * sp(i);
-        const size_t o = (size_t)i * a.S + s;
-        a.CA[o] = sp(i) * ppv;
-        a.CB[o] = cbv;
-        a.CC[o] = cbv * ppv;
-    }
-}
-
-// P1~[n][e], e = 1..n-1 (Eq. b / Eq. probelidedade).
-// K = 5, order 3: with (a, b, c) the decreasing order of (i, j, e), the terms with
-// a = e come from the product rows (X_e(n), times Pp~[n-1][e+1]); the others
-// (a = i > e) from the per-pair sums p2_kernel leaves in T.
-template <class R, int K>
-__global__ void __launch_bounds__(ETB) p1_kernel(Args<R> a, int n) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
-    const size_t S = (size_t)a.S;
-    for (int e = 1 + blockIdx.y; e < n; e += gridDim.y) {
-        Spins<R> sp(a, s);
-        const R cn = sp(n);
-        R acc = R(0);
-        if (a.op1 >= 2)
-            for (int i = 1; i < n; ++i) {
-                if (i == e) continue;
-                const int hi = i > e ? i : e, lo = i > e ? e : i;
-                const R g2 = k2(a, i, n) * sp(i);
-                if (K == 3) acc = fma(g2 * pp(a, n - 1, hi + 1, s), p1(a, hi - 1, lo, s), acc);
-                else acc = fma(g2, p2(a, n - 1, hi, lo, s), acc);
-            }
-        if (K >= 4 && a.op1 >= 3) {
-            if (e >= 3) acc = fma(pp(a, n - 1, e + 1, s), a.X[i_z(e, n) * S + s], acc);
-            // pairs (e, d), d < e, carry chi_d-weighted parts for e; pairs (j, e), j > e, for e
-            const R *T = a.T + s;
-            Spins<R> sd(a, s);
-            for (int d = 1; d < e; ++d) acc = fma(sd(d), T[(2 * (cb(e - 1, 2) + (uint64_t)(d - 1))) * S], acc);
-            for (int j = e + 1; j < n; ++j) acc = fma(sd(j), T[(2 * (cb(j - 1, 2) + (uint64_t)(e - 1)) + 1) * S], acc);
-        }
-        const auto ld = lead(a, n);
-        a.P1[i_p1(n, e) * S + s] = fma(cn, acc, fma(ld.x, cn, ld.y) * p1(a, n - 1, e, s));
-    }
-}
+// ---------------------------------------------------------------- table rows of one step
+// The kernels below take one table entry (or a few) and 32 VW consecutive samples
+// per warp, VW per lane, the sample groups on the slow grid axis, so that all
+// entries of a group are in flight together and its rows are shared in L2. Every
+// sum over earlier variables is one chain of FMAs per sample in ascending order,
+// whatever VW: the results don't depend on the schedule. The loads of a chain
+// don't depend on it, so walk() issues U of them ahead of the FMAs that use them.
 
 // VW consecutive samples of one lane, loaded and stored as one vector.
 template <class R, int VW>
@@ -864,15 +733,12 @@ __device__ __forceinline__ Lanes<R, VW> ldl(const R *p) {
         r.v[0] = q.x;
         r.v[1] = q.y;
     } else {
-        static_assert(VW % 4 == 0 && sizeof(R) == 4, "four or more lanes: float only");
-#pragma unroll
-        for (int h = 0; h < VW / 4; ++h) {
-            const float4 q = reinterpret_cast<const float4 *>(p)[h];
-            r.v[4 * h] = q.x;
-            r.v[4 * h + 1] = q.y;
-            r.v[4 * h + 2] = q.z;
-            r.v[4 * h + 3] = q.w;
-        }
+        static_assert(VW == 4 && sizeof(R) == 4, "four lanes: float only");
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        r.v[0] = q.x;
+        r.v[1] = q.y;
+        r.v[2] = q.z;
+        r.v[3] = q.w;
     }
     return r;
 }
@@ -886,18 +752,218 @@ __device__ __forceinline__ void stl(R *p, const R (&x)[VW]) {
         q.y = x[1];
         *reinterpret_cast<typename Pair2<R>::T *>(p) = q;
     } else {
-#pragma unroll
-        for (int h = 0; h < VW / 4; ++h)
-            reinterpret_cast<float4 *>(p)[h] = make_float4(x[4 * h], x[4 * h + 1], x[4 * h + 2], x[4 * h + 3]);
+        *reinterpret_cast<float4 *>(p) = make_float4(x[0], x[1], x[2], x[3]);
     }
 }
+template <class R, int VW>
+__device__ __forceinline__ Lanes<R, VW> ones() {
+    Lanes<R, VW> r;
+#pragma unroll
+    for (int k = 0; k < VW; ++k) r.v[k] = R(1);
+    return r;
+}
+
+// for i = i0 .. i1-1: use(i, load(i)), the loads of U terms issued before the
+// first of them is used (load may keep running offsets: it is called in order).
+template <int U, class Load, class Use>
+__device__ __forceinline__ void walk(int i0, int i1, Load load, Use use) {
+    using T = decltype(load(0));
+    int i = i0;
+    for (; i + U <= i1; i += U) {
+        T b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) b[u] = load(i + u);
+#pragma unroll
+        for (int u = 0; u < U; ++u) use(i + u, b[u]);
+    }
+    if (i < i1) {
+        T b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < i1) b[u] = load(i + u);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (i + u < i1) use(i + u, b[u]);
+    }
+}
+
+// C(i, 2) in 32 bits, i <= 4096.
+__device__ __forceinline__ unsigned c2u(int i) { return (unsigned)i * (unsigned)(i - 1) / 2u; }
+
 // Sample-independent part of the address of P2~[x][e][d] (with its boundary
 // cases P2~[x][x][d] = P1~[x-1][d], P1~[y][y] = P~[y-1]).
 template <class R>
-__device__ __forceinline__ const R *p2_row(const Args<R> &a, int x, int e, int d) {
-    const size_t S = (size_t)a.S;
-    if (e != x) return a.P2 + i_p2(x, e, d) * S;
-    return d == x - 1 ? a.P + (size_t)(x - 2) * S : a.P1 + i_p1(x - 1, d) * S;
+__device__ __forceinline__ const R *p2_row(const Grp<R> &t, int x, int e, int d) {
+    if (e != x) return t.P2 + i_p2(x, e, d) * SG;
+    return d == x - 1 ? t.P + (size_t)(x - 2) * SG : t.P1 + i_p1(x - 1, d) * SG;
+}
+// P1~[x][e] with P1~[x][x] = P~[x-1].
+template <class R>
+__device__ __forceinline__ const R *p1_row(const Grp<R> &t, int x, int e) {
+    return e == x ? t.P + (size_t)(x - 1) * SG : t.P1 + i_p1(x, e) * SG;
+}
+// Pp~[x][b] (1 when the range is empty, b > x).
+template <class R, int VW>
+__device__ __forceinline__ Lanes<R, VW> ppl(const Grp<R> &t, int x, int b) {
+    if (b > x) return ones<R, VW>();
+    return ldl<R, VW>(t.Pp + i_pp(x, b) * SG);
+}
+
+template <class R, int VW>
+struct Two {
+    Lanes<R, VW> c, v;
+};
+
+// K = 5: Y[i][s] = Z3_i(n) + sum_{3 <= j < i} chi_j Pp~[i-1][j+1] Z5_j(i, n), 3 <= i < n.
+template <class R, int VW, int U, int WPB>
+__global__ void __launch_bounds__(32 * WPB) yv_kernel(Args<R> a, int n) {
+    const int i = 3 + (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
+    if (i >= n) return;
+    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    Lanes<R, VW> y = ldl<R, VW>(t.Z + i_z(i, n) * SG);
+    const R *z5 = t.Z5 + i_z5(0, i, n) * SG, *q = t.Pp + (size_t)c2u(i - 1) * SG;  // Z5_j(i, n) and Pp~[i-1][j+1] at j
+    struct Three {
+        Lanes<R, VW> c, w, z;
+    };
+    walk<U>(
+        3, i,
+        [&](int j) {
+            return Three{ldl<R, VW>(t.chi + j * SG), j == i - 1 ? ones<R, VW>() : ldl<R, VW>(q + (size_t)j * SG),
+                         ldl<R, VW>(z5 + (size_t)j * SG)};
+        },
+        [&](int, const Three &b) {
+#pragma unroll
+            for (int k = 0; k < VW; ++k) y.v[k] = fma(b.c.v[k] * b.w.v[k], b.z.v[k], y.v[k]);
+        });
+    stl<R, VW>(t.Y + (size_t)i * SG, y.v);
+}
+
+// ---------------------------------------------------------------- step n: bias and draw
+// The bias of 32 samples per block. Its sums over i are one chain of FMAs per
+// sample, which one warp runs out of shared memory while all BIAS_W warps bring
+// in the next tile of its operands (a thread per sample that loads its own terms
+// waits for memory at every few of up to M steps of the chain: 340 us of a step
+// at M = 1152, K = 3, 256 samples). The same tiles leave the step's coefficient
+// rows behind, one per (i < n, sample):
+//   CA = chi_i Pp~[n-1][i+1],  CB = kappa(i,n) chi_i,  CC = kappa(i,n) chi_i Pp~[n-1][i+1].
+constexpr int BIAS_W = 16;
+
+template <class R, int K>
+__global__ void __launch_bounds__(32 * BIAS_W) bias_kernel(Args<R> a, int n) {
+    constexpr int TI = 256 / sizeof(R);  // i per tile
+    constexpr int PER = TI / BIAS_W;     // per thread
+    __shared__ R cs[2][TI][32], vs[2][TI][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, s = (int)blockIdx.x * 32 + lane;
+    const Grp<R> t(a, s);
+    const R *k2n = a.kap + a.off[2] + c2u(n - 1) - 1;       // kappa(i, n) at i
+    const R *ppn = t.Pp + (size_t)c2u(n - 1) * SG;          // Pp~[n-1][i+1] at i < n-1
+    const R *yz = K == 5 ? t.Y : t.Z + ((size_t)c2u(n - 1) - 1) * SG;  // Y_i, or Z_i(n), at i
+    R B = R(0), Pm = R(0);
+    if (w == 0) {
+        Pm = t.P[(size_t)(n - 1) * SG];
+        B = k1(a, n) * Pm;
+        if (K == 3 && n >= 2) B += t.G[0];
+    }
+    // pass 0 (K = 4, 5): kappa(i, n) chi_i P1~[n-1][i]; pass 1: chi_i Pp~[n-1][i+1] Y_i
+    // (K = 4: Z_i, from i = 3; K = 3: Z_i, from i = 2) and the coefficient rows
+#pragma unroll
+    for (int pass = K == 3 ? 1 : 0; pass < 2; ++pass) {
+        const int first = pass == 0 ? 1 : K == 3 ? 2 : 3;
+        R rc[PER], rv[PER];
+        auto load = [&](int i0) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = i0 + w + BIAS_W * q;
+                rc[q] = rv[q] = R(0);
+                if (i >= n) continue;
+                const R x = t.chi[(size_t)i * SG];
+                if (pass == 0) {
+                    rc[q] = k2n[i] * x;
+                    rv[q] = *p1_row(t, n - 1, i);
+                } else {
+                    const R p = i == n - 1 ? R(1) : ppn[(size_t)i * SG], cbv = k2n[i] * x, ca = x * p;
+                    if (K != 3) t.CA[(size_t)i * SG] = ca;
+                    t.CB[(size_t)i * SG] = cbv;
+                    t.CC[(size_t)i * SG] = cbv * p;
+                    rc[q] = ca;
+                    if (i >= first) rv[q] = yz[(size_t)i * SG];
+                }
+            }
+        };
+        load(1);
+        int buf = 0;
+        for (int i0 = 1; i0 < n; i0 += TI, buf ^= 1) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                cs[buf][w + BIAS_W * q][lane] = rc[q];
+                vs[buf][w + BIAS_W * q][lane] = rv[q];
+            }
+            __syncthreads();
+            if (i0 + TI < n) load(i0 + TI);
+            if (w == 0) {
+                const int hi = min(TI, n - i0);
+#pragma unroll 8
+                for (int q = max(0, first - i0); q < hi; ++q) B = fma(cs[buf][q][lane], vs[buf][q][lane], B);
+            }
+        }
+        if (K != 3 && pass == 0) {
+            if (w == 0 && n >= 3) B += t.G[0];
+            __syncthreads();  // the tiles are free again
+        }
+    }
+    if (w != 0) return;
+    const R hn = lead(a, n).y;
+    const R p0 = fma(hn, Pm, B), p1v = fma(hn, Pm, -B);
+    const R c0 = p0 > R(0) ? p0 : R(0), c1 = p1v > R(0) ? p1v : R(0);
+    const R q = (c0 + c1 > R(0)) ? c0 / (c0 + c1) : R(0.5);
+    int x = 0;
+    if (s < a.n_valid) {
+        const size_t o = (size_t)s * a.M + (n - 1);
+        if (a.force) x = a.force[o] ? 1 : 0;
+        else x = (a.u[o] < (double)q) ? 0 : 1;
+        a.bits[o] = (uint8_t)x;
+        if (a.q0) a.q0[o] = (double)q;
+    }
+    t.chi[(size_t)n * SG] = x ? R(-1) : R(1);
+    if (x) a.bw[(size_t)(n >> 5) * a.S + s] |= 1u << (n & 31);
+    t.P[(size_t)n * SG] = x ? p1v : p0;
+}
+
+// ---------------------------------------------------------------- step n: table rows
+
+// Order-3 part of the p+ update, factored: the term
+//   sum_{i > j >= l} kappa(j,i,n) chi_i chi_j chi_n Pp~[n-1][i+1] Pp~[i-1][j+1] Pp~[j-1][l]
+// equals chi_n sum_{j >= l} Pp~[j-1][l] v(j) with
+//   v(j) = chi_j sum_{i > j} kappa(j,i,n) chi_i Pp~[n-1][i+1] Pp~[i-1][j+1],
+// which does not depend on l. v goes to Y (free after the bias).
+template <class R, int VW, int U, int WPB>
+__global__ void __launch_bounds__(32 * WPB) pvv_kernel(Args<R> a, int n) {
+    const int j = 1 + (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
+    if (j >= n) return;
+    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    const R *k3n = a.kap + a.off[3] + cb(n - 1, 3) + (j - 1);  // kappa(j, i, n) at C(i-1, 2)
+    Lanes<R, VW> v;
+#pragma unroll
+    for (int k = 0; k < VW; ++k) v.v[k] = R(0);
+    struct Term {
+        Lanes<R, VW> c, q;
+        R k3;
+    };
+    walk<U>(
+        j + 1, n,
+        [&](int i) {
+            const unsigned o = c2u(i - 1);  // Pp~[i-1][j+1] is entry C(i-1, 2) + j
+            return Term{ldl<R, VW>(t.CA + (size_t)i * SG),
+                        i == j + 1 ? ones<R, VW>() : ldl<R, VW>(t.Pp + (size_t)(o + j) * SG), k3n[o]};
+        },
+        [&](int, const Term &b) {
+#pragma unroll
+            for (int k = 0; k < VW; ++k) v.v[k] = fma(b.k3 * b.c.v[k], b.q.v[k], v.v[k]);
+        });
+    const auto cj = ldl<R, VW>(t.chi + (size_t)j * SG);
+#pragma unroll
+    for (int k = 0; k < VW; ++k) v.v[k] = v.v[k] * cj.v[k];
+    stl<R, VW>(t.Y + (size_t)j * SG, v.v);
 }
 
 // P2~[n][e][d], n-1 >= e > d >= 1 (Eq. probdoubleelidedade).
@@ -909,351 +975,332 @@ __device__ __forceinline__ const R *p2_row(const Args<R> &a, int x, int e, int d
 // whose largest index is i (Eq. probelidedade with (a, b, c) = (i, e, d)): they
 // enter P1~[n][e] with weight CA[i] kappa(d,i,n) chi_d and P1~[n][d] with weight
 // CA[i] kappa(e,i,n) chi_e. Both sums are formed here, without chi_d / chi_e, and
-// left in T for p1_kernel, so each value is read once per step.
-// Schedule: one warp (one block) per pair (e, d) and 32 VW consecutive samples,
-// VW per lane (vector loads), the samples along the slow grid axis, so that the
-// pairs of one sample group run together and the three reads of each p2 value
-// (two in the row sums over i < e, one in the column sum over i > e) fall close
-// in time and are mostly served by L2. The kernel is bound by load latency: the
-// bounds cap it at 64 registers, so that 32 one-warp blocks (the per-SM block
-// limit) stay resident.
+// left in T for rows_kernel, so each value is read once per step.
+// Schedule: one warp (one block) per pair (e, d) and 32 VW consecutive samples.
+// The kernel is bound by load latency: the bounds cap it at 64 registers, so that
+// 32 one-warp blocks (the per-SM block limit) stay resident.
 template <class R, int VW>
 __global__ void __launch_bounds__(32, 32) p2_kernel(Args<R> a, int n) {
-    const int s = (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW;
-    const size_t S = (size_t)a.S;
-    const uint64_t nr = cb(n - 1, 2);
-    const R *P1 = a.P1 + s, *P2 = a.P2 + s, *P = a.P + s;
-    const R *CA = a.CA + s, *CB = a.CB + s, *CC = a.CC + s;
-    R cn[VW];
-    {
-        const uint32_t *bw = a.bw + (size_t)(n >> 5) * S + s;
-#pragma unroll
-        for (int k = 0; k < VW; ++k) cn[k] = (bw[k] >> (n & 31)) & 1u ? R(-1) : R(1);
-    }
+    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW);
+    const unsigned r = blockIdx.x;
+    int hi, lo;
+    pair_of(r, hi, lo);
+    const int e = hi + 1, d = lo + 1;
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
     const auto ld = lead(a, n);
-    for (uint64_t r = blockIdx.x; r < nr; r += gridDim.x) {
-        int hi, lo;
-        pair_of(r, hi, lo);
-        const int e = hi + 1, d = lo + 1;
-        R acc[VW], tE[VW], tD[VW];
+    R acc[VW], tE[VW], tD[VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = tE[k] = tD[k] = R(0);
+    for (int k = 0; k < VW; ++k) acc[k] = tE[k] = tD[k] = R(0);
+    if (a.op2 >= 2) {
+        R x[VW];
+#pragma unroll
+        for (int k = 0; k < VW; ++k) x[k] = R(0);
+        auto use = [&](int, const Two<R, VW> &b) {
+#pragma unroll
+            for (int k = 0; k < VW; ++k) x[k] = fma(b.c.v[k], b.v.v[k], x[k]);
+        };
+        // i < d: P2~[e-1][d][i]
+        const R *q = d < e - 1 ? t.P2 + i_p2(e - 1, d, 0) * SG : t.P1 + (e >= 3 ? i_p1(e - 2, 0) : 0) * SG;
+        const R *pb = t.P + (size_t)(e - 3) * SG;  // its boundary entry, i = d - 1 = e - 2
+        walk<4>(
+            1, d,
+            [&](int i) {
+                return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG),
+                                  ldl<R, VW>(d == e - 1 && i == e - 2 ? pb : q + (size_t)i * SG)};
+            },
+            use);
+        // d < i < e - 1: P2~[e-1][i][d]
+        const R *qc = t.P2 + (i_p2(e - 1, 1, 0) + d) * SG;
+        walk<4>(
+            d + 1, e - 1,
+            [&](int i) {
+                return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG), ldl<R, VW>(qc + (size_t)c2u(i - 1) * SG)};
+            },
+            use);
+        if (d < e - 1)
+            use(e - 1, Two<R, VW>{ldl<R, VW>(t.CB + (size_t)(e - 1) * SG), ldl<R, VW>(p1_row(t, e - 2, d))});
+        const auto w = ppl<R, VW>(t, n - 1, e + 1);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) acc[k] = w.v[k] * x[k];
+    }
+    if ((a.op2 >= 2 || a.op1 >= 3) && e + 1 < n) {
+        const R *k3n = a.kap + a.off[3] + cb(n - 1, 3) - 1;  // k3n[C(i-1,2) + j] = kappa(j, i, n)
+        R a2[VW];
+        // i = e + 1: P1~[e-1][d], or P~[e-2] when d = e - 1
+        {
+            const auto v = ldl<R, VW>(p1_row(t, e - 1, d));
+            const R *kp = k3n + c2u(e);
+            const R kd = kp[d], ke = kp[e];
+            const auto ca = ldl<R, VW>(t.CA + (size_t)(e + 1) * SG), cc = ldl<R, VW>(t.CC + (size_t)(e + 1) * SG);
+#pragma unroll
+            for (int k = 0; k < VW; ++k) {
+                a2[k] = cc.v[k] * v.v[k];
+                tE[k] = ca.v[k] * kd * v.v[k];
+                tD[k] = ca.v[k] * ke * v.v[k];
+            }
+        }
+        struct Col {
+            Lanes<R, VW> v, ca, cc;
+            R kd, ke;
+        };
+        const R *q = t.P2 + i_p2(e + 1, e, d) * SG;
+        walk<2>(
+            e + 2, n,
+            [&](int i) {
+                const R *kp = k3n + c2u(i - 1);
+                const Col b{ldl<R, VW>(q), ldl<R, VW>(t.CA + (size_t)i * SG), ldl<R, VW>(t.CC + (size_t)i * SG), kp[d], kp[e]};
+                q += (size_t)c2u(i - 2) * SG;
+                return b;
+            },
+            [&](int, const Col &b) {
+#pragma unroll
+                for (int k = 0; k < VW; ++k) {
+                    a2[k] = fma(b.cc.v[k], b.v.v[k], a2[k]);
+                    tE[k] = fma(b.ca.v[k] * b.kd, b.v.v[k], tE[k]);
+                    tD[k] = fma(b.ca.v[k] * b.ke, b.v.v[k], tD[k]);
+                }
+            });
         if (a.op2 >= 2) {
-            R t[VW];
 #pragma unroll
-            for (int k = 0; k < VW; ++k) t[k] = R(0);
-            // i < d: P2~[e-1][d][i]
-            if (d < e - 1) {
-                const R *q = P2 + i_p2(e - 1, d, 1) * S;
-#pragma unroll 4
-                for (int i = 1; i < d; ++i, q += S) {
-                    const auto c = ldl<R, VW>(CB + i * S), v = ldl<R, VW>(q);
-#pragma unroll
-                    for (int k = 0; k < VW; ++k) t[k] = fma(c.v[k], v.v[k], t[k]);
-                }
-            } else {
-                const R *q = P1 + (e >= 3 ? i_p1(e - 2, 1) : 0) * S;
-                for (int i = 1; i < d; ++i, q += S) {
-                    const auto c = ldl<R, VW>(CB + i * S), v = ldl<R, VW>(i == e - 2 ? P + (size_t)(e - 3) * S : q);
-#pragma unroll
-                    for (int k = 0; k < VW; ++k) t[k] = fma(c.v[k], v.v[k], t[k]);
-                }
-            }
-            // d < i < e: P2~[e-1][i][d]
-            if (d + 1 <= e - 2) {
-                uint64_t idx = i_p2(e - 1, d + 1, d);
-#pragma unroll 4
-                for (int i = d + 1; i < e - 1; ++i) {
-                    const auto c = ldl<R, VW>(CB + i * S), v = ldl<R, VW>(P2 + idx * S);
-#pragma unroll
-                    for (int k = 0; k < VW; ++k) t[k] = fma(c.v[k], v.v[k], t[k]);
-                    idx += (uint64_t)(i - 1);
-                }
-            }
-            if (d < e - 1) {
-                const auto c = ldl<R, VW>(CB + (e - 1) * S);
-                const auto v = ldl<R, VW>(d == e - 2 ? P + (size_t)(e - 3) * S : P1 + i_p1(e - 2, d) * S);
-#pragma unroll
-                for (int k = 0; k < VW; ++k) t[k] = fma(c.v[k], v.v[k], t[k]);
-            }
-            if (e + 1 > n - 1) {
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = t[k];
-            } else {
-                const auto w = ldl<R, VW>(a.Pp + i_pp(n - 1, e + 1) * S + s);
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = w.v[k] * t[k];
-            }
+            for (int k = 0; k < VW; ++k) acc[k] += a2[k];
         }
-        if ((a.op2 >= 2 || a.op1 >= 3) && e + 1 < n) {
-            const R *k3n = a.kap + a.off[3] + cb(n - 1, 3) - 1;  // k3n[C(i-1,2) + j] = kappa(j, i, n)
-            R a2[VW];
-            // i = e + 1: P1~[e-1][d], or P~[e-2] when d = e - 1
-            {
-                const auto v = ldl<R, VW>(d == e - 1 ? P + (size_t)(e - 2) * S : P1 + i_p1(e - 1, d) * S);
-                const R *kp = k3n + cb(e, 2);
-                const R kd = kp[d], ke = kp[e];
-                const auto ca = ldl<R, VW>(CA + (e + 1) * S), cc = ldl<R, VW>(CC + (e + 1) * S);
-#pragma unroll
-                for (int k = 0; k < VW; ++k) {
-                    a2[k] = cc.v[k] * v.v[k];
-                    tE[k] = ca.v[k] * kd * v.v[k];
-                    tD[k] = ca.v[k] * ke * v.v[k];
-                }
-            }
-            uint64_t idx = i_p2(e + 1, e, d);
-#pragma unroll 4
-            for (int i = e + 2; i < n; ++i) {
-                const auto v = ldl<R, VW>(P2 + idx * S);
-                const R *kp = k3n + cb(i - 1, 2);
-                const R kd = kp[d], ke = kp[e];
-                const auto ca = ldl<R, VW>(CA + i * S), cc = ldl<R, VW>(CC + i * S);
-#pragma unroll
-                for (int k = 0; k < VW; ++k) {
-                    a2[k] = fma(cc.v[k], v.v[k], a2[k]);
-                    tE[k] = fma(ca.v[k] * kd, v.v[k], tE[k]);
-                    tD[k] = fma(ca.v[k] * ke, v.v[k], tD[k]);
-                }
-                idx += cb(i - 2, 2);
-            }
-            if (a.op2 >= 2) {
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] += a2[k];
-            }
-        }
-        if (a.op1 >= 3) {
-            const uint64_t o = 2 * r;
-            stl<R, VW>(a.T + o * S + s, tE);
-            stl<R, VW>(a.T + (o + 1) * S + s, tD);
-        }
-        const auto pv = ldl<R, VW>(p2_row(a, n - 1, e, d) + s);
-        R out[VW];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) out[k] = fma(cn[k], acc[k], fma(ld.x, cn[k], ld.y) * pv.v[k]);
-        stl<R, VW>(a.P2 + i_p2(n, e, d) * S + s, out);
     }
+    if (a.op1 >= 3) {
+        stl<R, VW>(t.T + (size_t)(2 * r) * SG, tE);
+        stl<R, VW>(t.T + (size_t)(2 * r + 1) * SG, tD);
+    }
+    const auto pv = ldl<R, VW>(p2_row(t, n - 1, e, d));
+    R out[VW];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[k], fma(ld.x, cn.v[k], ld.y) * pv.v[k]);
+    stl<R, VW>(t.P2 + i_p2(n, e, d) * SG, out);
 }
 
-// Spins of VW consecutive samples from their packed bits (vector loads); the
-// current 32-bit words are cached as in Spins.
-template <class R, int VW>
-struct SpinsV {
-    const uint32_t *bw;
-    size_t S;
-    int s, w;
-    uint32_t cur[VW];
-    __device__ SpinsV(const Args<R> &a, int s_) : bw(a.bw), S((size_t)a.S), s(s_), w(-1) {}
-    __device__ __forceinline__ void operator()(int v, R (&x)[VW]) {
-        if ((v >> 5) != w) {
-            w = v >> 5;
-            const uint32_t *p = bw + (size_t)w * S + s;
-            if constexpr (VW == 4) {
-                const uint4 q = *reinterpret_cast<const uint4 *>(p);
-                cur[0] = q.x;
-                cur[1] = q.y;
-                cur[2] = q.z;
-                cur[3] = q.w;
-            } else if constexpr (VW == 2) {
-                const uint2 q = *reinterpret_cast<const uint2 *>(p);
-                cur[0] = q.x;
-                cur[1] = q.y;
-            } else {
-                cur[0] = *p;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < VW; ++k) x[k] = (cur[k] >> (v & 31)) & 1u ? R(-1) : R(1);
-    }
-};
-
-// P1~[n][e] (Eq. probelidedade; K = 3: Eq. b), the same sums as p1_kernel, one
-// warp per elided variable e and 32 VW consecutive samples (VW per lane), the
-// sample groups on the slow grid axis as in p2_kernel: each p2 value of row
-// n - 1 is read by the warps of e = hi and e = lo of the same group.
-template <class R, int K, int VW>
-__global__ void __launch_bounds__(32, 32) p1v_kernel(Args<R> a, int n) {
-    const int s = (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW;
-    const size_t S = (size_t)a.S;
-    R cn[VW];
-    {
-        SpinsV<R, VW> sn(a, s);
-        sn(n, cn);
-    }
+// Pp~[n][l], l0 <= l < l0 + LB (Eq. a / Eq. probpartialade): LB rows share each
+// coefficient load, and their p+ entries of one i are neighbours.
+template <class R, int VW, int U, int LB>
+__device__ __forceinline__ void pp_rows(const Args<R> &a, const Grp<R> &t, int n, int l0) {
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
     const auto ld = lead(a, n);
-    for (int e = 1 + (int)blockIdx.x; e < n; e += (int)gridDim.x) {
-        R acc[VW];
+    R acc[LB][VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = R(0);
-        if (a.op1 >= 2) {
-            SpinsV<R, VW> sp(a, s);
-            for (int i = 1; i < n; ++i) {
-                if (i == e) continue;
-                const int hi = i > e ? i : e, lo = i > e ? e : i;
-                R c[VW];
-                sp(i, c);
-                const R k2v = k2(a, i, n);
-                if (K == 3) {
-                    const auto q = ldl<R, VW>((lo == hi - 1 ? a.P + (size_t)(hi - 2) * S : a.P1 + i_p1(hi - 1, lo) * S) + s);
-                    if (hi + 1 > n - 1) {
+    for (int b = 0; b < LB; ++b)
 #pragma unroll
-                        for (int k = 0; k < VW; ++k) acc[k] = fma(k2v * c[k] * R(1), q.v[k], acc[k]);
-                    } else {
-                        const auto w = ldl<R, VW>(a.Pp + i_pp(n - 1, hi + 1) * S + s);
+        for (int k = 0; k < VW; ++k) acc[b][k] = R(0);
+    struct Row {
+        Lanes<R, VW> c, v[LB];
+    };
+    // coef rows (CC, then the order-3 factors Y) against Pp~[i-1][l], i in [l, hi)
+    auto sum = [&](const R *coef, int hi) {
+        // i within LB of l0: some rows have not begun, or begin with an empty range (1)
 #pragma unroll
-                        for (int k = 0; k < VW; ++k) acc[k] = fma(k2v * c[k] * w.v[k], q.v[k], acc[k]);
-                    }
-                } else {
-                    const auto q = ldl<R, VW>(p2_row(a, n - 1, hi, lo) + s);
+        for (int q = 0; q < LB; ++q) {
+            const int i = l0 + q;
+            if (i >= hi) break;
+            const auto c = ldl<R, VW>(coef + (size_t)i * SG);
 #pragma unroll
-                    for (int k = 0; k < VW; ++k) acc[k] = fma(k2v * c[k], q.v[k], acc[k]);
-                }
+            for (int b = 0; b <= q; ++b) {
+                const auto v = b == q ? ones<R, VW>() : ldl<R, VW>(t.Pp + (size_t)(c2u(i - 1) + l0 + b - 1) * SG);
+#pragma unroll
+                for (int k = 0; k < VW; ++k) acc[b][k] = fma(c.v[k], v.v[k], acc[b][k]);
             }
         }
-        if (K >= 4 && a.op1 >= 3) {
-            if (e >= 3) {
-                const auto x = ldl<R, VW>(a.X + i_z(e, n) * S + s);
-                if (e + 1 > n - 1) {
+        walk<U>(
+            l0 + LB, hi,
+            [&](int i) {
+                Row r;
+                r.c = ldl<R, VW>(coef + (size_t)i * SG);
+                const R *p = t.Pp + (size_t)(c2u(i - 1) + l0 - 1) * SG;
 #pragma unroll
-                    for (int k = 0; k < VW; ++k) acc[k] = fma(R(1), x.v[k], acc[k]);
-                } else {
-                    const auto w = ldl<R, VW>(a.Pp + i_pp(n - 1, e + 1) * S + s);
+                for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(p + (size_t)b * SG);
+                return r;
+            },
+            [&](int, const Row &r) {
 #pragma unroll
-                    for (int k = 0; k < VW; ++k) acc[k] = fma(w.v[k], x.v[k], acc[k]);
-                }
-            }
-            // pairs (e, d), d < e, carry chi_d-weighted parts for e; pairs (j, e), j > e, for e
-            const R *T = a.T + s;
-            SpinsV<R, VW> sd(a, s);
-            for (int d = 1; d < e; ++d) {
-                R c[VW];
-                sd(d, c);
-                const auto t = ldl<R, VW>(T + (2 * (cb(e - 1, 2) + (uint64_t)(d - 1))) * S);
+                for (int b = 0; b < LB; ++b)
 #pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = fma(c[k], t.v[k], acc[k]);
-            }
-            for (int j = e + 1; j < n; ++j) {
-                R c[VW];
-                sd(j, c);
-                const auto t = ldl<R, VW>(T + (2 * (cb(j - 1, 2) + (uint64_t)(e - 1)) + 1) * S);
+                    for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k], r.v[b].v[k], acc[b][k]);
+            });
+    };
+    if (a.opp >= 2) sum(t.CC, n);
+    if (a.opp >= 3) sum(t.Y, n - 1);
 #pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = fma(c[k], t.v[k], acc[k]);
-            }
-        }
-        const auto pv = ldl<R, VW>((e == n - 1 ? a.P + (size_t)(n - 2) * S : a.P1 + i_p1(n - 1, e) * S) + s);
+    for (int b = 0; b < LB; ++b) {
+        const int l = l0 + b;
+        if (l > n) break;
+        const auto w = ppl<R, VW>(t, n - 1, l);
         R out[VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) out[k] = fma(cn[k], acc[k], fma(ld.x, cn[k], ld.y) * pv.v[k]);
-        stl<R, VW>(a.P1 + i_p1(n, e) * S + s, out);
+        for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[b][k], fma(ld.x, cn.v[k], ld.y) * w.v[k]);
+        stl<R, VW>(t.Pp + i_pp(n, l) * SG, out);
     }
 }
 
-// Pp~[x][b] of VW consecutive samples (1 when the range is empty, b > x).
-template <class R, int VW>
-__device__ __forceinline__ Lanes<R, VW> ppl(const Args<R> &a, int x, int b, int s) {
-    if (b > x) {
-        Lanes<R, VW> r;
-#pragma unroll
-        for (int k = 0; k < VW; ++k) r.v[k] = R(1);
-        return r;
-    }
-    return ldl<R, VW>(a.Pp + i_pp(x, b) * (size_t)a.S + s);
-}
-
-// FP32 forms of y_kernel, pv_kernel and pp_kernel with the schedule of p2_kernel:
-// one warp per entry and 32 VW consecutive samples (VW per lane), the sample
-// groups on the slow grid axis; the same terms in the same order per sample.
-template <class R, int VW>
-__global__ void __launch_bounds__(32, 32) yv_kernel(Args<R> a, int n) {
-    const int s = (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW;
-    const size_t S = (size_t)a.S;
-    for (int i = 3 + (int)blockIdx.x; i < n; i += (int)gridDim.x) {
-        SpinsV<R, VW> sp(a, s);
-        const auto z = ldl<R, VW>(a.Z + i_z(i, n) * S + s);
-        R y[VW];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) y[k] = z.v[k];
-        for (int j = 3; j < i; ++j) {
-            R c[VW];
-            sp(j, c);
-            const auto w = ppl<R, VW>(a, i - 1, j + 1, s);
-            const auto z5 = ldl<R, VW>(a.Z5 + i_z5(j, i, n) * S + s);
-#pragma unroll
-            for (int k = 0; k < VW; ++k) y[k] = fma(c[k] * w.v[k], z5.v[k], y[k]);
-        }
-        stl<R, VW>(a.Y + (size_t)i * S + s, y);
-    }
-}
-
-template <class R, int VW>
-__global__ void __launch_bounds__(32, 32) pvv_kernel(Args<R> a, int n) {
-    const int s = (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW;
-    const size_t S = (size_t)a.S;
-    for (int j = 1 + (int)blockIdx.x; j < n; j += (int)gridDim.x) {
-        SpinsV<R, VW> sp(a, s);
-        R v[VW];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) v[k] = R(0);
-        for (int i = j + 1; i < n; ++i) {
-            R c[VW];
-            sp(i, c);
-            const R k3v = k3(a, j, i, n);
-            const auto w = ppl<R, VW>(a, n - 1, i + 1, s), q = ppl<R, VW>(a, i - 1, j + 1, s);
-#pragma unroll
-            for (int k = 0; k < VW; ++k) v[k] = fma(k3v * c[k] * w.v[k], q.v[k], v[k]);
-        }
-        R cj[VW];
-        sp(j, cj);
-#pragma unroll
-        for (int k = 0; k < VW; ++k) v[k] = v[k] * cj[k];
-        stl<R, VW>(a.Y + (size_t)j * S + s, v);
-    }
-}
-
-template <class R, int VW>
-__global__ void __launch_bounds__(32, 32) ppv_kernel(Args<R> a, int n) {
-    const int s = (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW;
-    const size_t S = (size_t)a.S;
-    R cn[VW];
-    {
-        SpinsV<R, VW> sn(a, s);
-        sn(n, cn);
-    }
+// K = 3: P1~[n][e], e0 <= e < e0 + LB (Eq. b), i < e with weight
+// kappa(i,n) chi_i Pp~[n-1][e+1] and i > e with CC_i. Rows e >= n are formed
+// from whatever lies there (in bounds: e0 < n <= M) and not stored.
+template <class R, int VW, int U, int LB>
+__device__ __forceinline__ void p1_rows_k3(const Args<R> &a, const Grp<R> &t, int n, int e0) {
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
     const auto ld = lead(a, n);
-    for (int l = 1 + (int)blockIdx.x; l <= n; l += (int)gridDim.x) {
-        R acc[VW];
+    const int nb = min(LB, n - e0);  // rows of this warp
+    R acc[LB][VW];
+    Lanes<R, VW> w[LB];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = R(0);
-        if (a.opp >= 2) {
-            SpinsV<R, VW> sp(a, s);
-            for (int i = l; i < n; ++i) {
-                R c[VW];
-                sp(i, c);
-                const R k2v = k2(a, i, n);
-                const auto w = ppl<R, VW>(a, n - 1, i + 1, s), q = ppl<R, VW>(a, i - 1, l, s);
+    for (int b = 0; b < LB; ++b) {
+        w[b] = ppl<R, VW>(t, n - 1, b < nb ? e0 + b + 1 : n);
 #pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = fma(k2v * c[k] * w.v[k], q.v[k], acc[k]);
-            }
+        for (int k = 0; k < VW; ++k) acc[b][k] = R(0);
+    }
+    struct Row {
+        Lanes<R, VW> c, v[LB];
+    };
+    // one term of row b for any i != e
+    auto any = [&](int b, int i, const Lanes<R, VW> &cbv, const Lanes<R, VW> &ccv) {
+        const int e = e0 + b;
+        if (i < e) {
+            const auto v = ldl<R, VW>(p1_row(t, e - 1, i));
+#pragma unroll
+            for (int k = 0; k < VW; ++k) acc[b][k] = fma(cbv.v[k] * w[b].v[k], v.v[k], acc[b][k]);
+        } else if (i > e) {
+            const auto v = ldl<R, VW>(p1_row(t, i - 1, e));
+#pragma unroll
+            for (int k = 0; k < VW; ++k) acc[b][k] = fma(ccv.v[k], v.v[k], acc[b][k]);
         }
-        if (a.opp >= 3)
-            for (int j = l; j < n - 1; ++j) {
-                const auto y = ldl<R, VW>(a.Y + (size_t)j * S + s), q = ppl<R, VW>(a, j - 1, l, s);
+    };
+    // i <= e0 - 2: P1~[e-1][i]
+    const R *rowp[LB];
 #pragma unroll
-                for (int k = 0; k < VW; ++k) acc[k] = fma(y.v[k], q.v[k], acc[k]);
-            }
-        const auto w = ppl<R, VW>(a, n - 1, l, s);
+    for (int b = 0; b < LB; ++b) rowp[b] = t.P1 + (e0 >= 3 ? (size_t)(c2u(e0 + (b < nb ? b : 0) - 2)) * SG : 0) - SG;
+    walk<U>(
+        1, e0 - 1,
+        [&](int i) {
+            Row r;
+            r.c = ldl<R, VW>(t.CB + (size_t)i * SG);
+#pragma unroll
+            for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(rowp[b] + (size_t)i * SG);
+            return r;
+        },
+        [&](int, const Row &r) {
+#pragma unroll
+            for (int b = 0; b < LB; ++b)
+#pragma unroll
+                for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k] * w[b].v[k], r.v[b].v[k], acc[b][k]);
+        });
+    // i around the rows' own indices: every case
+#pragma unroll
+    for (int q = 0; q < LB + 2; ++q) {
+        const int i = e0 - 1 + q;
+        if (i < 1 || i >= n) continue;
+        const auto cbv = ldl<R, VW>(t.CB + (size_t)i * SG), ccv = ldl<R, VW>(t.CC + (size_t)i * SG);
+#pragma unroll
+        for (int b = 0; b < LB; ++b)
+            if (b < nb) any(b, i, cbv, ccv);
+    }
+    // i > e0 + LB: P1~[i-1][e]
+    walk<U>(
+        e0 + LB + 1, n,
+        [&](int i) {
+            Row r;
+            r.c = ldl<R, VW>(t.CC + (size_t)i * SG);
+            const R *p = t.P1 + (size_t)(c2u(i - 2) + e0 - 1) * SG;
+#pragma unroll
+            for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(p + (size_t)b * SG);
+            return r;
+        },
+        [&](int, const Row &r) {
+#pragma unroll
+            for (int b = 0; b < LB; ++b)
+#pragma unroll
+                for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k], r.v[b].v[k], acc[b][k]);
+        });
+#pragma unroll
+    for (int b = 0; b < LB; ++b) {
+        if (b >= nb) break;
+        const int e = e0 + b;
+        const auto pv = ldl<R, VW>(p1_row(t, n - 1, e));
         R out[VW];
 #pragma unroll
-        for (int k = 0; k < VW; ++k) out[k] = fma(cn[k], acc[k], fma(ld.x, cn[k], ld.y) * w.v[k]);
-        stl<R, VW>(a.Pp + i_pp(n, l) * S + s, out);
+        for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[b][k], fma(ld.x, cn.v[k], ld.y) * pv.v[k]);
+        stl<R, VW>(t.P1 + i_p1(n, e) * SG, out);
     }
 }
+
+// K = 4, 5: P1~[n][e] (Eq. probelidedade). Order 3: with (a, b, c) the decreasing
+// order of (i, j, e), the terms with a = e come from the product rows (X_e(n),
+// times Pp~[n-1][e+1]); the others (a = i > e) from the per-pair sums p2_kernel
+// leaves in T: pairs (e, d), d < e, carry chi_d-weighted parts for e; pairs (j, e),
+// j > e, for e.
+template <class R, int VW, int U>
+__device__ __forceinline__ void p1_row_k45(const Args<R> &a, const Grp<R> &t, int n, int e) {
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
+    const auto ld = lead(a, n);
+    R acc[VW];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) acc[k] = R(0);
+    auto use = [&](int, const Two<R, VW> &b) {
+#pragma unroll
+        for (int k = 0; k < VW; ++k) acc[k] = fma(b.c.v[k], b.v.v[k], acc[k]);
+    };
+    if (a.op1 >= 2) {
+        walk<U>(
+            1, e,
+            [&](int i) { return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG), ldl<R, VW>(p2_row(t, n - 1, e, i))}; }, use);
+        const R *q = t.P2 + (i_p2(n - 1, 1, 0) + e) * SG;  // P2~[n-1][i][e] at C(i-1, 2)
+        walk<U>(
+            e + 1, n - 1,
+            [&](int i) {
+                return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG), ldl<R, VW>(q + (size_t)c2u(i - 1) * SG)};
+            },
+            use);
+        if (e < n - 1)
+            use(n - 1, Two<R, VW>{ldl<R, VW>(t.CB + (size_t)(n - 1) * SG), ldl<R, VW>(p1_row(t, n - 2, e))});
+    }
+    if (a.op1 >= 3) {
+        if (e >= 3) use(e, Two<R, VW>{ppl<R, VW>(t, n - 1, e + 1), ldl<R, VW>(t.X + i_z(e, n) * SG)});
+        const R *T = t.T + 2 * ((size_t)c2u(e - 1) - 1) * SG;  // pair (e, d) at 2 d
+        walk<U>(
+            1, e,
+            [&](int d) { return Two<R, VW>{ldl<R, VW>(t.chi + (size_t)d * SG), ldl<R, VW>(T + (size_t)(2 * d) * SG)}; },
+            use);
+        T = t.T + (2 * (size_t)(e - 1) + 1) * SG;  // pair (j, e) at 2 C(j-1, 2)
+        walk<U>(
+            e + 1, n,
+            [&](int j) {
+                return Two<R, VW>{ldl<R, VW>(t.chi + (size_t)j * SG), ldl<R, VW>(T + (size_t)(2 * c2u(j - 1)) * SG)};
+            },
+            use);
+    }
+    const auto pv = ldl<R, VW>(p1_row(t, n - 1, e));
+    R out[VW];
+#pragma unroll
+    for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[k], fma(ld.x, cn.v[k], ld.y) * pv.v[k]);
+    stl<R, VW>(t.P1 + i_p1(n, e) * SG, out);
+}
+
+// The p1 rows e = 1..n-1 and the p+ rows l = 1..n of one step in one launch (they
+// read rows below n only): the p1 warps first, the p+ warps by falling length.
+template <class R, int K, int VW, int U, int LB, int WPB>
+__global__ void __launch_bounds__(32 * WPB, VW * LB * sizeof(R) > 16 ? 1 : 32 / WPB) rows_kernel(Args<R> a, int n) {
+    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    constexpr int EB = K == 3 ? LB : 1;
+    const int item = (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
+    const int n1 = (n - 1 + EB - 1) / EB;
+    if (item < n1) {
+        if constexpr (K == 3) p1_rows_k3<R, VW, U, LB>(a, t, n, 1 + item * LB);
+        else p1_row_k45<R, VW, U>(a, t, n, 1 + item);
+    } else if (1 + (item - n1) * LB <= n) {
+        pp_rows<R, VW, U, LB>(a, t, n, 1 + (item - n1) * LB);
+    }
+}
+
 
 template <class R>
 __global__ void init_kernel(Args<R> a) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < a.S) {
-        a.P[s] = R(1);
-        a.chi[s] = R(1);
+        const Grp<R> t(a, s);
+        t.P[0] = R(1);
         for (int w = 0; w <= a.M / 32; ++w) a.bw[(size_t)w * a.S + s] = 0u;
     }
 }
@@ -1265,7 +1312,7 @@ __global__ void logp_kernel(Args<R> a, double *logp) {
     if (s >= a.n_valid) return;
     double h = 0.0;
     for (int v = 1; v <= a.M; ++v) h += a.H[v];
-    const double P = (double)a.P[(size_t)a.M * a.S + s];
+    const double P = (double)Grp<R>(a, s).P[(size_t)a.M * SG];
     logp[s] = P > 0.0 ? log(P) - h : __longlong_as_double(0x7ff8000000000000ULL);
 }
 
@@ -1324,27 +1371,41 @@ __global__ void kscale_kernel(const double *__restrict__ kap, int M, int d, uint
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+static Tabs sampler_tabs(int M, int K) {
+    Tabs o{};
+    size_t n = 0;
+    auto take = [&](size_t &field, size_t entries) {
+        field = n;
+        n += entries;
+    };
+    take(o.chi, (size_t)M + 1);
+    take(o.P, (size_t)M + 1);
+    take(o.G, 1);
+    take(o.CA, K >= 4 ? (size_t)M + 1 : 0);
+    take(o.CB, (size_t)M + 1);
+    take(o.CC, (size_t)M + 1);
+    take(o.Y, K >= 4 ? (size_t)M + 1 : 0);
+    take(o.Pp, cb(M, 2) + (size_t)M);
+    take(o.P1, cb(M, 2));
+    take(o.Z, cb(M, 2));
+    take(o.X, K >= 4 ? cb(M, 2) : 0);
+    take(o.T, K >= 4 ? 2 * cb(M - 1, 2) : 0);
+    take(o.P2, K >= 4 ? cb(M, 3) : 0);
+    take(o.Z5, K == 5 ? cb(M, 3) : 0);
+    o.entries = n;
+    return o;
+}
+
 SamplerLayout sampler_layout(int M, int K, int S, int precision) {
     SamplerLayout L{};
     const size_t es = precision == 0 ? sizeof(double) : sizeof(float);
     const size_t Ss = (size_t)S;
     size_t off = 256;  // status word first (read by gbs_stream_status)
-    auto take = [&](size_t &field, size_t entries) {
-        field = off;
-        off = a256(off + entries * Ss * es);
-    };
-    take(L.chi, (size_t)M + 1);
-    take(L.P, (size_t)M + 1);
-    take(L.Pp, cb(M, 2) + (size_t)M);
-    take(L.P1, cb(M, 2));
-    take(L.P2, K >= 4 ? cb(M, 3) : 0);
-    take(L.Z, cb(M, 2));
-    take(L.Z5, K == 5 ? cb(M, 3) : 0);
-    take(L.G, 1);
-    take(L.Y, K >= 4 ? (size_t)M + 1 : 0);
-    take(L.X, K >= 4 ? cb(M, 2) : 0);
+    L.tab = off;       // S is a multiple of SG: whole groups
+    off = a256(off + sampler_tabs(M, K).entries * Ss * es);
     // W: plain [r][S], or for the tensor-core product hi / lo copies of 32-padded chunks
-    take(L.W, 2 * ((K >= 4 ? cb(M - 1, 2) : (size_t)M) + 32));
+    L.W = off;
+    off = a256(off + 2 * ((K >= 4 ? cb(M - 1, 2) : (size_t)M) + 32) * Ss * es);
     // tensor-core product rows: max over the steps of (row tiles x chunks) x 8192 floats
     size_t at = 0;
     if (precision != 0)
@@ -1358,8 +1419,6 @@ SamplerLayout sampler_layout(int M, int K, int S, int precision) {
         }
     L.At = off;
     off = a256(off + at * sizeof(float));
-    take(L.CA, K >= 4 ? 3 * ((size_t)M + 1) : 0);
-    take(L.T, K >= 4 ? 2 * cb(M - 1, 2) : 0);
     L.bw = off;
     off = a256(off + (size_t)(M / 32 + 1) * Ss * sizeof(uint32_t));
     L.kap = off;  // the rescaled cumulants kappa', in the arithmetic precision
@@ -1387,10 +1446,33 @@ static dim3 egrid(int S, uint64_t entries) {
     return dim3((unsigned)bx, (unsigned)by);
 }
 
+// The kernels of step t after its products: VW samples per lane, U loads of a
+// chain ahead, LB rows per warp (rows_kernel), WPB warps per block.
+template <class R, int K, int VW, int U, int LB, int WPB>
+static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
+    const unsigned gy = (unsigned)(a.S / (32 * VW));
+    auto grid = [&](int warps) { return dim3((unsigned)((warps + WPB - 1) / WPB), gy); };
+    constexpr int NT = 32 * WPB;
+    if (K == 5 && t > 3) yv_kernel<R, VW, U, WPB><<<grid(t - 3), NT, 0, st>>>(a, t);
+    bias_kernel<R, K><<<(unsigned)(a.S / 32), 32 * BIAS_W, 0, st>>>(a, t);
+    if (K >= 4 && a.opp >= 3 && t > 1) pvv_kernel<R, VW, U, WPB><<<grid(t - 1), NT, 0, st>>>(a, t);
+    if (K >= 4 && t > 2) {  // before the p1 rows: fills T
+        constexpr int VP = sizeof(R) == 4 ? 4 : 2;
+        p2_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), (unsigned)(a.S / (32 * VP))), 32, 0, st>>>(a, t);
+    }
+    const int n1 = K == 3 ? (t - 1 + LB - 1) / LB : t - 1, np = (t + LB - 1) / LB;
+    rows_kernel<R, K, VW, U, LB, WPB><<<grid(n1 + np), NT, 0, st>>>(a, t);
+    return cudaGetLastError();
+}
+
 template <class R, int K>
 static cudaError_t run_chunk(Args<R> a, double *prob, cudaStream_t st) {
     const int S = a.S, M = a.M;
     const int TB = 256;
+    // one sample per lane until the rows of a step give every multiprocessor a
+    // full set of warps with VW of them
+    const bool wide = (uint64_t)M * S >= 1u << 19;
+    cudaError_t e = cudaSuccess;
     constexpr int TM = sizeof(R) == 4 ? 8 : 4, TN = TM;
     init_kernel<R><<<(S + TB - 1) / TB, TB, 0, st>>>(a);
     for (int t = 1; t <= M; ++t) {
@@ -1420,32 +1502,7 @@ static cudaError_t run_chunk(Args<R> a, double *prob, cudaStream_t st) {
                 zgemm_kernel<R, K, TM, TN><<<grid, 256, 0, st>>>(a, t, rows, D);
             }
         }
-        // FP32 (large batches): warp-per-entry kernels over 128-sample groups; FP64
-        // calls, a few hundred samples, keep the (samples, entries) grids
-        constexpr bool grouped = sizeof(R) == 4;
-        const unsigned gy = (unsigned)(S / 128);
-        if (K == 5 && t > 3) {
-            if constexpr (grouped) yv_kernel<R, 4><<<dim3((unsigned)(t - 3), gy), 32, 0, st>>>(a, t);
-            else y_kernel<R><<<egrid(S, (uint64_t)(t - 3)), ETB, 0, st>>>(a, t);
-        }
-        bias_kernel<R, K><<<(S + TB - 1) / TB, TB, 0, st>>>(a, t);
-        if (K >= 4 && a.opp >= 3 && t > 1) {
-            if constexpr (grouped) pvv_kernel<R, 4><<<dim3((unsigned)(t - 1), gy), 32, 0, st>>>(a, t);
-            else pv_kernel<R><<<egrid(S, (uint64_t)(t - 1)), ETB, 0, st>>>(a, t);
-        }
-        if constexpr (grouped) ppv_kernel<R, 4><<<dim3((unsigned)t, gy), 32, 0, st>>>(a, t);
-        else pp_kernel<R><<<egrid(S, (uint64_t)t), ETB, 0, st>>>(a, t);
-        if (K >= 4 && t > 1) coef_kernel<R><<<egrid(S, (uint64_t)(t - 1)), ETB, 0, st>>>(a, t);
-        if (K >= 4 && t > 2) {  // before p1: fills T
-            constexpr int VW = sizeof(R) == 4 ? 4 : 2;  // samples per lane (batch: a multiple of 128)
-            const uint64_t nr = cb(t - 1, 2);
-            p2_kernel<R, VW><<<dim3((unsigned)(nr < (1u << 30) ? nr : (1u << 30)), (unsigned)(S / (32 * VW))), 32, 0, st>>>(a, t);
-        }
-        if (t > 1) {
-            if constexpr (grouped) p1v_kernel<R, K, 4><<<dim3((unsigned)(t - 1), gy), 32, 0, st>>>(a, t);
-            else p1_kernel<R, K><<<egrid(S, (uint64_t)(t - 1)), ETB, 0, st>>>(a, t);
-        }
-        cudaError_t e = cudaGetLastError();
+        e = wide ? step_rows<R, K, sizeof(R) == 4 ? 4 : 2, 4, 1, 1>(a, t, st) : step_rows<R, K, 1, 8, sizeof(R) == 4 ? 4 : 2, 2>(a, t, st);
         if (e != cudaSuccess) return e;
     }
     if (prob) logp_kernel<R><<<(S + TB - 1) / TB, TB, 0, st>>>(a, prob);
@@ -1465,21 +1522,10 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
     a.op2 = c.orders[2];  // the caller resolves the defaults per K
     a.off[0] = 0;
     for (int d = 1; d <= 5; ++d) a.off[d] = order_offset(c.M, d);
-    a.chi = reinterpret_cast<R *>(w + L.chi);
-    a.P = reinterpret_cast<R *>(w + L.P);
-    a.Pp = reinterpret_cast<R *>(w + L.Pp);
-    a.P1 = reinterpret_cast<R *>(w + L.P1);
-    a.P2 = reinterpret_cast<R *>(w + L.P2);
-    a.Z = reinterpret_cast<R *>(w + L.Z);
-    a.Z5 = reinterpret_cast<R *>(w + L.Z5);
-    a.G = reinterpret_cast<R *>(w + L.G);
-    a.Y = reinterpret_cast<R *>(w + L.Y);
-    a.X = reinterpret_cast<R *>(w + L.X);
+    a.tab = reinterpret_cast<R *>(w + L.tab);
+    a.o = sampler_tabs(c.M, c.K);
+    a.gs = a.o.entries * SG;
     a.W = reinterpret_cast<R *>(w + L.W);
-    a.CA = reinterpret_cast<R *>(w + L.CA);
-    a.CB = a.CA + ((size_t)c.M + 1) * c.S;
-    a.CC = a.CB + ((size_t)c.M + 1) * c.S;
-    a.T = reinterpret_cast<R *>(w + L.T);
     a.At = reinterpret_cast<float *>(w + L.At);
     a.bw = reinterpret_cast<uint32_t *>(w + L.bw);
     a.status = reinterpret_cast<unsigned *>(w);

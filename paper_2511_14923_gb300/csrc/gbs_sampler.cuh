@@ -7,9 +7,10 @@
 namespace gbs {
 namespace smp {
 
-// Byte offsets of the per-sample arrays ([entries][S]) in the workspace.
+// Byte offsets of the workspace's parts: tab holds the per-sample tables, one
+// block per group of samples.
 struct SamplerLayout {
-    size_t chi, P, Pp, P1, P2, Z, Z5, G, Y, X, W, CA, T, bw, kap, hs, H, lead, At, total;
+    size_t tab, W, At, bw, kap, hs, H, lead, total;
 };
 SamplerLayout sampler_layout(int M, int K, int S, int precision);
 
