@@ -86,7 +86,7 @@ constexpr int SG = 128;
 
 // First entry of each table inside a group's block.
 struct Tabs {
-    size_t chi, P, Pp, P1, P2, Z, Z5, G, Y, X, CA, CB, CC, T, entries;
+    size_t chi, P, Pp, P1, P2, Z, Z5, G, Y, X, CA, CB, CC, T, R2, entries;
 };
 
 template <class R>
@@ -98,6 +98,7 @@ struct Args {
     size_t gs;             // elements per group block (Tabs::entries x SG)
     Tabs o;
     R *W;
+    const R *kb;           // kappa(i, n) regrouped for p2_block_kernel, or null (p2_kernel then walks every row itself)
     float *At;             // tensor-core product: the step's rows, split and tiled (atc_kernel)
     const R *hs;           // per-variable half scale s_v / 2, hs[v], v = 1..M
     const R *lead;         // per-variable pairs (kappa'({v}), hs[v]) at lead[2v], lead[2v+1]
@@ -117,7 +118,7 @@ struct Args {
 // The tables of one group, each shifted to the calling thread's (first) sample.
 template <class R>
 struct Grp {
-    R *chi, *P, *Pp, *P1, *P2, *Z, *Z5, *G, *Y, *X, *CA, *CB, *CC, *T;
+    R *chi, *P, *Pp, *P1, *P2, *Z, *Z5, *G, *Y, *X, *CA, *CB, *CC, *T, *R2;
     __device__ __forceinline__ Grp(const Args<R> &a, int s) {
         R *b = a.tab + (size_t)(s / SG) * a.gs + (s % SG);
         chi = b + a.o.chi * SG;
@@ -134,6 +135,7 @@ struct Grp {
         CB = b + a.o.CB * SG;
         CC = b + a.o.CC * SG;
         T = b + a.o.T * SG;
+        R2 = b + a.o.R2 * SG;
     }
 };
 
@@ -966,11 +968,86 @@ __global__ void __launch_bounds__(32 * WPB) pvv_kernel(Args<R> a, int n) {
     stl<R, VW>(t.Y + (size_t)j * SG, v.v);
 }
 
+// Terms i < e of P2~[n][e][d]: use(i, {coef row i, P2~[e-1][max(i,d)][min(i,d)]})
+// for i = 1 .. e-1, i != d, ascending; coef is an [i][SG] table.
+template <class R, int VW, int U, class Use>
+__device__ __forceinline__ void p2_row_terms(const Grp<R> &t, int e, int d, const R *coef, Use use) {
+    // i < d: P2~[e-1][d][i]; for d = e - 1 that row is P1~[e-2][i], ending with P~[e-3]
+    const R *q = d < e - 1 ? t.P2 + i_p2(e - 1, d, 0) * SG : t.P1 + (e >= 3 ? i_p1(e - 2, 0) : 0) * SG;
+    const R *pb = t.P + (size_t)(e - 3) * SG;
+    walk<U>(
+        1, d,
+        [&](int i) {
+            return Two<R, VW>{ldl<R, VW>(coef + (size_t)i * SG),
+                              ldl<R, VW>(d == e - 1 && i == e - 2 ? pb : q + (size_t)i * SG)};
+        },
+        use);
+    // d < i < e - 1: P2~[e-1][i][d]
+    const R *qc = t.P2 + (i_p2(e - 1, 1, 0) + d) * SG;
+    walk<U>(
+        d + 1, e - 1,
+        [&](int i) {
+            return Two<R, VW>{ldl<R, VW>(coef + (size_t)i * SG), ldl<R, VW>(qc + (size_t)c2u(i - 1) * SG)};
+        },
+        use);
+    if (d < e - 1) use(e - 1, Two<R, VW>{ldl<R, VW>(coef + (size_t)(e - 1) * SG), ldl<R, VW>(p1_row(t, e - 2, d))});
+}
+
+// The sums over i < e of the p2 update at steps n0 .. n0 + P2_NB - 1, for every
+// pair (e, d) with e < n0: sum_i kappa(i,n) chi_i P2~[e-1][max(i,d)][min(i,d)] only
+// needs bits and rows below n0, so one pass over the table serves P2_NB steps:
+// a value loaded once feeds P2_NB chains of FMAs (kappa(i,n) uniform, chi_i times
+// the value formed once; the products are the ones p2_kernel would form, in the
+// same order). Left in R2 for p2_kernel. What p2_kernel still walks each step is
+// the column i > e, whose weights Pp~[n-1][i+1] are known at step n only, and the
+// rows e >= n0.
+constexpr int P2_NB = 8;
+
+template <class R, int VW>
+__global__ void __launch_bounds__(32, 20) p2_block_kernel(Args<R> a, int n0, unsigned npairs) {
+    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW);
+    const unsigned r = blockIdx.x;
+    int hi, lo;
+    pair_of(r, hi, lo);
+    const R *kb = a.kb + (size_t)((n0 - 1) / P2_NB) * (a.M + 1) * P2_NB;
+    R x[P2_NB][VW];
+#pragma unroll
+    for (int m = 0; m < P2_NB; ++m)
+#pragma unroll
+        for (int k = 0; k < VW; ++k) x[m][k] = R(0);
+    p2_row_terms<R, VW, 4>(t, hi + 1, lo + 1, t.chi, [&](int i, const Two<R, VW> &b) {
+        R v[VW], kn[P2_NB];
+#pragma unroll
+        for (int k = 0; k < VW; ++k) v[k] = b.c.v[k] * b.v.v[k];
+        constexpr int KV = 16 / sizeof(R);
+#pragma unroll
+        for (int m = 0; m < P2_NB; m += KV) {
+            const auto q = ldl<R, KV>(kb + (size_t)i * P2_NB + m);
+#pragma unroll
+            for (int u = 0; u < KV; ++u) kn[m + u] = q.v[u];
+        }
+#pragma unroll
+        for (int m = 0; m < P2_NB; ++m)
+#pragma unroll
+            for (int k = 0; k < VW; ++k) x[m][k] = fma(kn[m], v[k], x[m][k]);
+    });
+#pragma unroll
+    for (int m = 0; m < P2_NB; ++m)
+        if (n0 + m <= a.M) stl<R, VW>(t.R2 + ((size_t)m * npairs + r) * SG, x[m]);
+}
+
+// kb[b][i][m] = kappa(i, n), n = 1 + P2_NB b + m (0 where i >= n or n > M).
+template <class R>
+__global__ void kb_kernel(const R *__restrict__ kap2, int M, int n, R *__restrict__ kb) {
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= n) return;
+    const int m = q % P2_NB, i = q / P2_NB % (M + 1), v = 1 + q / (P2_NB * (M + 1)) * P2_NB + m;
+    kb[q] = i >= 1 && i < v && v <= M ? kap2[c2u(v - 1) + (unsigned)(i - 1)] : R(0);
+}
+
 // P2~[n][e][d], n-1 >= e > d >= 1 (Eq. probdoubleelidedade).
 // Order 2: i > e reaches P2~[i-1][e][d] (factor Pp~[n-1][i+1]); i < e reaches
-// P2~[e-1][max(i,d)][min(i,d)] (common factor Pp~[n-1][e+1]). The loops walk the
-// p2 rows by running offsets; the boundary entries (P2~[i-1][i-1][.] =
-// P1~[i-2][.], P1~[i-2][i-2] = P~[i-3]) are taken apart.
+// P2~[e-1][max(i,d)][min(i,d)] (common factor Pp~[n-1][e+1]).
 // The same values P2~[i-1][e][d], i > e, are every term of the p1 order-3 sums
 // whose largest index is i (Eq. probelidedade with (a, b, c) = (i, e, d)): they
 // enter P1~[n][e] with weight CA[i] kappa(d,i,n) chi_d and P1~[n][d] with weight
@@ -980,48 +1057,31 @@ __global__ void __launch_bounds__(32 * WPB) pvv_kernel(Args<R> a, int n) {
 // The kernel is bound by load latency: the bounds cap it at 64 registers, so that
 // 32 one-warp blocks (the per-SM block limit) stay resident.
 template <class R, int VW>
-__global__ void __launch_bounds__(32, 32) p2_kernel(Args<R> a, int n) {
+__global__ void __launch_bounds__(32, 32) p2_kernel(Args<R> a, int n, unsigned npairs) {
     const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW);
     const unsigned r = blockIdx.x;
     int hi, lo;
     pair_of(r, hi, lo);
     const int e = hi + 1, d = lo + 1;
-    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
-    const auto ld = lead(a, n);
     R acc[VW], tE[VW], tD[VW];
 #pragma unroll
     for (int k = 0; k < VW; ++k) acc[k] = tE[k] = tD[k] = R(0);
     if (a.op2 >= 2) {
-        R x[VW];
+        const int m = (n - 1) % P2_NB;
+        Lanes<R, VW> x;
+        if (a.kb && e < n - m) {  // formed by p2_block_kernel at step n - m
+            x = ldl<R, VW>(t.R2 + ((size_t)m * npairs + r) * SG);
+        } else {
 #pragma unroll
-        for (int k = 0; k < VW; ++k) x[k] = R(0);
-        auto use = [&](int, const Two<R, VW> &b) {
+            for (int k = 0; k < VW; ++k) x.v[k] = R(0);
+            p2_row_terms<R, VW, 4>(t, e, d, t.CB, [&](int, const Two<R, VW> &b) {
 #pragma unroll
-            for (int k = 0; k < VW; ++k) x[k] = fma(b.c.v[k], b.v.v[k], x[k]);
-        };
-        // i < d: P2~[e-1][d][i]
-        const R *q = d < e - 1 ? t.P2 + i_p2(e - 1, d, 0) * SG : t.P1 + (e >= 3 ? i_p1(e - 2, 0) : 0) * SG;
-        const R *pb = t.P + (size_t)(e - 3) * SG;  // its boundary entry, i = d - 1 = e - 2
-        walk<4>(
-            1, d,
-            [&](int i) {
-                return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG),
-                                  ldl<R, VW>(d == e - 1 && i == e - 2 ? pb : q + (size_t)i * SG)};
-            },
-            use);
-        // d < i < e - 1: P2~[e-1][i][d]
-        const R *qc = t.P2 + (i_p2(e - 1, 1, 0) + d) * SG;
-        walk<4>(
-            d + 1, e - 1,
-            [&](int i) {
-                return Two<R, VW>{ldl<R, VW>(t.CB + (size_t)i * SG), ldl<R, VW>(qc + (size_t)c2u(i - 1) * SG)};
-            },
-            use);
-        if (d < e - 1)
-            use(e - 1, Two<R, VW>{ldl<R, VW>(t.CB + (size_t)(e - 1) * SG), ldl<R, VW>(p1_row(t, e - 2, d))});
+                for (int k = 0; k < VW; ++k) x.v[k] = fma(b.c.v[k], b.v.v[k], x.v[k]);
+            });
+        }
         const auto w = ppl<R, VW>(t, n - 1, e + 1);
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[k] = w.v[k] * x[k];
+        for (int k = 0; k < VW; ++k) acc[k] = w.v[k] * x.v[k];
     }
     if ((a.op2 >= 2 || a.op1 >= 3) && e + 1 < n) {
         const R *k3n = a.kap + a.off[3] + cb(n - 1, 3) - 1;  // k3n[C(i-1,2) + j] = kappa(j, i, n)
@@ -1069,6 +1129,8 @@ __global__ void __launch_bounds__(32, 32) p2_kernel(Args<R> a, int n) {
         stl<R, VW>(t.T + (size_t)(2 * r) * SG, tE);
         stl<R, VW>(t.T + (size_t)(2 * r + 1) * SG, tD);
     }
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
+    const auto ld = lead(a, n);
     const auto pv = ldl<R, VW>(p2_row(t, n - 1, e, d));
     R out[VW];
 #pragma unroll
@@ -1390,6 +1452,7 @@ static Tabs sampler_tabs(int M, int K) {
     take(o.Z, cb(M, 2));
     take(o.X, K >= 4 ? cb(M, 2) : 0);
     take(o.T, K >= 4 ? 2 * cb(M - 1, 2) : 0);
+    take(o.R2, K == 5 ? P2_NB * cb(M - 1, 2) : 0);  // K = 4 runs order 1 (no such sums) unless told otherwise
     take(o.P2, K >= 4 ? cb(M, 3) : 0);
     take(o.Z5, K == 5 ? cb(M, 3) : 0);
     o.entries = n;
@@ -1431,6 +1494,8 @@ SamplerLayout sampler_layout(int M, int K, int S, int precision) {
     off = a256(off + ((size_t)M + 1) * sizeof(double));
     L.lead = off;
     off = a256(off + 2 * ((size_t)M + 1) * es);
+    L.kb = off;
+    off = a256(off + (K == 5 ? (size_t)((M - 1) / P2_NB + 1) * (M + 1) * P2_NB : 0) * es);
     L.total = off;
     return L;
 }
@@ -1458,7 +1523,10 @@ static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
     if (K >= 4 && a.opp >= 3 && t > 1) pvv_kernel<R, VW, U, WPB><<<grid(t - 1), NT, 0, st>>>(a, t);
     if (K >= 4 && t > 2) {  // before the p1 rows: fills T
         constexpr int VP = sizeof(R) == 4 ? 4 : 2;
-        p2_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), (unsigned)(a.S / (32 * VP))), 32, 0, st>>>(a, t);
+        const unsigned gs = (unsigned)(a.S / (32 * VP)), npairs = (unsigned)cb(a.M - 1, 2);
+        if (a.kb && (t - 1) % P2_NB == 0 && t > 3)  // pairs e < t
+            p2_block_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
+        p2_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
     }
     const int n1 = K == 3 ? (t - 1 + LB - 1) / LB : t - 1, np = (t + LB - 1) / LB;
     rows_kernel<R, K, VW, U, LB, WPB><<<grid(n1 + np), NT, 0, st>>>(a, t);
@@ -1562,6 +1630,12 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
             const uint64_t n = cb(c.M, d), threads = (n + KS_CHUNK - 1) / KS_CHUNK;
             kscale_kernel<R><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(c.kappa, c.M, d, off, n, hs, kf);
             off += n;
+        }
+        if (c.K == 5 && a.op2 >= 2) {
+            R *kb = reinterpret_cast<R *>(w + L.kb);
+            const int n = ((c.M - 1) / P2_NB + 1) * (c.M + 1) * P2_NB;
+            kb_kernel<R><<<(n + 255) / 256, 256, 0, st>>>(kf + a.off[2], c.M, n, kb);
+            a.kb = kb;
         }
         a.kap = kf;
         a.hs = hs;

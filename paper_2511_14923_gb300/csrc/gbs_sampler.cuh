@@ -10,7 +10,7 @@ namespace smp {
 // Byte offsets of the workspace's parts: tab holds the per-sample tables, one
 // block per group of samples.
 struct SamplerLayout {
-    size_t tab, W, At, bw, kap, hs, H, lead, total;
+    size_t tab, W, At, bw, kap, hs, H, lead, kb, total;
 };
 SamplerLayout sampler_layout(int M, int K, int S, int precision);
 
