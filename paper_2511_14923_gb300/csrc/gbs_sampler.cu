@@ -281,72 +281,75 @@ __global__ void __launch_bounds__(ETB) w_kernel(Args<R> a, int t, int D) {
 }
 
 // Z[row][s] = sum_{r < D} kappa[kbase(row) + r] W_t[r][s] for rows [0, rows) and
-// all samples. 256 threads, (16 TM) x (16 TN) results per CTA, TM x TN per
-// thread (two 4-wide halves each way when 8), 8 inner entries per stage with
-// the next stage prefetched into registers.
-template <class R, int K, int TM, int TN>
+// all samples: one chain of FMAs per result, in ascending r, whatever the tile.
+// 256 threads, a tile of 16 T x 16 T results per CTA, T x T per thread (two 4-wide
+// halves each way when T = 8), BK inner entries per stage with the next stage
+// prefetched into registers. Late steps have few rows and long chains, so the
+// tile is chosen by the CTAs it leaves (launch_zgemm).
+template <class R, int K, int T>
 __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t rows, int D) {
-    constexpr int BMt = 16 * TM, BNt = 16 * TN, BKt = 8;
-    constexpr int AE = BMt * BKt / 256, BE = BNt * BKt / 256;  // elements per thread per stage
-    __shared__ __align__(16) R As[2][BKt][BMt];
-    __shared__ __align__(16) R Bs[2][BKt][BNt];
-    __shared__ uint64_t kb[BMt];
-    __shared__ uint64_t dst[BMt];
+    constexpr int BT = 16 * T, BK = T == 1 ? 16 : 8;
+    constexpr int E = BT * BK / 256;  // elements of each operand per thread per stage
+    __shared__ __align__(16) R As[2][BK][BT];
+    __shared__ __align__(16) R Bs[2][BK][BT];
+    __shared__ uint64_t kb[BT];
+    __shared__ uint64_t dst[BT];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const uint64_t m0 = (uint64_t)blockIdx.x * BMt;
-    const int s0 = blockIdx.y * BNt;
-    for (int m = tid; m < BMt; m += 256) {
+    const uint64_t m0 = (uint64_t)blockIdx.x * BT;
+    const int s0 = blockIdx.y * BT;
+    for (int m = tid; m < BT; m += 256) {
         const uint64_t q = m0 + m;
         if (q < rows) zrow(K, a.M, t, q, a.off, a.o, kb[m], dst[m]);
         else kb[m] = ~0ull;
     }
     __syncthreads();
-    // stage loaders: A element e = tid + 256 q -> (row e / 8, inner e % 8);
-    // B: BE consecutive samples of inner row tid / (BNt / BE)
-    const int bk = tid / (BNt / BE), bs = (tid % (BNt / BE)) * BE;
-    R ra[AE], rb[BE];
+    // stage loaders: A element e = tid + 256 q -> (row e / BK, inner e % BK);
+    // B: E consecutive samples of inner row tid / (BT / E)
+    const int bk = tid / (BT / E), bs = (tid % (BT / E)) * E;
+    R ra[E], rb[E];
     auto load = [&](int k0) {
 #pragma unroll
-        for (int q = 0; q < AE; ++q) {
-            const int e = tid + 256 * q, m = e / BKt, k = e % BKt;
+        for (int q = 0; q < E; ++q) {
+            const int e = tid + 256 * q, m = e / BK, k = e % BK;
             ra[q] = (kb[m] != ~0ull && k0 + k < D) ? a.kap[kb[m] + k0 + k] : R(0);
         }
         const R *w = a.W + (size_t)(k0 + bk) * a.S + s0 + bs;
 #pragma unroll
-        for (int q = 0; q < BE; ++q) rb[q] = (k0 + bk < D) ? w[q] : R(0);
+        for (int q = 0; q < E; ++q) rb[q] = (k0 + bk < D) ? w[q] : R(0);
     };
     auto store = [&](int buf) {
 #pragma unroll
-        for (int q = 0; q < AE; ++q) {
+        for (int q = 0; q < E; ++q) {
             const int e = tid + 256 * q;
-            As[buf][e % BKt][e / BKt] = ra[q];
+            As[buf][e % BK][e / BK] = ra[q];
         }
 #pragma unroll
-        for (int q = 0; q < BE; ++q) Bs[buf][bk][bs + q] = rb[q];
+        for (int q = 0; q < E; ++q) Bs[buf][bk][bs + q] = rb[q];
     };
-    R acc[TM][TN];
+    auto at = [](int th, int i) { return T == 8 ? (i < 4 ? 0 : BT / 2) + th * 4 + (i & 3) : th * T + i; };
+    R acc[T][T];
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+    for (int i = 0; i < T; ++i)
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = R(0);
+        for (int j = 0; j < T; ++j) acc[i][j] = R(0);
     load(0);
     store(0);
     __syncthreads();
     int buf = 0;
-    for (int k0 = 0; k0 < D; k0 += BKt) {
-        const bool more = k0 + BKt < D;
-        if (more) load(k0 + BKt);
+    for (int k0 = 0; k0 < D; k0 += BK) {
+        const bool more = k0 + BK < D;
+        if (more) load(k0 + BK);
 #pragma unroll
-        for (int k = 0; k < BKt; ++k) {
-            R av[TM], bv[TN];
+        for (int k = 0; k < BK; ++k) {
+            R av[T], bv[T];
 #pragma unroll
-            for (int i = 0; i < TM; ++i) av[i] = As[buf][k][(i < 4 ? 0 : BMt / 2) + ty * 4 + (i & 3)];
+            for (int i = 0; i < T; ++i) av[i] = As[buf][k][at(ty, i)];
 #pragma unroll
-            for (int j = 0; j < TN; ++j) bv[j] = Bs[buf][k][(j < 4 ? 0 : BNt / 2) + tx * 4 + (j & 3)];
+            for (int j = 0; j < T; ++j) bv[j] = Bs[buf][k][at(tx, j)];
 #pragma unroll
-            for (int i = 0; i < TM; ++i)
+            for (int i = 0; i < T; ++i)
 #pragma unroll
-                for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+                for (int j = 0; j < T; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
         }
         if (more) {
             store(buf ^ 1);
@@ -354,13 +357,33 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
             buf ^= 1;
         }
     }
+    R *const out0 = a.tab + (size_t)(s0 / SG) * a.gs + s0 % SG;  // the tile lies in one group
 #pragma unroll
-    for (int i = 0; i < TM; ++i) {
-        const int m = (i < 4 ? 0 : BMt / 2) + ty * 4 + (i & 3);
+    for (int i = 0; i < T; ++i) {
+        const int m = at(ty, i);
         if (kb[m] == ~0ull) continue;
-        R *out = a.tab + (size_t)(s0 / SG) * a.gs + dst[m] * SG + s0 % SG;  // the tile lies in one group
 #pragma unroll
-        for (int j = 0; j < TN; ++j) out[(j < 4 ? 0 : BNt / 2) + tx * 4 + (j & 3)] = acc[i][j];
+        for (int j = 0; j < T; ++j) out0[dst[m] * SG + at(tx, j)] = acc[i][j];
+    }
+}
+
+// FP32: the largest of the 128, 64 and 32-wide tiles that leaves two CTAs for
+// every multiprocessor. FP64: the FP64 pipe (2 FMAs per clock) binds with any
+// tile, so only the split counts: 32 wide from eight CTAs per multiprocessor on
+// (the last wave then costs little), else 16 wide. At M = 100, K = 5, 256 samples
+// the 64-wide FP64 tiles used before left 56-80 CTAs for 152 multiprocessors at
+// the heaviest steps: 179 ms a call, 31 ms being the pipe's.
+template <class R, int K>
+static void launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
+    auto ctas = [&](int bt) { return (rows + bt - 1) / bt * (uint64_t)(a.S / bt); };
+    auto grid = [&](int bt) { return dim3((unsigned)((rows + bt - 1) / bt), (unsigned)(a.S / bt)); };
+    if constexpr (sizeof(R) == 4) {
+        if (ctas(128) >= 2 * (uint64_t)sms) zgemm_kernel<R, K, 8><<<grid(128), 256, 0, st>>>(a, t, rows, D);
+        else if (ctas(64) >= 2 * (uint64_t)sms) zgemm_kernel<R, K, 4><<<grid(64), 256, 0, st>>>(a, t, rows, D);
+        else zgemm_kernel<R, K, 2><<<grid(32), 256, 0, st>>>(a, t, rows, D);
+    } else {
+        if (ctas(32) >= 8 * (uint64_t)sms) zgemm_kernel<R, K, 2><<<grid(32), 256, 0, st>>>(a, t, rows, D);
+        else zgemm_kernel<R, K, 1><<<grid(16), 256, 0, st>>>(a, t, rows, D);
     }
 }
 
@@ -1534,14 +1557,13 @@ static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
 }
 
 template <class R, int K>
-static cudaError_t run_chunk(Args<R> a, double *prob, cudaStream_t st) {
+static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) {
     const int S = a.S, M = a.M;
     const int TB = 256;
     // one sample per lane until the rows of a step give every multiprocessor a
     // full set of warps with VW of them
     const bool wide = (uint64_t)M * S >= 1u << 19;
     cudaError_t e = cudaSuccess;
-    constexpr int TM = sizeof(R) == 4 ? 8 : 4, TN = TM;
     init_kernel<R><<<(S + TB - 1) / TB, TB, 0, st>>>(a);
     for (int t = 1; t <= M; ++t) {
         // products for this step and later ones (inputs: rows < t of the tables)
@@ -1562,12 +1584,10 @@ static cudaError_t run_chunk(Args<R> a, double *prob, cudaStream_t st) {
                     atc_kernel<K><<<dim3(nrt, nk), 128, 0, st>>>(a, t, rows, D);
                     ztc_kernel<K><<<dim3(nrt, (unsigned)(S / TC_N)), 128, TC_SMEM, st>>>(a, t, rows, D);
                 } else {
-                    dim3 grid((unsigned)((rows + 16 * TM - 1) / (16 * TM)), (unsigned)(S / (16 * TN)));
-                    zgemm_kernel<R, K, TM, TN><<<grid, 256, 0, st>>>(a, t, rows, D);
+                    launch_zgemm<R, K>(a, t, rows, D, sms, st);
                 }
             } else {
-                dim3 grid((unsigned)((rows + 16 * TM - 1) / (16 * TM)), (unsigned)(S / (16 * TN)));
-                zgemm_kernel<R, K, TM, TN><<<grid, 256, 0, st>>>(a, t, rows, D);
+                launch_zgemm<R, K>(a, t, rows, D, sms, st);
             }
         }
         e = wide ? step_rows<R, K, sizeof(R) == 4 ? 4 : 2, 4, 1, 1>(a, t, st) : step_rows<R, K, 1, 8, sizeof(R) == 4 ? 4 : 2, 2>(a, t, st);
@@ -1581,6 +1601,12 @@ template <class R>
 static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
     const SamplerLayout L = sampler_layout(c.M, c.K, c.S, c.precision);
     char *w = static_cast<char *>(c.ws);
+    int dev = 0, sms = 0;
+    {
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+    }
     Args<R> a{};
     a.M = c.M;
     a.K = c.K;
@@ -1650,7 +1676,7 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
         a.bits = c.bits + o;
         a.q0 = c.q0 ? c.q0 + o : nullptr;
         double *pr = c.prob ? c.prob + s0 : nullptr;
-        cudaError_t e = c.K == 3 ? run_chunk<R, 3>(a, pr, st) : c.K == 4 ? run_chunk<R, 4>(a, pr, st) : run_chunk<R, 5>(a, pr, st);
+        cudaError_t e = c.K == 3 ? run_chunk<R, 3>(a, pr, sms, st) : c.K == 4 ? run_chunk<R, 4>(a, pr, sms, st) : run_chunk<R, 5>(a, pr, sms, st);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
