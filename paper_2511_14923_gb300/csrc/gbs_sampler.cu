@@ -1419,36 +1419,95 @@ __global__ void scale_kernel(const double *__restrict__ kap, int M, R *hs, R *le
     lead[2 * v + 1] = (R)half;
 }
 
-// kappa'(S) = kappa(S) prod_{v in S} s_v / 2 for every table entry, in the
-// arithmetic precision R. A thread takes KS_CHUNK consecutive entries of one
-// order: it unranks the first and steps through the rest by colex successor.
-constexpr int KS_CHUNK = 64;
+// x rounded to R; FP32 results in the normal range by integer rounding (the
+// conversion instruction runs on GB300's narrow FP64 pipe).
+template <class R>
+__device__ __forceinline__ R round_to(double x) {
+    if constexpr (sizeof(R) == 8) {
+        return x;
+    } else {
+        const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+        const int e = (int)((hi >> 20) & 0x7ffu) - 896;
+        if (e < 1 || e > 253) return (float)x;
+        unsigned r = (hi & 0x80000000u) | ((unsigned)e << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+        const unsigned rest = lo << 3;  // to nearest, ties to even; a carry moves into the exponent
+        r += rest > 0x80000000u || (rest == 0x80000000u && (r & 1u));
+        return __uint_as_float(r);
+    }
+}
+
+// kappa'(S) = kappa(S) prod_{v in S} s_v / 2 for every entry of order d, in the
+// arithmetic precision R, the product formed from the largest mode down. A warp
+// takes `run` consecutive entries, 32 at a time (coalesced); each lane keeps the
+// modes c_2 < .. < c_{d-1} of its entry, whose C(c_2, 2) pairs (c_0, c_1) are
+// consecutive ranks, and their scales' product, and moves on to the next such set
+// when its rank leaves them. Bound by the FP64 pipe (3 multiplications per entry)
+// and HBM (12 bytes per entry): M = 144, K = 5 took 9.3 ms with one thread walking
+// 64 entries, whose loads did not coalesce.
+template <class R, int D>
+__global__ void __launch_bounds__(256) kscale_kernel(const double *__restrict__ kap, int M, uint64_t off, uint64_t n,
+                                                     const R *__restrict__ hs, R *__restrict__ out, int run) {
+    extern __shared__ double hd[];  // hd[c] = scale of mode c
+    for (int c = threadIdx.x; c < M; c += blockDim.x) hd[c] = (double)hs[c + 1];
+    __syncthreads();
+    const uint64_t r0 = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * run;
+    if (r0 >= n) return;
+    const uint64_t r1 = r0 + run < n ? r0 + run : n;
+    uint64_t r = r0 + (threadIdx.x & 31);
+    if (r >= r1) return;
+    int c[D + 1];
+    colex_unrank(r, D, c);
+    c[D] = M + 1;  // beyond the last mode
+    unsigned t = 0, len = 0;  // rank within the pairs of c[2..], and their number
+    double fu = 1.0;          // product of the scales of c[2..D-1]
+    auto upper = [&]() {
+        fu = 1.0;
+#pragma unroll
+        for (int i = D - 1; i >= 2; --i) fu *= hd[c[i]];
+        len = D >= 3 ? (unsigned)binom2(c[2]) : ~0u;
+    };
+    if constexpr (D >= 2) {
+        t = (unsigned)binom2(c[1]) + (unsigned)c[0];
+        upper();
+    }
+    for (; r < r1; r += 32) {
+        const double x = kap[off + r];
+        if constexpr (D == 1) {
+            out[off + r] = round_to<R>(x * (1.0 * hd[(int)r]));
+        } else {
+            while (t >= len) {  // next set of upper modes (colex successor)
+                t -= len;
+                int i = 2;
+#pragma unroll
+                for (int k = 2; k < D - 1; ++k)
+                    if (i == k && c[k] + 1 == c[k + 1]) i = k + 1;
+#pragma unroll
+                for (int k = 2; k < D; ++k) c[k] = k < i ? k : k == i ? c[k] + 1 : c[k];
+                upper();
+            }
+            int c1, c0;
+            pair_decode(t, c1, c0);
+            out[off + r] = round_to<R>(x * ((fu * hd[c1]) * hd[c0]));
+            t += 32;
+        }
+    }
+}
 
 template <class R>
-__global__ void kscale_kernel(const double *__restrict__ kap, int M, int d, uint64_t off, uint64_t n,
-                              const R *__restrict__ hs, R *__restrict__ out) {
-    const uint64_t r0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) * KS_CHUNK;
-    if (r0 >= n) return;
-    const uint64_t r1 = r0 + KS_CHUNK < n ? r0 + KS_CHUNK : n;
-    int c[6];
-    colex_unrank(r0, d, c);
-    c[d] = M;  // sentinel
-    // product of the scales of c[1..d-1], formed again only when one of them moves
-    // (GB300's FP64 pipe is narrow: most successors move c[0] alone)
-    auto upper = [&]() {
-        double f = 1.0;
-        for (int i = d - 1; i >= 1; --i) f *= (double)hs[c[i] + 1];
-        return f;
-    };
-    double fu = upper();
-    for (uint64_t r = r0; r < r1; ++r) {
-        out[off + r] = (R)(kap[off + r] * (fu * (double)hs[c[0] + 1]));
-        // successor: the first element that can move up moves up, the ones below reset
-        int i = 0;
-        while (i < d - 1 && c[i] + 1 == c[i + 1]) ++i;
-        ++c[i];
-        for (int j = 0; j < i; ++j) c[j] = j;
-        if (i > 0 && r + 1 < r1) fu = upper();
+static void launch_kscale(const double *kap, int M, int K, const R *hs, R *out, cudaStream_t st) {
+    uint64_t off = 0;
+    for (int d = 1; d <= K; ++d) {
+        const uint64_t n = cb(M, d);
+        // 8 warps a block; short runs until they fill the GPU's warps several times
+        const int run = n >= 1u << 25 ? 4096 : 512;
+        const unsigned grid = (unsigned)((n + 8 * run - 1) / (8 * run));
+        const size_t smem = sizeof(double) * (size_t)M;  // at most 32 KB
+        if (d == 1) kscale_kernel<R, 1><<<grid, 256, smem, st>>>(kap, M, off, n, hs, out, run);
+        if (d == 2) kscale_kernel<R, 2><<<grid, 256, smem, st>>>(kap, M, off, n, hs, out, run);
+        if (d == 3) kscale_kernel<R, 3><<<grid, 256, smem, st>>>(kap, M, off, n, hs, out, run);
+        if (d == 4) kscale_kernel<R, 4><<<grid, 256, smem, st>>>(kap, M, off, n, hs, out, run);
+        if (d == 5) kscale_kernel<R, 5><<<grid, 256, smem, st>>>(kap, M, off, n, hs, out, run);
+        off += n;
     }
 }
 
@@ -1651,12 +1710,7 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
         R *ldp = reinterpret_cast<R *>(w + L.lead);
         R *kf = reinterpret_cast<R *>(w + L.kap);
         scale_kernel<R><<<(c.M + 255) / 256, 256, 0, st>>>(c.kappa, c.M, hs, ldp, H);
-        uint64_t off = 0;
-        for (int d = 1; d <= c.K; ++d) {
-            const uint64_t n = cb(c.M, d), threads = (n + KS_CHUNK - 1) / KS_CHUNK;
-            kscale_kernel<R><<<(unsigned)((threads + 255) / 256), 256, 0, st>>>(c.kappa, c.M, d, off, n, hs, kf);
-            off += n;
-        }
+        launch_kscale<R>(c.kappa, c.M, c.K, hs, kf, st);
         if (c.K == 5 && a.op2 >= 2) {
             R *kb = reinterpret_cast<R *>(w + L.kb);
             const int n = ((c.M - 1) / P2_NB + 1) * (c.M + 1) * P2_NB;
