@@ -277,20 +277,20 @@ struct TreeShared {
     uint64_t baseT[CC][NQ];
     double p0R[CC][NQ];
     double m3[CC][3];
-    float m3f[CC][6];  // refined path: m3 as float pairs (h, l) x 3
+    float p3f[CC][6];  // refined path: the c3 pivot's factors i0, l, i1 as pairs (Piv)
     double g3[DISP ? CC : 1][2];  // displaced: whitened half-mean of each child's c3 pivot
     // Per x-entry data, structure of arrays. FP64 path (10 double rows):
     // z(x) = m3 * S_U[c3, x] (rows 0-3), d(x) = S_U[x,x] - z^T z (rows 4-6),
     // inverse c2-pivot factor m2(x) (rows 7-9). Refined-FP32 path (6 float4
-    // rows, so that a leaf loads its x-entries with 9 vector loads, consecutive
-    // entries in consecutive 16-byte words): z hi (0), z lo (1), (d hi 00 01 11,
-    // d lo 00) (2), (d lo 01 11, c2 pivot FP32 factor l00 l10) (3), (l11, its
-    // inverse m00 m10 m11) (4), residual d - l l^T (e00 e01 e11, 0) (5).
+    // rows, consecutive entries in consecutive 16-byte words): z hi (0), z lo (1),
+    // (d hi 00 01 11, d lo 00) (2), (d lo 01 11, 0, 0) (3), the c2 pivot's factors
+    // (i0 h l, l h l) (4), (i1 h l, 0, 0) (5). A leaf loads rows 0-3 of j and
+    // 0, 1, 4, 5 of c2.
     // Displaced states add 4 double rows: the reduced half-mean r(x) after
     // eliminating U and c3 (rows 10-11) and its whitened form g2(x) = m2(x) r(x)
     // as a c2 pivot (rows 12-13).
     // Before the batches of an item start, the same storage holds Y(x) of the
-    // elimination of U (8 doubles per mode x < c4).
+    // elimination of U (8 doubles per mode x < c4, or 4 float4 rows of pairs).
     static constexpr int XROWS = DISP ? 14 : 10;
     static constexpr int XBYTES = (6 * 16 > XROWS * 8 ? 6 * 16 : XROWS * 8) * XC;
     alignas(16) unsigned char xraw[XBYTES];
@@ -298,85 +298,49 @@ struct TreeShared {
     // four float4 rows, row r holding floats 4r..4r+3 of every x
     alignas(16) float4 yq[YC > 0 ? 4 : 1][YC > 0 ? YC : 1];
     __device__ double (*xe())[XC] { return reinterpret_cast<double(*)[XC]>(xraw); }
-    __device__ float (*xf())[XC] { return reinterpret_cast<float(*)[XC]>(xraw); }
     __device__ float4 (*xq())[XC] { return reinterpret_cast<float4(*)[XC]>(xraw); }
 };
 
-// Schur-complement slot access. FP64 path: 2x2 blocks as 4 doubles. Refined
-// path: the same 32 bytes hold 4 hi floats then 4 lo floats (value = hi + lo).
-template <int PREC>
-__device__ __forceinline__ Blk slot_pair_f64(const double *slot, size_t q) {
-    if (PREC == 0) return load_blk(slot + 4 * q);
+// Schur-complement slots: 2x2 blocks at pair index, then the diagonal blocks, 32
+// bytes each. FP64 path: 4 doubles (diagonal: 00 01 11). Refined path: 4 hi floats
+// then 4 lo floats (diagonal: h00 h01 h11 l00 | l01 l11).
+__device__ __forceinline__ Sym slot_diag(const double *sdiag, int x) {
+    return Sym{sdiag[4 * x], sdiag[4 * x + 1], sdiag[4 * x + 2]};
+}
+__device__ __forceinline__ ABlk slot_pair_df(const double *slot, size_t q) {
     const float4 *f = reinterpret_cast<const float4 *>(slot) + 2 * q;
     const float4 h = f[0], l = f[1];
-    return Blk{join_df(h.x, l.x), join_df(h.y, l.y), join_df(h.z, l.z), join_df(h.w, l.w)};
+    return ABlk{Acc{h.x, l.x}, Acc{h.y, l.y}, Acc{h.z, l.z}, Acc{h.w, l.w}};
 }
-template <int PREC>
-__device__ __forceinline__ Sym slot_diag_f64(const double *sdiag, int x) {
-    if (PREC == 0) return Sym{sdiag[4 * x], sdiag[4 * x + 1], sdiag[4 * x + 2]};
-    const float *f = reinterpret_cast<const float *>(sdiag) + 8 * x;
-    return Sym{join_df(f[0], f[3]), join_df(f[1], f[4]), join_df(f[2], f[5])};
-}
-template <int PREC>
-__device__ __forceinline__ void slot_store_pair(double *slot, size_t q, const Blk &b) {
-    if (PREC == 0) {
-        store_blk(slot + 4 * q, b);
-        return;
-    }
-    float4 h, l;
-    split_df(b.a00, h.x, l.x);
-    split_df(b.a01, h.y, l.y);
-    split_df(b.a10, h.z, l.z);
-    split_df(b.a11, h.w, l.w);
-    float4 *f = reinterpret_cast<float4 *>(slot) + 2 * q;
-    f[0] = h;
-    f[1] = l;
-}
-template <int PREC>
-__device__ __forceinline__ void slot_store_diag(double *sdiag, int x, const Sym &d) {
-    if (PREC == 0) {
-        store_blk(sdiag + 4 * (size_t)x, Blk{d.s00, d.s01, d.s11, 0.0});
-        return;
-    }
-    float4 h, l;
-    split_df(d.s00, h.x, h.w);
-    split_df(d.s01, h.y, l.x);
-    split_df(d.s11, h.z, l.y);
-    l.z = l.w = 0.f;
-    // layout: h00 h01 h11 l00 | l01 l11 _ _
-    float4 *f = reinterpret_cast<float4 *>(sdiag) + 2 * (size_t)x;
-    f[0] = h;
-    f[1] = l;
+__device__ __forceinline__ ASym slot_diag_df(const double *sdiag, int x) {
+    const float4 *f = reinterpret_cast<const float4 *>(sdiag) + 2 * (size_t)x;
+    const float4 a = f[0];
+    const float2 b = *reinterpret_cast<const float2 *>(f + 1);
+    return ASym{Acc{a.x, a.w}, Acc{a.y, b.x}, Acc{a.z, b.y}};
 }
 
 // Schur-complement block S_U[x][y] (x >= y) of the refined path formed from A's
-// float-pair block and the rows Y(x), Y(y) of the eliminated modes U:
-// b_uv -= sum_k y(x)_ku y(y)_kv over the pivot rows k of c5 (D = 5) and c4, in
-// float pairs on the FP32 pipe. The same operations in the same order as the
-// slot build, so both forms give the same bits.
-template <int D, int YC>
-__device__ __forceinline__ void su_block(const float *__restrict__ Af, int M, const float4 (*yq)[YC], int x, int y,
-                                         DF (&b)[4]) {
-    const float4 a0 = reinterpret_cast<const float4 *>(Af)[2 * ((size_t)x * M + y)];
-    const float4 a1 = reinterpret_cast<const float4 *>(Af)[2 * ((size_t)x * M + y) + 1];
-    b[0] = DF{a0.x, a1.x};
-    b[1] = DF{a0.y, a1.y};
-    b[2] = DF{a0.z, a1.z};
-    b[3] = DF{a0.w, a1.w};
-    // one pivot row k of one eliminated mode at a time: x's elements (k, 0), (k, 1)
-    // and y's in one float4 each; every element still takes its four updates in
-    // the build's order (c5 row 0, c5 row 1, c4 row 0, c4 row 1)
+// blocks and the rows Y(x), Y(y) of the eliminated modes U (rows 0, 1 of c5 for
+// D = 5, then 2, 3 of c4), normalised:
+// b_uv -= sum_k y(x)_ku y(y)_kv. Shared by the slot build and the slot-free form,
+// so both give the same bits.
+template <int D, class Rows>
+__device__ __forceinline__ DFBlk su_block(const float *__restrict__ Af, int M, const Rows yq, int x, int y) {
+    const float4 *f = reinterpret_cast<const float4 *>(Af) + 2 * ((size_t)x * M + y);
+    const float4 h = f[0], l = f[1];
+    ABlk b{Acc{h.x, l.x}, Acc{h.y, l.y}, Acc{h.z, l.z}, Acc{h.w, l.w}};
 #pragma unroll
-    for (int blk = (D == 5 ? 0 : 1); blk < 2; ++blk)
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            const float4 xr = yq[2 * blk + k][x], yr = yq[2 * blk + k][y];
-            const DF x0{xr.x, xr.y}, x1{xr.z, xr.w}, y0{yr.x, yr.y}, y1{yr.z, yr.w};
-            b[0] = df_sub_mul(b[0], x0, y0);
-            b[1] = df_sub_mul(b[1], x0, y1);
-            b[2] = df_sub_mul(b[2], x1, y0);
-            b[3] = df_sub_mul(b[3], x1, y1);
-        }
+    for (int k = (D == 5 ? 0 : 2); k < 4; ++k) {
+        const float4 u = yq[k][x], v = yq[k][y];
+        acc_sub_row(b, DF{u.x, u.y}, DF{u.z, u.w}, DF{v.x, v.y}, DF{v.z, v.w});
+    }
+    return DFBlk{acc_norm(b.a00), acc_norm(b.a01), acc_norm(b.a10), acc_norm(b.a11)};
+}
+__device__ __forceinline__ ABlk acc_of(const DFBlk &b) {
+    return ABlk{Acc{b.a00.h, b.a00.l}, Acc{b.a01.h, b.a01.l}, Acc{b.a10.h, b.a10.l}, Acc{b.a11.h, b.a11.l}};
+}
+__device__ __forceinline__ ASym acc_sym(const DFBlk &b) {
+    return ASym{Acc{b.a00.h, b.a00.l}, Acc{b.a01.h, b.a01.l}, Acc{b.a11.h, b.a11.l}};
 }
 
 // Number of stride classes the children c3 in [2, c4) of one U are split into.
@@ -466,7 +430,6 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
     constexpr int NQ = SH::NQ;
     constexpr int PALL = NQ - 1;
     double(*const xe)[XC] = sh.xe();
-    float(*const xf)[XC] = sh.xf();
     float4(*const xq)[XC] = sh.xq();
     const int tid = threadIdx.x;
     const int M = a.M;
@@ -510,9 +473,8 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
     __syncthreads();
     {
         // Y(x) = [y5(x); y4(x)] into the x-entry area (it is free until the batches start):
-        // 8 doubles per x (FP64 path) or 8 float pairs per x (refined path); x < c4 <= 1023
+        // 8 doubles per x (FP64 path) or 4 float4 rows of pairs (refined path); x < c4 <= 1023
         double *Y = &xe[0][0];
-        float *Yf = &xf[0][0];
         const LInv m5{sh.upiv[0], sh.upiv[1], sh.upiv[2]};
         const LInv m4{sh.upiv[3], sh.upiv[4], sh.upiv[5]};
         Blk y5c4{0, 0, 0, 0};
@@ -533,18 +495,18 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                 rU[2 * x + 1] = r.v1;
             }
             const double v[8] = {y5.a00, y5.a01, y5.a10, y5.a11, y4.a00, y4.a01, y4.a10, y4.a11};
-            if constexpr (NOSLOT) {
-                float f[16];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) split_df(v[k], f[2 * k], f[2 * k + 1]);
-#pragma unroll
-                for (int r = 0; r < 4; ++r) sh.yq[r][x] = make_float4(f[4 * r], f[4 * r + 1], f[4 * r + 2], f[4 * r + 3]);
-            } else if (PREC == 0) {
+            if constexpr (PREC == 0) {
 #pragma unroll
                 for (int k = 0; k < 8; ++k) Y[8 * x + k] = v[k];
             } else {
 #pragma unroll
-                for (int k = 0; k < 8; ++k) split_df(v[k], Yf[16 * x + 2 * k], Yf[16 * x + 2 * k + 1]);
+                for (int k = 0; k < 4; ++k) {
+                    float4 r;
+                    split_df(v[2 * k], r.x, r.y);
+                    split_df(v[2 * k + 1], r.z, r.w);
+                    if constexpr (NOSLOT) sh.yq[k][x] = r;
+                    else xq[k][x] = r;
+                }
             }
         }
         __syncthreads();
@@ -562,32 +524,16 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                 const Blk y4x{px[4], px[5], px[6], px[7]}, y4y{py[4], py[5], py[6], py[7]};
                 if (D == 5) b = blk_sub_cross(b, y5x, y5y);
                 b = blk_sub_cross(b, y4x, y4y);
-                if (qi < npairs) slot_store_pair<PREC>(slot, qi, b);
-                else slot_store_diag<PREC>(sdiag, x, Sym{b.a00, 0.5 * (b.a01 + b.a10), b.a11});
+                if (qi < npairs) store_blk(slot + 4 * (size_t)qi, b);
+                else store_blk(sdiag + 4 * (size_t)x, Blk{b.a00, 0.5 * (b.a01 + b.a10), b.a11, 0.0});
             } else {
-                // the same elimination in float pairs: b_uv -= sum_k y(x)_ku y(y)_kv over the
-                // pivot rows k of each eliminated mode (y as a 2x2 block {00, 01, 10, 11})
-                const float *af = a.Af + 8 * ((size_t)x * M + y);
-                DF b[4] = {{af[0], af[4]}, {af[1], af[5]}, {af[2], af[6]}, {af[3], af[7]}};
-                const float *px = Yf + 16 * x, *py = Yf + 16 * y;
-#pragma unroll
-                for (int blk = (D == 5 ? 0 : 1); blk < 2; ++blk) {
-                    const float *qx = px + 8 * blk, *qy = py + 8 * blk;
-#pragma unroll
-                    for (int u = 0; u < 2; ++u)
-#pragma unroll
-                        for (int v = 0; v < 2; ++v)
-#pragma unroll
-                            for (int k = 0; k < 2; ++k)
-                                b[2 * u + v] = df_sub_mul(b[2 * u + v], DF{qx[2 * (2 * k + u)], qx[2 * (2 * k + u) + 1]},
-                                                          DF{qy[2 * (2 * k + v)], qy[2 * (2 * k + v) + 1]});
-                }
+                const DFBlk g = su_block<D>(a.Af, M, xq, x, y);
+                const DF b[4] = {g.a00, g.a01, g.a10, g.a11};
                 if (qi < npairs) {
                     float4 *f = reinterpret_cast<float4 *>(slot) + 2 * (size_t)qi;
                     f[0] = make_float4(b[0].h, b[1].h, b[2].h, b[3].h);
                     f[1] = make_float4(b[0].l, b[1].l, b[2].l, b[3].l);
                 } else {
-                    // layout: h00 h01 h11 l00 | l01 l11 _ _
                     float4 *f = reinterpret_cast<float4 *>(sdiag) + 2 * (size_t)x;
                     f[0] = make_float4(b[0].h, b[1].h, b[3].h, b[0].l);
                     f[1] = make_float4(b[1].l, b[3].l, 0.f, 0.f);
@@ -641,28 +587,24 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
 #pragma unroll
             for (int q = 1; q < NQ; ++q) sh.p0R[b][q] = a.p0[idxQ[q]];
             bool ok;
-            double dd;
-            Sym p3;
-            if constexpr (NOSLOT) {
-                DF b[4];
-                su_block<D, YC>(a.Af, M, sh.yq, c3, c3, b);
-                p3 = Sym{join_df(b[0].h, b[0].l), join_df(b[1].h, b[1].l), join_df(b[3].h, b[3].l)};
+            if constexpr (PREC == 0) {
+                double dd;
+                const LInv m3 = chol2_inv(slot_diag(sdiag, c3), ok, dd);
+                sh.m3[b][0] = m3.m00; sh.m3[b][1] = m3.m10; sh.m3[b][2] = m3.m11;
+                if constexpr (DISP) {
+                    const Vec2 g3 = lvec(m3, Vec2{rU[2 * c3], rU[2 * c3 + 1]});
+                    sh.g3[b][0] = g3.v0;
+                    sh.g3[b][1] = g3.v1;
+                }
             } else {
-                p3 = slot_diag_f64<PREC>(sdiag, c3);
+                ASym p;
+                if constexpr (NOSLOT) p = acc_sym(su_block<D>(a.Af, M, sh.yq, c3, c3));
+                else p = slot_diag_df(sdiag, c3);
+                const Piv p3 = pivot_of(p, ok);
+                sh.p3f[b][0] = p3.i0.h; sh.p3f[b][1] = p3.i0.l; sh.p3f[b][2] = p3.l.h;
+                sh.p3f[b][3] = p3.l.l; sh.p3f[b][4] = p3.i1.h; sh.p3f[b][5] = p3.i1.l;
             }
-            const LInv m3 = chol2_inv(p3, ok, dd);
             if (!ok) flag_status(a.status, ST_NOT_POSDEF);
-            sh.m3[b][0] = m3.m00; sh.m3[b][1] = m3.m10; sh.m3[b][2] = m3.m11;
-            if constexpr (DISP) {
-                const Vec2 g3 = lvec(m3, Vec2{rU[2 * c3], rU[2 * c3 + 1]});
-                sh.g3[b][0] = g3.v0;
-                sh.g3[b][1] = g3.v1;
-            }
-            if (PREC == 1) {
-                split_df(m3.m00, sh.m3f[b][0], sh.m3f[b][1]);
-                split_df(m3.m10, sh.m3f[b][2], sh.m3f[b][3]);
-                split_df(m3.m11, sh.m3f[b][4], sh.m3f[b][5]);
-            }
         }
         __syncthreads();
         // setup: eliminate c3 for every x < c3 of every child in the batch
@@ -678,8 +620,8 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
             const int x = e - sh.xoff[b];
             if (PREC == 0) {
                 const LInv m3{sh.m3[b][0], sh.m3[b][1], sh.m3[b][2]};
-                const Blk z = lmul(m3, slot_pair_f64<PREC>(slot, binom2(c3) + x));
-                const Sym dx = sym_sub_gram(slot_diag_f64<PREC>(sdiag, x), z);
+                const Blk z = lmul(m3, load_blk(slot + 4 * (binom2(c3) + x)));
+                const Sym dx = sym_sub_gram(slot_diag(sdiag, x), z);
                 xe[0][e] = z.a00; xe[1][e] = z.a01; xe[2][e] = z.a10; xe[3][e] = z.a11;
                 xe[4][e] = dx.s00; xe[5][e] = dx.s01; xe[6][e] = dx.s11;
                 Vec2 r3{0, 0};
@@ -699,55 +641,32 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                     }
                 }
             } else {
-                // z(x) = m3 S_U[c3, x] and d(x) = S_U[x, x] - z^T z in float pairs (FP32 pipe)
-                DF S00, S01, S10, S11, D00, D01, D11;
+                // the pivot rows z(x) of c3, d(x) = S_U[x, x] - z^T z, and x as a c2 pivot
+                ABlk S;
+                ASym dx;
                 if constexpr (NOSLOT) {
-                    DF b[4];
-                    su_block<D, YC>(a.Af, M, sh.yq, c3, x, b);
-                    S00 = b[0]; S01 = b[1]; S10 = b[2]; S11 = b[3];
-                    su_block<D, YC>(a.Af, M, sh.yq, x, x, b);
-                    D00 = b[0]; D01 = b[1]; D11 = b[3];
+                    S = acc_of(su_block<D>(a.Af, M, sh.yq, c3, x));
+                    dx = acc_sym(su_block<D>(a.Af, M, sh.yq, x, x));
                 } else {
-                    const float *fs = reinterpret_cast<const float *>(slot) + 8 * (binom2(c3) + x);
-                    const float *fd = reinterpret_cast<const float *>(sdiag) + 8 * x;
-                    S00 = DF{fs[0], fs[4]}; S01 = DF{fs[1], fs[5]}; S10 = DF{fs[2], fs[6]}; S11 = DF{fs[3], fs[7]};
-                    D00 = DF{fd[0], fd[3]}; D01 = DF{fd[1], fd[4]}; D11 = DF{fd[2], fd[5]};
+                    S = slot_pair_df(slot, binom2(c3) + x);
+                    dx = slot_diag_df(sdiag, x);
                 }
-                const DF m00{sh.m3f[b][0], sh.m3f[b][1]}, m10{sh.m3f[b][2], sh.m3f[b][3]}, m11{sh.m3f[b][4], sh.m3f[b][5]};
-                const DF z00 = df_mul(m00, S00), z01 = df_mul(m00, S01);
-                const DF z10 = df_add_mul(df_mul(m10, S00), m11, S10);
-                const DF z11 = df_add_mul(df_mul(m10, S01), m11, S11);
-                const DF d00 = df_sub_mul(df_sub_mul(D00, z00, z00), z10, z10);
-                const DF d01 = df_sub_mul(df_sub_mul(D01, z00, z01), z10, z11);
-                const DF d11 = df_sub_mul(df_sub_mul(D11, z01, z01), z11, z11);
-                xq[0][e] = make_float4(z00.h, z01.h, z10.h, z11.h);
-                xq[1][e] = make_float4(z00.l, z01.l, z10.l, z11.l);
-                xq[2][e] = make_float4(d00.h, d01.h, d11.h, d00.l);
-                float4 q3 = make_float4(d01.l, d11.l, 0.f, 0.f), q4 = make_float4(0.f, 0.f, 0.f, 0.f),
-                       q5 = make_float4(0.f, 0.f, 0.f, 0.f);
+                const float *pf = sh.p3f[b];
+                DFBlk z = pivot_rows(S, Piv{DF{pf[0], pf[1]}, DF{pf[2], pf[3]}, DF{pf[4], pf[5]}});
+                z = DFBlk{df_norm(z.a00.h, z.a00.l), df_norm(z.a01.h, z.a01.l), df_norm(z.a10.h, z.a10.l),
+                          df_norm(z.a11.h, z.a11.l)};
+                dx = acc_sub_gram(dx, z);
+                xq[0][e] = make_float4(z.a00.h, z.a01.h, z.a10.h, z.a11.h);
+                xq[1][e] = make_float4(z.a00.l, z.a01.l, z.a10.l, z.a11.l);
+                xq[2][e] = make_float4(dx.s00.s, dx.s01.s, dx.s11.s, dx.s00.t);
+                xq[3][e] = make_float4(dx.s01.t, dx.s11.t, 0.f, 0.f);
                 if (x >= 1) {
-                    // FP32 Cholesky factor of the c2 pivot d(x), its inverse, and the residual
-                    // d - l l^T formed exactly (two-product, two-sum)
-                    const float pa = d00.h, pb = d01.h, pc = d11.h;
-                    const float i0 = rsqrtf(pa);
-                    const float l00 = pa * i0, l10 = pb * i0;
-                    const float pq = __fmaf_rn(-l10, l10, pc);
-                    const float i1 = rsqrtf(pq);
-                    const float l11 = pq * i1;
-                    if (!(pa > 0.f) || !(pq > 0.f)) flag_status(a.status, ST_NOT_POSDEF);
-                    q3.z = l00;
-                    q3.w = l10;
-                    q4 = make_float4(l11, i0, -l10 * i0 * i1, i1);
-                    EftAcc r00{d00.h, d00.l}, r01{d01.h, d01.l}, r11{d11.h, d11.l};
-                    eft_sub_prod(r00, l00, l00);
-                    eft_sub_prod(r01, l00, l10);
-                    eft_sub_prod(r11, l10, l10);
-                    eft_sub_prod(r11, l11, l11);
-                    q5 = make_float4(eft_val(r00), eft_val(r01), eft_val(r11), 0.f);
+                    bool ok;
+                    const Piv p = pivot_of(dx, ok);
+                    if (!ok) flag_status(a.status, ST_NOT_POSDEF);
+                    xq[4][e] = make_float4(p.i0.h, p.i0.l, p.l.h, p.l.l);
+                    xq[5][e] = make_float4(p.i1.h, p.i1.l, 0.f, 0.f);
                 }
-                xq[3][e] = q3;
-                xq[4][e] = q4;
-                xq[5][e] = q5;
             }
         }
         __syncthreads();
@@ -759,18 +678,10 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
             int c2, j;
             pair_decode(t, c2, j);
             Blk S64{0, 0, 0, 0};
-            DFBlk Sdf{};
-            if constexpr (PREC == 0) {
-                S64 = load_blk(slot + 4 * (size_t)t);
-            } else if constexpr (NOSLOT) {
-                DF b[4];
-                su_block<D, YC>(a.Af, M, sh.yq, c2, j, b);
-                Sdf = DFBlk{b[0].h, b[1].h, b[2].h, b[3].h, b[0].l, b[1].l, b[2].l, b[3].l};
-            } else {
-                const float4 *fs = reinterpret_cast<const float4 *>(slot) + 2 * (size_t)t;
-                const float4 sh4 = fs[0], sl4 = fs[1];
-                Sdf = DFBlk{sh4.x, sh4.y, sh4.z, sh4.w, sl4.x, sl4.y, sl4.z, sl4.w};
-            }
+            ABlk Sg{};
+            if constexpr (PREC == 0) S64 = load_blk(slot + 4 * (size_t)t);
+            else if constexpr (NOSLOT) Sg = acc_of(su_block<D>(a.Af, M, sh.yq, c2, j));
+            else Sg = slot_pair_df(slot, t);
             for (int b = 0; b < nb && c2 < sh.c3[b]; ++b) {
                 const int xo = sh.xoff[b];
                 const int e2 = xo + c2, ej = xo + j;
@@ -797,18 +708,19 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                     ok = det2 > 0.0;
                 } else {
                     const float4 zh2 = xq[0][e2], zl2 = xq[1][e2], zhj = xq[0][ej], zlj = xq[1][ej];
-                    const float4 dj0 = xq[2][ej], dj1 = xq[3][ej];
-                    const float4 p3 = xq[3][e2], p4 = xq[4][e2], p5 = xq[5][e2];
-                    const DFBlk z2{zh2.x, zh2.y, zh2.z, zh2.w, zl2.x, zl2.y, zl2.z, zl2.w};
-                    const DFBlk zj{zhj.x, zhj.y, zhj.z, zhj.w, zlj.x, zlj.y, zlj.z, zlj.w};
-                    const DFSym dj{dj0.x, dj0.y, dj0.z, dj0.w, dj1.x, dj1.y};
-                    const F32Piv pv{p3.z, p3.w, p4.x, p4.y, p4.z, p4.w, p5.x, p5.y, p5.z};
+                    const float4 d0 = xq[2][ej], p4 = xq[4][e2];
+                    const float2 d1 = *reinterpret_cast<const float2 *>(&xq[3][ej]);
+                    const float2 p5 = *reinterpret_cast<const float2 *>(&xq[5][e2]);
+                    const DFBlk z2{DF{zh2.x, zl2.x}, DF{zh2.y, zl2.y}, DF{zh2.z, zl2.z}, DF{zh2.w, zl2.w}};
+                    const DFBlk zj{DF{zhj.x, zlj.x}, DF{zhj.y, zlj.y}, DF{zhj.z, zlj.z}, DF{zhj.w, zlj.w}};
+                    const ASym dj{Acc{d0.x, d0.w}, Acc{d0.y, d1.x}, Acc{d0.z, d1.y}};
+                    const Piv pv{DF{p4.x, p4.y}, DF{p4.z, p4.w}, DF{p5.x, p5.y}};
+                    float r0, eta;
+                    refined_leaf_factor(Sg, z2, zj, dj, pv, r0, eta, ok);
                     if constexpr (MODE == MODE_KAPPA || MODE == MODE_SPINK) {
                         if (!write_p0 && a.p0f) {
                             // P0(S) is not stored: its product with P0(S') folds into the
                             // recursion's leading term (15 FP64 instructions per entry)
-                            float r0, eta;
-                            refined_leaf_factor(Sdf, z2, zj, dj, pv, r0, eta, ok);
                             const float2 pj = reinterpret_cast<const float2 *>(a.p0f)[j];
                             double v = combine_tail<NP, MODE>(
                                 refined_lead_term<(lead_sign<NP, MODE>() < 0)>(P0Sp, r0, eta, pj.x, pj.y), j, c2, t,
@@ -821,7 +733,7 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                             continue;
                         }
                     }
-                    P0 = refined_leaf_p0(P0Sp, Sdf, z2, zj, dj, pv, ok);
+                    P0 = refined_leaf_p0(P0Sp, r0, eta);
                 }
                 if (!ok) {
                     flag_status(a.status, ST_NOT_POSDEF);
