@@ -403,13 +403,14 @@ static void launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms,
 // multiprocessor (and its 512 tensor-memory columns) and one's epilogue
 // overlaps the other's MMAs. Every wait is bounded; one that runs out sets ST_TIMEOUT in the status
 // word.
-constexpr int TC_M = 128, TC_N = 256, TC_KC = 8, TC_NS = 4;  // TC_NS stages of TC_KC-wide chunks
+constexpr int TC_M = 128, TC_N = 256, TC_KC = 8;
 constexpr int TC_ACH = TC_M * TC_KC;            // floats of one A copy (hi or lo) of one chunk
 constexpr int TC_BCH = TC_N * TC_KC;            // floats of one B copy of one chunk
 constexpr int TC_AB = TC_M * TC_KC * 4;         // bytes of one A copy per stage (4 KB)
 constexpr int TC_BB = TC_N * TC_KC * 4;         // bytes of one B copy per stage (8 KB)
 constexpr int TC_STAGE = 2 * TC_AB + 2 * TC_BB;  // A hi, A lo, B hi, B lo
-constexpr int TC_SMEM = TC_NS * TC_STAGE + 256;  // stages, then 2 x TC_NS mbarriers, TMEM slot, flag
+constexpr int TC_NS = 4, TC_NS_DEEP = 8;         // stages of the ring (see launch_ztc)
+constexpr int tc_smem(int ns) { return ns * TC_STAGE + 256; }  // stages, then 2 x ns mbarriers, TMEM slot, flag
 // instruction descriptor: D f32, A and B tf32, both K-major, N = 256, M = 128
 constexpr uint32_t TC_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_N >> 3) << 17) |
                               ((uint32_t)(TC_M >> 4) << 24);
@@ -588,20 +589,20 @@ __global__ void __launch_bounds__(128) atc_kernel(Args<float> a, int t, uint64_t
 // loaded into the stage of chunk c-1 once the MMAs of chunk c-1 have completed,
 // while those of chunk c run. All threads then read
 // the accumulator (thread i = row i) and write the rows out.
-template <int K>
-__global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint64_t rows, int D) {
+template <int K, int NS>
+__global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<float> a, int t, uint64_t rows, int D) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    static_assert(TC_NS <= 8, "barrier area");
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + TC_NS * TC_STAGE);
+    static_assert(NS <= 8, "barrier area");
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + NS * TC_STAGE);
     uint64_t *empty = full + 8;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + TC_NS * TC_STAGE + 128);
-    int *flag = reinterpret_cast<int *>(smem + TC_NS * TC_STAGE + 192);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + NS * TC_STAGE + 128);
+    int *flag = reinterpret_cast<int *>(smem + NS * TC_STAGE + 192);
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint64_t m0 = (uint64_t)blockIdx.x * TC_M;
     const int rt = blockIdx.x, sb = blockIdx.y, s0 = sb * TC_N, nsb = a.S / TC_N;
     const int nk = (D + TC_KC - 1) / TC_KC;
     if (tid == 0) {
-        for (int i = 0; i < TC_NS; ++i) {
+        for (int i = 0; i < NS; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&empty[i], 1);
         }
@@ -623,27 +624,27 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
         const float *Ab = a.At + (size_t)rt * nk * 2 * TC_ACH;
         const float *Wb = a.W + (size_t)sb * 2 * TC_BCH;
         auto load = [&](int c) {
-            const int st = c % TC_NS;
+            const int st = c % NS;
             unsigned char *sp = smem + st * TC_STAGE;
             mbar_expect(&full[st], 2 * TC_AB + 2 * TC_BB);
             tma_bulk(sp, Ab + (size_t)c * 2 * TC_ACH, 2 * TC_AB, &full[st]);
             tma_bulk(sp + 2 * TC_AB, Wb + (size_t)c * nsb * 2 * TC_BCH, 2 * TC_BB, &full[st]);
         };
-        // chunk c uses stage c % TC_NS and completes phase (c / TC_NS) & 1 of its
+        // chunk c uses stage c % NS and completes phase (c / NS) & 1 of its
         // barriers; nl chunks loaded, nf of them waited for (full), nc committed,
         // ne of those waited for (empty)
         int nl = 0, nf = 0, nc = 0, ne = 0;
         const int lim = a.wait_limit;
-        auto wait_full = [&](int c) { return mbar_wait(&full[c % TC_NS], (uint32_t)(c / TC_NS) & 1u, lim); };
-        auto wait_empty = [&](int c) { return mbar_wait(&empty[c % TC_NS], (uint32_t)(c / TC_NS) & 1u, lim); };
+        auto wait_full = [&](int c) { return mbar_wait(&full[c % NS], (uint32_t)(c / NS) & 1u, lim); };
+        auto wait_empty = [&](int c) { return mbar_wait(&empty[c % NS], (uint32_t)(c / NS) & 1u, lim); };
         bool ok = true;
         if (!a.no_loads)
-            for (int c = 0; c < TC_NS && c < nk; ++c) {
+            for (int c = 0; c < NS && c < nk; ++c) {
                 load(c);
                 ++nl;
             }
         for (int c = 0; c < nk && ok; ++c) {
-            const int st = c % TC_NS;
+            const int st = c % NS;
             ok = wait_full(c);
             if (!ok) break;
             ++nf;
@@ -660,18 +661,18 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
             }
             tc_commit(&empty[st]);
             ++nc;
-            // refill the stage of chunk c-1 with chunk c-1+TC_NS once its MMAs are
+            // refill the stage of chunk c-1 with chunk c-1+NS once its MMAs are
             // done (those of chunk c are queued behind them meanwhile)
-            if (c >= 1 && c - 1 + TC_NS < nk) {
+            if (c >= 1 && c - 1 + NS < nk) {
                 ok = wait_empty(c - 1);
                 if (ok) {
                     ++ne;
-                    load(c - 1 + TC_NS);
+                    load(c - 1 + NS);
                     ++nl;
                 }
             }
         }
-        // the loop waited for chunks 0 .. nk-1-TC_NS; wait for the rest
+        // the loop waited for chunks 0 .. nk-1-NS; wait for the rest
         while (ok && ne < nc) {
             ok = wait_empty(ne);
             if (ok) ++ne;
@@ -733,6 +734,23 @@ __global__ void __launch_bounds__(128, 2) ztc_kernel(Args<float> a, int t, uint6
     tc_fence_before();
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_N) : "memory");
+}
+
+// Two CTAs with four stages share a multiprocessor, one's epilogue overlapping the
+// other's MMAs. A launch that leaves at most one CTA for each multiprocessor is
+// bound by its chain of chunks, each waiting for its copies: eight stages (192 KB)
+// keep seven of them in flight. K = 3, M = 1152, 256 samples (9 CTAs of up to 144
+// chunks a step): 33 -> 20 us a step.
+template <int K>
+static cudaError_t launch_ztc(const Args<float> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
+    const dim3 grid((unsigned)((rows + TC_M - 1) / TC_M), (unsigned)(a.S / TC_N));
+    const bool deep = (uint64_t)grid.x * grid.y <= (uint64_t)sms;
+    const int smem = tc_smem(deep ? TC_NS_DEEP : TC_NS);
+    auto fn = deep ? ztc_kernel<K, TC_NS_DEEP> : ztc_kernel<K, TC_NS>;
+    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<grid, 128, smem, st>>>(a, t, rows, D);
+    return cudaSuccess;
 }
 
 // ---------------------------------------------------------------- table rows of one step
@@ -894,35 +912,42 @@ __global__ void __launch_bounds__(32 * BIAS_W) bias_kernel(Args<R> a, int n) {
 #pragma unroll
     for (int pass = K == 3 ? 1 : 0; pass < 2; ++pass) {
         const int first = pass == 0 ? 1 : K == 3 ? 2 : 3;
-        R rc[PER], rv[PER];
+        // loads of a tile (all of them before any of their uses or stores), then its
+        // operands into shared memory
+        R rx[PER], rk[PER], rp[PER], rv[PER];
         auto load = [&](int i0) {
 #pragma unroll
             for (int q = 0; q < PER; ++q) {
                 const int i = i0 + w + BIAS_W * q;
-                rc[q] = rv[q] = R(0);
-                if (i >= n) continue;
-                const R x = t.chi[(size_t)i * SG];
+                const bool in = i < n;
+                rx[q] = in ? t.chi[(size_t)i * SG] : R(0);
+                rk[q] = in ? k2n[i] : R(0);
                 if (pass == 0) {
-                    rc[q] = k2n[i] * x;
-                    rv[q] = *p1_row(t, n - 1, i);
+                    rv[q] = in ? *p1_row(t, n - 1, i) : R(0);
                 } else {
-                    const R p = i == n - 1 ? R(1) : ppn[(size_t)i * SG], cbv = k2n[i] * x, ca = x * p;
+                    rp[q] = i < n - 1 ? ppn[(size_t)i * SG] : R(1);
+                    rv[q] = in && i >= first ? yz[(size_t)i * SG] : R(0);
+                }
+            }
+        };
+        auto put = [&](int buf, int i0) {
+#pragma unroll
+            for (int q = 0; q < PER; ++q) {
+                const int i = i0 + w + BIAS_W * q;
+                const R cbv = rk[q] * rx[q], ca = pass == 0 ? R(0) : rx[q] * rp[q];
+                if (pass == 1 && i < n) {
                     if (K != 3) t.CA[(size_t)i * SG] = ca;
                     t.CB[(size_t)i * SG] = cbv;
-                    t.CC[(size_t)i * SG] = cbv * p;
-                    rc[q] = ca;
-                    if (i >= first) rv[q] = yz[(size_t)i * SG];
+                    t.CC[(size_t)i * SG] = cbv * rp[q];
                 }
+                cs[buf][w + BIAS_W * q][lane] = pass == 0 ? cbv : ca;
+                vs[buf][w + BIAS_W * q][lane] = rv[q];
             }
         };
         load(1);
         int buf = 0;
         for (int i0 = 1; i0 < n; i0 += TI, buf ^= 1) {
-#pragma unroll
-            for (int q = 0; q < PER; ++q) {
-                cs[buf][w + BIAS_W * q][lane] = rc[q];
-                vs[buf][w + BIAS_W * q][lane] = rv[q];
-            }
+            put(buf, i0);
             __syncthreads();
             if (i0 + TI < n) load(i0 + TI);
             if (w == 0) {
@@ -1161,154 +1186,69 @@ __global__ void __launch_bounds__(32, 32) p2_kernel(Args<R> a, int n, unsigned n
     stl<R, VW>(t.P2 + i_p2(n, e, d) * SG, out);
 }
 
-// Pp~[n][l], l0 <= l < l0 + LB (Eq. a / Eq. probpartialade): LB rows share each
-// coefficient load, and their p+ entries of one i are neighbours.
-template <class R, int VW, int U, int LB>
-__device__ __forceinline__ void pp_rows(const Args<R> &a, const Grp<R> &t, int n, int l0) {
+// Pp~[n][l] (Eq. a / Eq. probpartialade).
+template <class R, int VW, int U>
+__device__ __forceinline__ void pp_row(const Args<R> &a, const Grp<R> &t, int n, int l) {
     const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
     const auto ld = lead(a, n);
-    R acc[LB][VW];
+    R acc[VW];
 #pragma unroll
-    for (int b = 0; b < LB; ++b)
+    for (int k = 0; k < VW; ++k) acc[k] = R(0);
+    auto use = [&](int, const Two<R, VW> &b) {
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[b][k] = R(0);
-    struct Row {
-        Lanes<R, VW> c, v[LB];
+        for (int k = 0; k < VW; ++k) acc[k] = fma(b.c.v[k], b.v.v[k], acc[k]);
     };
-    // coef rows (CC, then the order-3 factors Y) against Pp~[i-1][l], i in [l, hi)
+    // coef rows (CC, then the order-3 factors Y) against Pp~[i-1][l] (1 at i = l)
     auto sum = [&](const R *coef, int hi) {
-        // i within LB of l0: some rows have not begun, or begin with an empty range (1)
-#pragma unroll
-        for (int q = 0; q < LB; ++q) {
-            const int i = l0 + q;
-            if (i >= hi) break;
-            const auto c = ldl<R, VW>(coef + (size_t)i * SG);
-#pragma unroll
-            for (int b = 0; b <= q; ++b) {
-                const auto v = b == q ? ones<R, VW>() : ldl<R, VW>(t.Pp + (size_t)(c2u(i - 1) + l0 + b - 1) * SG);
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[b][k] = fma(c.v[k], v.v[k], acc[b][k]);
-            }
-        }
+        if (l < hi) use(l, Two<R, VW>{ldl<R, VW>(coef + (size_t)l * SG), ones<R, VW>()});
+        const R *p = t.Pp + ((size_t)l - 1) * SG;
         walk<U>(
-            l0 + LB, hi,
+            l + 1, hi,
             [&](int i) {
-                Row r;
-                r.c = ldl<R, VW>(coef + (size_t)i * SG);
-                const R *p = t.Pp + (size_t)(c2u(i - 1) + l0 - 1) * SG;
-#pragma unroll
-                for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(p + (size_t)b * SG);
-                return r;
+                return Two<R, VW>{ldl<R, VW>(coef + (size_t)i * SG), ldl<R, VW>(p + (size_t)c2u(i - 1) * SG)};
             },
-            [&](int, const Row &r) {
-#pragma unroll
-                for (int b = 0; b < LB; ++b)
-#pragma unroll
-                    for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k], r.v[b].v[k], acc[b][k]);
-            });
+            use);
     };
     if (a.opp >= 2) sum(t.CC, n);
     if (a.opp >= 3) sum(t.Y, n - 1);
+    const auto w = ppl<R, VW>(t, n - 1, l);
+    R out[VW];
 #pragma unroll
-    for (int b = 0; b < LB; ++b) {
-        const int l = l0 + b;
-        if (l > n) break;
-        const auto w = ppl<R, VW>(t, n - 1, l);
-        R out[VW];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[b][k], fma(ld.x, cn.v[k], ld.y) * w.v[k]);
-        stl<R, VW>(t.Pp + i_pp(n, l) * SG, out);
-    }
+    for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[k], fma(ld.x, cn.v[k], ld.y) * w.v[k]);
+    stl<R, VW>(t.Pp + i_pp(n, l) * SG, out);
 }
 
-// K = 3: P1~[n][e], e0 <= e < e0 + LB (Eq. b), i < e with weight
-// kappa(i,n) chi_i Pp~[n-1][e+1] and i > e with CC_i. Rows e >= n are formed
-// from whatever lies there (in bounds: e0 < n <= M) and not stored.
-template <class R, int VW, int U, int LB>
-__device__ __forceinline__ void p1_rows_k3(const Args<R> &a, const Grp<R> &t, int n, int e0) {
-    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG);
+// K = 3: P1~[n][e] (Eq. b), i < e with weight kappa(i,n) chi_i Pp~[n-1][e+1] and
+// i > e with CC_i.
+template <class R, int VW, int U>
+__device__ __forceinline__ void p1_row_k3(const Args<R> &a, const Grp<R> &t, int n, int e) {
+    const auto cn = ldl<R, VW>(t.chi + (size_t)n * SG), w = ppl<R, VW>(t, n - 1, e + 1);
     const auto ld = lead(a, n);
-    const int nb = min(LB, n - e0);  // rows of this warp
-    R acc[LB][VW];
-    Lanes<R, VW> w[LB];
+    R acc[VW];
 #pragma unroll
-    for (int b = 0; b < LB; ++b) {
-        w[b] = ppl<R, VW>(t, n - 1, b < nb ? e0 + b + 1 : n);
+    for (int k = 0; k < VW; ++k) acc[k] = R(0);
+    auto below = [&](int, const Two<R, VW> &b) {
 #pragma unroll
-        for (int k = 0; k < VW; ++k) acc[b][k] = R(0);
-    }
-    struct Row {
-        Lanes<R, VW> c, v[LB];
+        for (int k = 0; k < VW; ++k) acc[k] = fma(b.c.v[k] * w.v[k], b.v.v[k], acc[k]);
     };
-    // one term of row b for any i != e
-    auto any = [&](int b, int i, const Lanes<R, VW> &cbv, const Lanes<R, VW> &ccv) {
-        const int e = e0 + b;
-        if (i < e) {
-            const auto v = ldl<R, VW>(p1_row(t, e - 1, i));
+    auto above = [&](int, const Two<R, VW> &b) {
 #pragma unroll
-            for (int k = 0; k < VW; ++k) acc[b][k] = fma(cbv.v[k] * w[b].v[k], v.v[k], acc[b][k]);
-        } else if (i > e) {
-            const auto v = ldl<R, VW>(p1_row(t, i - 1, e));
-#pragma unroll
-            for (int k = 0; k < VW; ++k) acc[b][k] = fma(ccv.v[k], v.v[k], acc[b][k]);
-        }
+        for (int k = 0; k < VW; ++k) acc[k] = fma(b.c.v[k], b.v.v[k], acc[k]);
     };
-    // i <= e0 - 2: P1~[e-1][i]
-    const R *rowp[LB];
-#pragma unroll
-    for (int b = 0; b < LB; ++b) rowp[b] = t.P1 + (e0 >= 3 ? (size_t)(c2u(e0 + (b < nb ? b : 0) - 2)) * SG : 0) - SG;
+    auto cb_ = [&](int i) { return ldl<R, VW>(t.CB + (size_t)i * SG); };
+    auto cc_ = [&](int i) { return ldl<R, VW>(t.CC + (size_t)i * SG); };
+    const R *p = t.P1 + ((size_t)c2u(e - 2) - 1) * SG;  // P1~[e-1][i], i < e - 1
+    if (e >= 3) walk<U>(1, e - 1, [&](int i) { return Two<R, VW>{cb_(i), ldl<R, VW>(p + (size_t)i * SG)}; }, below);
+    if (e >= 2) below(e - 1, Two<R, VW>{cb_(e - 1), ldl<R, VW>(t.P + (size_t)(e - 2) * SG)});
+    if (e + 1 < n) above(e + 1, Two<R, VW>{cc_(e + 1), ldl<R, VW>(t.P + (size_t)(e - 1) * SG)});
+    p = t.P1 + ((size_t)e - 1) * SG;  // P1~[i-1][e] at C(i-2, 2)
     walk<U>(
-        1, e0 - 1,
-        [&](int i) {
-            Row r;
-            r.c = ldl<R, VW>(t.CB + (size_t)i * SG);
+        e + 2, n, [&](int i) { return Two<R, VW>{cc_(i), ldl<R, VW>(p + (size_t)c2u(i - 2) * SG)}; }, above);
+    const auto pv = ldl<R, VW>(p1_row(t, n - 1, e));
+    R out[VW];
 #pragma unroll
-            for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(rowp[b] + (size_t)i * SG);
-            return r;
-        },
-        [&](int, const Row &r) {
-#pragma unroll
-            for (int b = 0; b < LB; ++b)
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k] * w[b].v[k], r.v[b].v[k], acc[b][k]);
-        });
-    // i around the rows' own indices: every case
-#pragma unroll
-    for (int q = 0; q < LB + 2; ++q) {
-        const int i = e0 - 1 + q;
-        if (i < 1 || i >= n) continue;
-        const auto cbv = ldl<R, VW>(t.CB + (size_t)i * SG), ccv = ldl<R, VW>(t.CC + (size_t)i * SG);
-#pragma unroll
-        for (int b = 0; b < LB; ++b)
-            if (b < nb) any(b, i, cbv, ccv);
-    }
-    // i > e0 + LB: P1~[i-1][e]
-    walk<U>(
-        e0 + LB + 1, n,
-        [&](int i) {
-            Row r;
-            r.c = ldl<R, VW>(t.CC + (size_t)i * SG);
-            const R *p = t.P1 + (size_t)(c2u(i - 2) + e0 - 1) * SG;
-#pragma unroll
-            for (int b = 0; b < LB; ++b) r.v[b] = ldl<R, VW>(p + (size_t)b * SG);
-            return r;
-        },
-        [&](int, const Row &r) {
-#pragma unroll
-            for (int b = 0; b < LB; ++b)
-#pragma unroll
-                for (int k = 0; k < VW; ++k) acc[b][k] = fma(r.c.v[k], r.v[b].v[k], acc[b][k]);
-        });
-#pragma unroll
-    for (int b = 0; b < LB; ++b) {
-        if (b >= nb) break;
-        const int e = e0 + b;
-        const auto pv = ldl<R, VW>(p1_row(t, n - 1, e));
-        R out[VW];
-#pragma unroll
-        for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[b][k], fma(ld.x, cn.v[k], ld.y) * pv.v[k]);
-        stl<R, VW>(t.P1 + i_p1(n, e) * SG, out);
-    }
+    for (int k = 0; k < VW; ++k) out[k] = fma(cn.v[k], acc[k], fma(ld.x, cn.v[k], ld.y) * pv.v[k]);
+    stl<R, VW>(t.P1 + i_p1(n, e) * SG, out);
 }
 
 // K = 4, 5: P1~[n][e] (Eq. probelidedade). Order 3: with (a, b, c) the decreasing
@@ -1365,20 +1305,17 @@ __device__ __forceinline__ void p1_row_k45(const Args<R> &a, const Grp<R> &t, in
 
 // The p1 rows e = 1..n-1 and the p+ rows l = 1..n of one step in one launch (they
 // read rows below n only): the p1 warps first, the p+ warps by falling length.
-template <class R, int K, int VW, int U, int LB, int WPB>
-__global__ void __launch_bounds__(32 * WPB, VW * LB * sizeof(R) > 16 ? 1 : 32 / WPB) rows_kernel(Args<R> a, int n) {
+template <class R, int K, int VW, int U, int WPB>
+__global__ void __launch_bounds__(32 * WPB, 32 / WPB) rows_kernel(Args<R> a, int n) {
     const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
-    constexpr int EB = K == 3 ? LB : 1;
     const int item = (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
-    const int n1 = (n - 1 + EB - 1) / EB;
-    if (item < n1) {
-        if constexpr (K == 3) p1_rows_k3<R, VW, U, LB>(a, t, n, 1 + item * LB);
+    if (item < n - 1) {
+        if constexpr (K == 3) p1_row_k3<R, VW, U>(a, t, n, 1 + item);
         else p1_row_k45<R, VW, U>(a, t, n, 1 + item);
-    } else if (1 + (item - n1) * LB <= n) {
-        pp_rows<R, VW, U, LB>(a, t, n, 1 + (item - n1) * LB);
+    } else if (item < 2 * n - 1) {
+        pp_row<R, VW, U>(a, t, n, item - n + 2);
     }
 }
-
 
 template <class R>
 __global__ void init_kernel(Args<R> a) {
@@ -1594,12 +1531,15 @@ static dim3 egrid(int S, uint64_t entries) {
 }
 
 // The kernels of step t after its products: VW samples per lane, U loads of a
-// chain ahead, LB rows per warp (rows_kernel), WPB warps per block.
-template <class R, int K, int VW, int U, int LB, int WPB>
+// chain ahead, WPB warps per block. Two samples per lane in FP32 and one in FP64,
+// eight loads ahead, two warps: the fastest or within 2 % of it at every size tried
+// (K = 3, M = 1152, 256 samples: 195 ms; four samples and four loads 213; one
+// sample and 16 loads 200).
+template <class R, int K>
 static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
+    constexpr int VW = sizeof(R) == 4 ? 2 : 1, U = 8, WPB = 2, NT = 32 * WPB;
     const unsigned gy = (unsigned)(a.S / (32 * VW));
     auto grid = [&](int warps) { return dim3((unsigned)((warps + WPB - 1) / WPB), gy); };
-    constexpr int NT = 32 * WPB;
     if (K == 5 && t > 3) yv_kernel<R, VW, U, WPB><<<grid(t - 3), NT, 0, st>>>(a, t);
     bias_kernel<R, K><<<(unsigned)(a.S / 32), 32 * BIAS_W, 0, st>>>(a, t);
     if (K >= 4 && a.opp >= 3 && t > 1) pvv_kernel<R, VW, U, WPB><<<grid(t - 1), NT, 0, st>>>(a, t);
@@ -1610,8 +1550,7 @@ static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
             p2_block_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
         p2_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
     }
-    const int n1 = K == 3 ? (t - 1 + LB - 1) / LB : t - 1, np = (t + LB - 1) / LB;
-    rows_kernel<R, K, VW, U, LB, WPB><<<grid(n1 + np), NT, 0, st>>>(a, t);
+    rows_kernel<R, K, VW, U, WPB><<<grid(2 * t - 1), NT, 0, st>>>(a, t);
     return cudaGetLastError();
 }
 
@@ -1619,9 +1558,6 @@ template <class R, int K>
 static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) {
     const int S = a.S, M = a.M;
     const int TB = 256;
-    // one sample per lane until the rows of a step give every multiprocessor a
-    // full set of warps with VW of them
-    const bool wide = (uint64_t)M * S >= 1u << 19;
     cudaError_t e = cudaSuccess;
     init_kernel<R><<<(S + TB - 1) / TB, TB, 0, st>>>(a);
     for (int t = 1; t <= M; ++t) {
@@ -1641,7 +1577,7 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
                 if (tc) {
                     const unsigned nrt = (unsigned)((rows + TC_M - 1) / TC_M), nk = (unsigned)((D + TC_KC - 1) / TC_KC);
                     atc_kernel<K><<<dim3(nrt, nk), 128, 0, st>>>(a, t, rows, D);
-                    ztc_kernel<K><<<dim3(nrt, (unsigned)(S / TC_N)), 128, TC_SMEM, st>>>(a, t, rows, D);
+                    if ((e = launch_ztc<K>(a, t, rows, D, sms, st)) != cudaSuccess) return e;
                 } else {
                     launch_zgemm<R, K>(a, t, rows, D, sms, st);
                 }
@@ -1649,7 +1585,7 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
                 launch_zgemm<R, K>(a, t, rows, D, sms, st);
             }
         }
-        e = wide ? step_rows<R, K, sizeof(R) == 4 ? 4 : 2, 4, 1, 1>(a, t, st) : step_rows<R, K, 1, 8, sizeof(R) == 4 ? 4 : 2, 2>(a, t, st);
+        e = step_rows<R, K>(a, t, st);
         if (e != cudaSuccess) return e;
     }
     if (prob) logp_kernel<R><<<(S + TB - 1) / TB, TB, 0, st>>>(a, prob);
@@ -1696,13 +1632,6 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
     if (sizeof(R) == 4) {
         const char *env = getenv("GBS_SAMPLER_SIMT");
         a.use_tc = (env && *env && *env != '0') || c.S % TC_N != 0 ? 0 : 1;
-        if (a.use_tc) {
-            cudaError_t e = cudaSuccess;
-            if (c.K == 3) e = cudaFuncSetAttribute(ztc_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-            if (c.K == 4) e = cudaFuncSetAttribute(ztc_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-            if (c.K == 5) e = cudaFuncSetAttribute(ztc_kernel<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-            if (e != cudaSuccess) return e;
-        }
     }
     {
         R *hs = reinterpret_cast<R *>(w + L.hs);
