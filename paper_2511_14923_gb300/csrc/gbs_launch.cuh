@@ -3,9 +3,17 @@
 // kernels, the persistent prefix-tree kernel and its launcher, each templated on
 // DISP (first moments carried through the elimination, FP64 only).
 #pragma once
+#include "gbs_chunk.cuh"
 #include "gbs_tree.cuh"
 
 namespace gbs {
+
+// Modes below which order 4 runs by chunks of pairs (launch_order4), and pairs per
+// chunk: one chunk a prefix up to 182 modes.
+constexpr int kOrder4ChunkedZ = 224, kOrder4ChunkedR = 64;
+constexpr uint32_t kOrder4Pairs = 16384;
+// Shared memory a chunk may take: 227 KB less the kernel's static part.
+constexpr size_t kChunkSmem = 226 * 1024;
 
 // Flat kernels of orders 1-3: one thread per subset of colex rank first + i,
 // i < count (the whole order, or the rank range of a range call's top order).
@@ -255,6 +263,47 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
     }
 }
 
+// Order 3, top elements in [c_lo, c_hi), by chunks (gbs_chunk.cuh) of 16 for every
+// multiprocessor; at least 256 pairs (two a thread) and at most 8192 (eliminating
+// c3, up to 12 operations for each of c2 modes, is then below 5 % of the leaves').
+// kt, FP64: M = 1152 43.4 -> 14.7 ms (36 FP64 instructions an entry: the FP64
+// pipe's own 14.6), M = 200 0.248 -> 0.112, M = 20 26.0 -> 23.5 us, against one
+// thread per subset redoing the elimination. That kernel is left for displaced
+// states whose modes do not fit shared memory.
+template <int MODE, bool DISP>
+static cudaError_t launch_order3(const FwdArgs &a, bool write_p0, int c_lo, int c_hi, cudaStream_t st) {
+    const uint64_t first = binom(c_lo, 3), n = binom(c_hi, 3) - first;
+    if (n == 0) return cudaSuccess;
+    const uint64_t want = (n / ((uint64_t)a.sms * 16) + 255) / 256 * 256;
+    const uint32_t L = want < 256 ? 256 : want > 8192 ? 8192 : (uint32_t)want;
+    using Shape = ChunkShape<1, 0, DISP>;
+    const size_t smem = chunk_smem(c_hi - 1, L, Shape::PX, Shape::PR);
+    if (smem <= kChunkSmem) return launch_chunk<1, MODE, 0, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
+    order3_kernel<MODE, DISP><<<(unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS), FLAT_THREADS, 0, st>>>(a, write_p0,
+                                                                                                 first, n);
+    return cudaGetLastError();
+}
+
+// Order 4, top elements in [c_lo, c_hi): by chunks below kOrder4ChunkedZ / R
+// modes (FP64, refined) and, for displaced states, wherever the modes fit shared
+// memory; else by the prefix tree. A chunk forms its leaves' blocks from the
+// prefix's pivot rows (8 FP64 or 48 pair operations more a leaf) and needs no
+// slot, queue or batches. kt, us, tree at its best schedule / chunks:
+//   FP64       M = 20 52.7 / 36.4  50 77.7 / 75  100 434 / 391  144 1526 / 1460  300 23500 / 25800
+//   refined    M = 20 43.7 / 35.4  50 53.6 / 52.5  77 85.7 / 93  144 461 / 492
+//   displaced  M = 50 124 / 98  100 787 / 629  300 49700 / 43900
+template <int MODE, int PREC, bool DISP>
+static cudaError_t launch_order4(const FwdArgs &a, bool write_p0, int c_lo, int c_hi, cudaStream_t st) {
+    using Shape = ChunkShape<2, PREC, DISP>;
+    const size_t smem = chunk_smem(a.M - 2, kOrder4Pairs, Shape::PX, Shape::PR);
+    const int below = DISP ? GBS_MAX_MODES + 1 : PREC == 1 ? kOrder4ChunkedR : kOrder4ChunkedZ;
+    if (a.M < below && smem <= kChunkSmem) {
+        if (c_hi <= 3 || c_hi <= c_lo) return cudaSuccess;
+        return launch_chunk<2, MODE, PREC, DISP>(a, write_p0, c_lo, c_hi, kOrder4Pairs, smem, st);
+    }
+    return launch_tree<4, MODE, PREC, DISP>(a, write_p0, st);
+}
+
 template <int MODE, bool DISP>
 static cudaError_t launch_mode(const FwdArgs &a, cudaStream_t st) {
     const int M = a.M;
@@ -287,18 +336,21 @@ static cudaError_t launch_mode(const FwdArgs &a, cudaStream_t st) {
     }
     mark(3);
     if (a.kmax >= 3) {
-        span(3, f, n);
-        if (n) order3_kernel<MODE, DISP><<<grid(n), FLAT_THREADS, 0, st>>>(a, wp(3), f, n);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const bool part = a.top && a.kmax == 3;
+        if ((e = launch_order3<MODE, DISP>(a, wp(3), part ? a.c_lo : 0, part ? a.c_hi : M, st)) != cudaSuccess) return e;
     }
     mark(4);
     if (a.kmax >= 4) {
-        e = a.precision == 0 ? launch_tree<4, MODE, 0, DISP>(a, wp(4), st) : launch_tree<4, MODE, 1, DISP>(a, wp(4), st);
+        const bool part = a.top && a.kmax == 4;
+        const int lo = part ? a.c_lo : 0, hi = part ? a.c_hi : M;
+        if constexpr (DISP) e = launch_order4<MODE, 0, true>(a, wp(4), lo, hi, st);
+        else e = a.precision == 0 ? launch_order4<MODE, 0, false>(a, wp(4), lo, hi, st) : launch_order4<MODE, 1, false>(a, wp(4), lo, hi, st);
         if (e != cudaSuccess) return e;
     }
     mark(5);
     if (a.kmax >= 5) {
-        e = a.precision == 0 ? launch_tree<5, MODE, 0, DISP>(a, wp(5), st) : launch_tree<5, MODE, 1, DISP>(a, wp(5), st);
+        if constexpr (DISP) e = launch_tree<5, MODE, 0, true>(a, wp(5), st);
+        else e = a.precision == 0 ? launch_tree<5, MODE, 0, false>(a, wp(5), st) : launch_tree<5, MODE, 1, false>(a, wp(5), st);
         if (e != cudaSuccess) return e;
     }
     mark(6);
