@@ -19,7 +19,9 @@ namespace gbs {
 cudaError_t launch_forward_displaced(const FwdArgs &a_in, cudaStream_t st) {
     FwdArgs a = a_in;
     a.precision = 0;
-    a.variant = 0;
+    a.variant = kDefaultCfg.variant;
+    a.grain = kDefaultCfg.grain;
+    a.ccap = kDefaultCfg.ccap;
     if (a.ev) cudaEventRecord(a.ev[0], st);
     cudaError_t e = launch_pack(a, st);
     if (e != cudaSuccess) return e;

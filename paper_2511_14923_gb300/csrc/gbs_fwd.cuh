@@ -75,6 +75,28 @@ constexpr int kVariant6MaxM = kQuadXC + 1;
 constexpr int kNoSlotCC = 24;
 constexpr int kNoSlotYC = 160;
 constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1
+// Schedule of an untuned forward call, from sweeps of shape x grain (kt, M = 20 to
+// 300, kmax = 4 and 5; the tuner still finds the last percents):
+//   refined: 256 x 4 where its x area admits M (M = 144, kmax = 5: 13.2 ms against
+//     17.7 at 512 x 1; M = 50: 0.177 against 0.300), 384 x 2 up to its own limit;
+//     one item per CTA slot below 128 modes with order 5 (77: 0.726 against 0.738),
+//     where a second round of items would wait for the first, else two;
+//   FP64: 256 x 2, one item per CTA slot (M = 111, kmax = 5: 11.2 against 12.3;
+//     M = 50: 0.35 against 0.47); a kmax = 4 table large enough for the prefix tree
+//     (gbs_launch.cuh) 512 x 1 with eight (M = 300: 23.5 against 24.9).
+inline TreeCfg default_cfg(int M, int kmax, int precision) {
+    TreeCfg c = kDefaultCfg;
+    if (precision == 1) {
+        c.variant = M <= kVariant6MaxM ? 6 : M <= kVariant5MaxM ? 5 : 0;
+        c.grain = kmax == 5 && M < 128 ? 1 : 2;
+    } else if (kmax == 5) {
+        c.variant = M <= kVariant1MaxM ? 1 : 0;
+        c.grain = c.variant == 1 ? 1 : 2;
+    } else {
+        c.grain = 8;
+    }
+    return c;
+}
 // Number of CTA shapes (variants 0..kNumVariants-1); 7 and 8 are the 256 x 4 and
 // 256 x 3 shapes in thread-block clusters of 4 and 3 CTAs sharing one slot, 9 the
 // 256 x 4 shape without slots.

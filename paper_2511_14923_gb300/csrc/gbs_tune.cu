@@ -179,7 +179,7 @@ TreeCfg tuned_cfg(int sms, int M, int kmax, int precision) {
     std::lock_guard<std::mutex> lock(g_mu);
     load_locked();
     auto it = g_table.find(Key{device_cc(), sms, M, kmax, precision});
-    return it == g_table.end() ? kDefaultCfg : it->second.cfg;
+    return it == g_table.end() ? default_cfg(M, kmax, precision) : it->second.cfg;
 }
 
 bool tuned_batch_cfg(int sms, const gbs_instance *inst, int n, int precision, TreeCfg &cfg) {
