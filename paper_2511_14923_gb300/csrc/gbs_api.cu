@@ -119,7 +119,10 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
     a.precision = precision;
     a.A = reinterpret_cast<double *>(w + L.A_off);
     a.Af = reinterpret_cast<float *>(a.A + 4 * (size_t)M * M);
-    a.p0f = reinterpret_cast<float *>(w + L.p0f_off);
+    if (precision == GBS_FP32_REFINED && kmax >= 4 && (mode == gbs::MODE_KAPPA || mode == gbs::MODE_SPINK)) {
+        a.p0p = reinterpret_cast<float2 *>(w + L.p0p_off);
+        a.kyp = reinterpret_cast<float2 *>(w + L.kyp_off);
+    }
     a.p0 = (mode == gbs::MODE_P0 && !range.on()) ? out : reinterpret_cast<double *>(w + L.p0_off);
     a.out = range.on() ? reinterpret_cast<double *>(w + range_low_off(L)) : out;
     if (range.on()) {
@@ -467,7 +470,10 @@ int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precis
     a.precision = precision;
     a.A = reinterpret_cast<double *>(w + L.A_off);
     a.Af = reinterpret_cast<float *>(a.A + 4 * (size_t)M * M);
-    a.p0f = reinterpret_cast<float *>(w + L.p0f_off);
+    if (precision == GBS_FP32_REFINED && kmax >= 4) {
+        a.p0p = reinterpret_cast<float2 *>(w + L.p0p_off);
+        a.kyp = reinterpret_cast<float2 *>(w + L.kyp_off);
+    }
     a.p0 = reinterpret_cast<double *>(w + L.p0_off);
     a.out = kappa_out;
     a.status = reinterpret_cast<unsigned *>(w + L.status_off);

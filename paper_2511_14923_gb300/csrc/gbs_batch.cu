@@ -41,7 +41,7 @@ struct InstDev {
     const double *V;
     double *out;
     double *A;
-    float *p0f;  // P0({x}) as float pairs (refined path)
+    float2 *p0p, *kyp;  // float pairs of the lower orders (refined path, kmax >= 4; else null)
     double *p0;
     int M, kmax;
     uint32_t c4off[2];   // offsets into the c4-prefix pool for orders 4 and 5
@@ -134,10 +134,16 @@ void build_plan(const gbs_instance *in, int n, int precision, int sms, int grid,
         I.kmax = x.kmax;
         I.A = reinterpret_cast<double *>(base + off);  // FP64 blocks, then the float-pair copy
         off = a256(off + 2 * sizeof(double) * 4 * (size_t)x.M * x.M);
-        I.p0f = reinterpret_cast<float *>(base + off);
-        off = a256(off + 2 * sizeof(float) * (size_t)x.M);
         I.p0 = reinterpret_cast<double *>(base + off);
         off = a256(off + sizeof(double) * (x.kmax > 1 ? order_offset(x.M, x.kmax) : 0));
+        I.p0p = I.kyp = nullptr;
+        if (x.kmax >= 4) {
+            const size_t n = sizeof(float2) * (size_t)order_offset(x.M, x.kmax);
+            if (precision == 1) I.p0p = reinterpret_cast<float2 *>(base + off);
+            off = a256(off + n);
+            if (precision == 1) I.kyp = reinterpret_cast<float2 *>(base + off);
+            off = a256(off + n);
+        }
         for (int d = 4; d <= 5; ++d) {
             I.target[d - 4] = target[d - 4];
             I.c4off[d - 4] = (uint32_t)hp.pool.size();
@@ -185,7 +191,8 @@ __device__ __forceinline__ FwdArgs inst_args(const InstDev &I, unsigned *status,
     a.precision = precision;
     a.A = I.A;
     a.Af = reinterpret_cast<float *>(I.A + 4 * (size_t)I.M * I.M);
-    a.p0f = I.p0f;
+    a.p0p = I.p0p;
+    a.kyp = I.kyp;
     a.p0 = I.p0;
     a.out = I.out;
     a.status = status;
@@ -194,10 +201,11 @@ __device__ __forceinline__ FwdArgs inst_args(const InstDev &I, unsigned *status,
     return a;
 }
 
-template <int D, int PREC, int NT, int XC>
+template <int D, int PREC, int NT, int XC, int CC>
 __device__ void tree_phase(const PlanHdr &h, const InstDev *inst, const uint64_t *pref, const uint32_t *pool,
                            unsigned *status, unsigned *counters, double *slot, unsigned char *smem) {
-    TreeShared<D, XC> &sh = *reinterpret_cast<TreeShared<D, XC> *>(smem);
+    using SH = TreeShared<D, XC, false, CC>;
+    SH &sh = *reinterpret_cast<SH *>(smem);
     __shared__ int s_dec[6];
     __shared__ FwdArgs s_args;
     const int n = h.n;
@@ -236,14 +244,14 @@ __device__ void tree_phase(const PlanHdr &h, const InstDev *inst, const uint64_t
         const int c4 = s_dec[1], c5 = s_dec[2], s = s_dec[3], nc = s_dec[4];
         __syncthreads();
         if (i < 0) break;
-        tree_item<D, MODE_KAPPA, PREC, NT, XC>(s_args, sh, slot, c4, c5, s, nc, D < GBS_MAX_ORDER && D < s_args.kmax,
+        tree_item<D, MODE_KAPPA, PREC, NT, XC, false, false, CC>(s_args, sh, slot, c4, c5, s, nc, D < GBS_MAX_ORDER && D < s_args.kmax,
                                                h.ccap);
     }
 }
 
 // The batched kernel for one CTA shape: NT threads, XC x-entries of shared
 // memory, at least MINB resident CTAs per multiprocessor.
-template <int PREC, int NT, int XC, int MINB>
+template <int PREC, int NT, int XC, int MINB, int CC>
 __global__ void __launch_bounds__(NT, MINB) batched_kernel(char *ws) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::grid_group grid = cg::this_grid();
@@ -293,14 +301,14 @@ __global__ void __launch_bounds__(NT, MINB) batched_kernel(char *ws) {
     grid.sync();
     double *slot = reinterpret_cast<double *>(ws + *reinterpret_cast<const size_t *>(ws + 128)) +
                    (size_t)blockIdx.x * h.slot_doubles;
-    tree_phase<4, PREC, NT, XC>(h, inst, pref, pool, status, counters, slot, smem_raw);
+    tree_phase<4, PREC, NT, XC, CC>(h, inst, pref, pool, status, counters, slot, smem_raw);
     grid.sync();
-    tree_phase<5, PREC, NT, XC>(h, inst, pref, pool, status, counters, slot, smem_raw);
+    tree_phase<5, PREC, NT, XC, CC>(h, inst, pref, pool, status, counters, slot, smem_raw);
 }
 
 // Kernel of one CTA shape (variant numbering as for the single-instance
-// schedules: 0 = 512 x 1, 1 = 256 x 2, refined only 2 = 640 x 1, 3 = 256 x 3,
-// 4 = 768 x 1 with a 2048-entry x area, 5 = 384 x 2 with a 960-entry x area,
+// schedules: 0 = 512 x 1, 1 = 256 x 2, refined only 2 = 128 x 6 with a 304-entry x
+// area, 3 = 256 x 3, 4 = 256 x 3 with a 672-entry x area, 5 = 384 x 2 with a 960-entry x area,
 // 6 = 256 x 4 with a 384-entry x area).
 struct KernelInfo {
     void *fn;
@@ -308,15 +316,17 @@ struct KernelInfo {
     size_t smem;
 };
 
-template <int PREC, int NT, int XC, int MINB>
+template <int PREC, int NT, int XC, int MINB, int CC = CCAP>
 KernelInfo kinfo() {
-    return KernelInfo{(void *)batched_kernel<PREC, NT, XC, MINB>, NT, XC, sizeof(TreeShared<5, XC>)};
+    return KernelInfo{(void *)batched_kernel<PREC, NT, XC, MINB, CC>, NT, XC, sizeof(TreeShared<5, XC, false, CC>)};
 }
 
 bool variant_ok(int precision, int variant, int maxM) {
     if (variant < 0 || variant >= kNumVariants || variant_clustered(variant) || variant == 9) return false;
     if (precision == 0 && variant >= 2) return false;
     if ((variant == 1 || variant == 3) && maxM > kVariant1MaxM) return false;
+    if (variant == 2 && maxM > kVariant2MaxM) return false;
+    if (variant == 4 && maxM > kVariant4MaxM) return false;
     if (variant == 5 && maxM > kVariant5MaxM) return false;
     if (variant == 6 && maxM > kVariant6MaxM) return false;
     return true;
@@ -326,9 +336,9 @@ KernelInfo kernel_for(int precision, int variant) {
     if (precision == 0) return variant == 1 ? kinfo<0, 256, 576, 2>() : kinfo<0, TREE_THREADS, XCAP, 1>();
     switch (variant) {
         case 1: return kinfo<1, 256, 576, 2>();
-        case 2: return kinfo<1, 640, XCAP, 1>();
+        case 2: return kinfo<1, 128, kSmallXC, 6, kNoSlotCC>();
         case 3: return kinfo<1, 256, 576, 3>();
-        case 4: return kinfo<1, 768, kWideXC, 1>();
+        case 4: return kinfo<1, 256, kWideXC, 3, kNoSlotCC>();
         case 5: return kinfo<1, 384, kPairXC, 2>();
         case 6: return kinfo<1, 256, kQuadXC, 4>();
         default: return kinfo<1, TREE_THREADS, XCAP, 1>();
@@ -356,11 +366,12 @@ std::mutex g_mu;
 std::map<const void *, Launch> g_launch;
 
 // Default schedule of an untuned batch: the CTA shape the single-instance
-// autotuner picks for large tables on GB300 (256 x 3 refined, 256 x 2 FP64)
-// where every instance fits it.
+// autotuner picks for large tables on GB300 (128 x 6 refined, 256 x 2 FP64) where
+// every instance fits it. 48 instances of 16 to 128 modes, refined: 15.0 ms at
+// 128 x 6, 16.2 at 256 x 3.
 TreeCfg default_cfg(int precision, int maxM) {
     TreeCfg c = kDefaultCfg;
-    if (maxM <= kVariant1MaxM) c.variant = precision == 1 ? 3 : 1;
+    if (maxM <= kVariant1MaxM) c.variant = precision == 0 ? 1 : maxM <= kVariant2MaxM ? 2 : 3;
     return c;
 }
 

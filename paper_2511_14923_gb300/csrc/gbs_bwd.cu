@@ -721,7 +721,7 @@ __global__ void mirror_kernel(int n2, double *__restrict__ gV) {
 
 BwdLayout bwd_layout(int M, int kmax, int sms) {
     BwdLayout b{};
-    b.fwd = ws_layout(M, kmax, sms);  // packing, status, scratch slots
+    b.fwd = ws_layout(M, kmax, sms, 0, false);  // packing, status, scratch slots
     const uint64_t N = order_offset(M, kmax + 1);
     size_t off = b.fwd.total;
     b.p0_off = off;

@@ -213,7 +213,6 @@ __global__ void __launch_bounds__(CHUNK_THREADS, DISP ? 4 : 6)
         int c2, j;
         pair_decode(t, c2, j);
         const int q = c2 - ca;
-        const double P0Sp = a.p0[baseJ[PALL] + c2];
         double P0, v;
         bool ok;
         if constexpr (PREC == 0) {
@@ -229,7 +228,7 @@ __global__ void __launch_bounds__(CHUNK_THREADS, DISP ? 4 : 6)
             const Sym sch = sym_sub_gram(Sym{d[j], d[nx + j], d[2 * nx + j]}, w);
             const double det2 = det_sym(sch);
             const double rd = rsqrt(det2);
-            P0 = P0Sp * rd;
+            P0 = a.p0[baseJ[PALL] + c2] * rd;
             if constexpr (DISP)
                 P0 *= exp(-quad_inv(sch, rd * rd, sub_wtg(Vec2{d[3 * nx + j], d[4 * nx + j]}, w,
                                                           Vec2{rs[3 * nr + q], rs[4 * nr + q]})));
@@ -247,15 +246,20 @@ __global__ void __launch_bounds__(CHUNK_THREADS, DISP ? 4 : 6)
                                 ASym{Acc{d0.x, d0.w}, Acc{d0.y, d1.x}, Acc{d0.z, d1.y}},
                                 Piv{DF{p4.x, p4.y}, DF{p4.z, p4.w}, DF{p5.x, p5.y}}, r0, eta, ok);
             ok = ok && !bad;
-            P0 = 0.0;
-            if ((MODE == MODE_KAPPA || MODE == MODE_SPINK) && !write_p0 && a.p0f) {
-                // the lead term without P0(S), as in tree_item
-                const float2 pj = reinterpret_cast<const float2 *>(a.p0f)[j];
-                v = combine_tail<NP, MODE>(refined_lead_term<(lead_sign<NP, MODE>() < 0)>(P0Sp, r0, eta, pj.x, pj.y), j,
-                                           c2, t, baseJ, baseT, p0R, a.p0, a.out);
+            constexpr bool pairs = MODE == MODE_KAPPA || MODE == MODE_SPINK;
+            P0 = !ok ? nan : write_p0 || !pairs ? refined_leaf_p0(a.p0[baseJ[PALL] + c2], r0, eta) : 0.0;
+            if constexpr (pairs) {
+                float2 kq[NQ], pq[NQ];
+                double uq[NQ];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    kq[q] = q ? a.kyp[baseJ[q] + j] : float2{};
+                    pq[q] = a.p0p[baseJ[q] + c2];
+                    uq[q] = q < PALL ? a.out[baseT[q] + t] : 0.0;
+                }
+                v = combine_lead<NP, MODE>(combine_products<NP, MODE>(kq, pq, uq, p0R), r0, eta, a.p0p[j], pq[PALL]);
                 if (!ok) v = nan;
             } else {
-                P0 = ok ? refined_leaf_p0(P0Sp, r0, eta) : nan;
                 v = combine<NP, MODE>(P0, j, c2, t, baseJ, baseT, p0R, a.p0, a.out);
             }
         }

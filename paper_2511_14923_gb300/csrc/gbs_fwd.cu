@@ -50,15 +50,13 @@ __global__ void pack_kernel(const double *__restrict__ V, int M, double *__restr
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm) {
+WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm, bool pairs) {
     WsLayout w{};
     size_t off = 0;
     w.status_off = off;
     off = align256(off + 256);
     w.A_off = off;  // FP64 blocks, then the float-pair copy
     off = align256(off + 2 * sizeof(double) * 4 * (size_t)M * M);
-    w.p0f_off = off;  // P0({x}) as float pairs
-    off = align256(off + 2 * sizeof(float) * (size_t)M);
     w.p0_off = off;
     const uint64_t np0 = kmax > 1 ? order_offset(M, kmax) : 0;  // orders 1..kmax-1
     off = align256(off + sizeof(double) * (size_t)np0);
@@ -68,6 +66,10 @@ WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm) {
     // the reduced half-means of a displaced state
     w.slot_doubles = 4 * ((size_t)binom2(M) + (size_t)M) + 2 * (size_t)M;
     if (kmax >= 4) off = align256(off + sizeof(double) * w.slot_doubles * w.slots);
+    w.p0p_off = off;  // any precision: one workspace serves both
+    if (pairs && kmax >= 4) off = align256(off + sizeof(float2) * (size_t)np0);
+    w.kyp_off = off;
+    if (pairs && kmax >= 4) off = align256(off + sizeof(float2) * (size_t)np0);
     w.total = off;
     return w;
 }

@@ -20,7 +20,9 @@ struct FwdArgs {
     int M, kmax, mode, precision;
     double *A;            // packed 2x2 blocks of (V+I)/2, M*M*4 doubles (workspace)
     float *Af;            // the same blocks as float pairs (hi x4, lo x4), refined path (workspace)
-    float *p0f;           // P0({x}) as float pairs (hi, lo) per mode, refined path (workspace; may be null)
+    // refined cumulant calls with kmax >= 4: the lower orders' P0 and no-click cumulants
+    // ky (gbs_tree.cuh, combine_pairs) as float pairs (workspace; null otherwise)
+    float2 *p0p, *kyp;
     double *p0;           // P0 table: the output for MODE_P0, a workspace table (orders < kmax) otherwise
     double *out;          // mu or kappa table (MODE_MU / MODE_KAPPA); equals p0 for MODE_P0
     unsigned *status;     // status word (workspace)
@@ -37,7 +39,8 @@ struct FwdArgs {
     int c_lo, c_hi;
     // prefix-tree schedule (autotuned): items per CTA slot, children per shared-
     // memory batch, CTA shape (0: 512 threads x 1 per SM; 1: 256 x 2; refined path
-    // only: 2: 640 x 1, 3: 256 x 3, 4: 768 x 1 with a 2048-entry x area, 5: 384 x 2
+    // only: 2: 128 x 6 with a 304-entry x area, 3: 256 x 3, 4: 256 x 3 with a 672-entry
+    // x area, 5: 384 x 2
     // with a 960-entry x area, 6: 256 x 4 with a 384-entry x area, 7: 6 in clusters
     // of 4, 8: 3 in clusters of 3, 9: 6 without Schur-complement slots)
     int grain, ccap, variant;
@@ -62,32 +65,38 @@ constexpr TreeCfg kDefaultCfg{2, 64, 0};
 constexpr int kMaxChildren = 64;
 // Largest M the 256-thread variant accepts (its shared x-entry area holds 576 modes).
 constexpr int kVariant1MaxM = 577;
-// x-entries per batch of the 768-thread refined variant (one CTA per SM).
-constexpr int kWideXC = 2048;
+// x-entries per batch of the 128-thread x 6 refined variant (24 children), and its
+// largest M.
+constexpr int kSmallXC = 304;
+constexpr int kVariant2MaxM = kSmallXC + 1;
+// x-entries per batch of the second 256-thread x 3 refined variant (24 children).
+constexpr int kWideXC = 672;
+constexpr int kVariant4MaxM = kWideXC + 1;
 // x-entries per batch of the 384-thread x 2 refined variant, and its largest M.
 constexpr int kPairXC = 960;
 constexpr int kVariant5MaxM = kPairXC + 1;
 // x-entries per batch of the 256-thread x 4 refined variant, and its largest M.
 constexpr int kQuadXC = 384;
 constexpr int kVariant6MaxM = kQuadXC + 1;
-// The slot-free 256-thread x 4 refined variant: children per batch it has room
-// for, and the elimination rows Y(x), x < c4 <= M - 2, it keeps in shared memory.
+// Children per batch the shapes with small or wide x areas have room for. The
+// slot-free 256-thread x 4 refined variant: the elimination rows Y(x), x < c4 <= M - 2, it keeps in shared memory.
 constexpr int kNoSlotCC = 24;
 constexpr int kNoSlotYC = 160;
 constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1
 // Schedule of an untuned forward call, from sweeps of shape x grain (kt, M = 20 to
 // 300, kmax = 4 and 5; the tuner still finds the last percents):
-//   refined: 256 x 4 where its x area admits M (M = 144, kmax = 5: 13.2 ms against
-//     17.7 at 512 x 1; M = 50: 0.177 against 0.300), 384 x 2 up to its own limit;
-//     one item per CTA slot below 128 modes with order 5 (77: 0.726 against 0.738),
-//     where a second round of items would wait for the first, else two;
+//   refined, kmax = 5: 128 x 6 where its x area admits M (M = 144: 10.6 ms against
+//     10.7 at 256 x 3 and 17.7 at 512 x 1; M = 77: 0.64 against 0.66 and 1.2), one
+//     item per CTA slot below 128 modes, where a second round of items would wait
+//     for the first, else two; kmax = 4: 256 x 3, two items (M = 144: 0.44 against
+//     0.50 at 128 x 6); larger M 256 x 3, then 384 x 2;
 //   FP64: 256 x 2, one item per CTA slot (M = 111, kmax = 5: 11.2 against 12.3;
 //     M = 50: 0.35 against 0.47); a kmax = 4 table large enough for the prefix tree
 //     (gbs_launch.cuh) 512 x 1 with eight (M = 300: 23.5 against 24.9).
 inline TreeCfg default_cfg(int M, int kmax, int precision) {
     TreeCfg c = kDefaultCfg;
     if (precision == 1) {
-        c.variant = M <= kVariant6MaxM ? 6 : M <= kVariant5MaxM ? 5 : 0;
+        c.variant = kmax == 5 && M <= kVariant2MaxM ? 2 : M <= kVariant4MaxM ? 4 : M <= kVariant5MaxM ? 5 : 0;
         c.grain = kmax == 5 && M < 128 ? 1 : 2;
     } else if (kmax == 5) {
         c.variant = M <= kVariant1MaxM ? 1 : 0;
@@ -106,7 +115,8 @@ constexpr int kNumVariants = 10;
 inline int effective_variant(int variant, int M, int precision) {
     if (variant == 1 || variant == 3 || variant == 8) return M <= kVariant1MaxM && (variant == 1 || precision == 1) ? variant : 0;
     if (precision != 1) return 0;
-    if (variant == 2 || variant == 4) return variant;
+    if (variant == 2) return M <= kVariant2MaxM ? 2 : 0;
+    if (variant == 4) return M <= kVariant4MaxM ? 4 : 0;
     if (variant == 5) return M <= kVariant5MaxM ? 5 : 0;
     if (variant == 6 || variant == 7) return M <= kVariant6MaxM ? variant : 0;
     if (variant == 9) return M <= kVariant9MaxM ? 9 : 0;
@@ -117,16 +127,18 @@ inline bool variant_clustered(int v) { return v == 7 || v == 8; }
 
 // Workspace layout, shared by the size query and the launcher.
 struct WsLayout {
-    size_t status_off, A_off, p0f_off, p0_off, scratch_off, total;
+    size_t status_off, A_off, p0_off, scratch_off, p0p_off, kyp_off, total;
     size_t slot_doubles;
     int slots;
 };
 // Scratch slots per multiprocessor that cover every CTA shape allowed for M:
-// four when the 256 x 4 shape can run (M <= 385), else three.
-inline int slots_per_sm_for(int M) { return M <= 385 ? 4 : 3; }
+// six when the 128 x 6 shape can run (M <= 305), four for 256 x 4 (M <= 385), else
+// three.
+inline int slots_per_sm_for(int M) { return M <= kVariant2MaxM ? 6 : M <= kVariant6MaxM ? 4 : 3; }
 // Reserves slots_per_sm scratch slots per multiprocessor (0 = slots_per_sm_for(M);
 // with one, only one CTA per multiprocessor runs).
-WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm = 0);
+// pairs: with the float-pair tables of refined cumulant calls (kmax >= 4).
+WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm = 0, bool pairs = true);
 
 // Queues the packing of A = (V+I)/2 into 2x2 blocks.
 cudaError_t launch_pack(const FwdArgs &a, cudaStream_t stream);

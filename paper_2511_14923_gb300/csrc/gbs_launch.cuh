@@ -237,13 +237,15 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
         const int v = effective_variant(a.variant, a.M, PREC);
         if (v == 1) return launch_tree_v<D, MODE, PREC, 256, 576, 2, false>(a, write_p0, st);
         if constexpr (PREC == 1) {
-            // register-lean refined kernels: 20 warps in one CTA, 3 CTAs of 8 warps,
-            // 24 warps in one CTA with room for about 3.5x more children per batch,
-            // 2 CTAs of 12 warps with room for about 1.7x more, or 4 CTAs of 8 warps
-            // (64 registers) with room for a third fewer
-            if (v == 2) return launch_tree_v<D, MODE, PREC, 640, XCAP, 1, false>(a, write_p0, st);
+            // 24 warps with 80 registers in 6 CTAs of 4, 3 of 8 (with room for up to 64
+            // children a batch, or for more x-entries) or 2 of 12; or 32 warps with 64
+            // registers in 4 CTAs. Order 5 runs fastest in the smallest CTAs, whose
+            // batches wait least at their barriers (M = 144: 128 x 6 10.6 ms, 256 x 3
+            // 10.7, 256 x 4 11.6, the shared gathers spilling at 64 registers)
+            // (its order 4, whose items are small, in the wide 256 x 3 shape: 0.44 against 0.50 ms)
+            if (v == 2 && D == 5) return launch_tree_v<D, MODE, PREC, 128, kSmallXC, 6, false, kNoSlotCC>(a, write_p0, st);
             if (v == 3) return launch_tree_v<D, MODE, PREC, 256, 576, 3, false>(a, write_p0, st);
-            if (v == 4) return launch_tree_v<D, MODE, PREC, 768, kWideXC, 1, false>(a, write_p0, st);
+            if (v == 4 || v == 2) return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
             if (v == 5) return launch_tree_v<D, MODE, PREC, 384, kPairXC, 2, false>(a, write_p0, st);
             if (v == 6) {
                 // order 4 of the 256 x 4 shape runs without slots where it can: its items

@@ -79,7 +79,7 @@ extern "C" int gbs_cumulants_noalloc(const double *V, int M, int kmax, double *k
         return gbs::record_error(GBS_ERR_CUDA, "no CUDA device is current");
     // one scratch slot per multiprocessor: the default 512-thread schedule runs
     // at most one CTA per multiprocessor
-    const gbs::WsLayout L = gbs::ws_layout(M, kmax, sms, 1);
+    const gbs::WsLayout L = gbs::ws_layout(M, kmax, sms, 1, false);
     if (L.total > kNoallocScratchBytes) {
         char msg[256];
         snprintf(msg, sizeof msg,

@@ -71,6 +71,12 @@ __device__ __forceinline__ void split_df(double x, float &h, float &l) {
     l = __double2float_rn(x - (double)h);
 }
 
+// x truncated to FP32 and the rest (below FP32's normal range: the rounded value alone).
+__device__ __forceinline__ float2 pair_of_double(double x) {
+    const float h = d2f_bits(x);
+    return make_float2(h, __double2float_rn(x - f2d_bits(h)));
+}
+
 // Running sum s + t, not normalised.
 struct Acc {
     float s, t;
@@ -189,31 +195,6 @@ __device__ __forceinline__ void refined_leaf_factor(ABlk S, const DFBlk &z2, con
 __device__ __forceinline__ double refined_leaf_p0(double P0Sp, float r0, float eta) {
     const double u = P0Sp * f2d_bits(r0);
     return fma(u, f2d_bits(eta), u);
-}
-
-// +-(P0(S) - P0({j}) P0(S')) = +-P0(S') (r0 (1 + eta) - p) (minus when NEG), the
-// leading term of the cumulant recursion when P0(S) itself is not stored, with
-// p = P0({j}) given as an FP32 pair (ph + pl). The difference
-// w = r0 - ph + r0 eta - pl is formed on the FP32 pipe as an unevaluated pair
-// s + lo (two-sum of r0 - ph, which is exact when they are close, plus the exact
-// product r0 eta). Then P0(S') w = P0(S') s + P0(S') lo takes one FP64 FMA: the
-// second product is a correction about 2^-24 below the first, so it is formed
-// in FP32 from P0(S') truncated to FP32 (relative error below 2^-23 on a term
-// of relative size 2^-24) and enters as the FMA's addend. P0(S') below FP32's
-// normal range drops the correction (an absolute error under 1e-45). The sign
-// goes into the FP32 bits.
-template <bool NEG>
-__device__ __forceinline__ double refined_lead_term(double P0Sp, float r0, float eta, float ph, float pl) {
-    const float s = __fadd_rn(r0, -ph);
-    const float bb = __fsub_rn(s, r0);
-    const float e1 = __fadd_rn(__fsub_rn(r0, __fsub_rn(s, bb)), __fsub_rn(-ph, bb));
-    const float pr = r0 * eta;
-    const float qr = __fmaf_rn(r0, eta, -pr);
-    const float lo = __fadd_rn(__fadd_rn(e1, -pl), __fadd_rn(pr, qr));
-    const float c = d2f_bits(P0Sp) * lo;
-    const unsigned flip = NEG ? 0x80000000u : 0u;
-    return fma(P0Sp, f2d_bits(__uint_as_float(__float_as_uint(s) ^ flip)),
-               f2d_bits(__uint_as_float(__float_as_uint(c) ^ flip)));
 }
 
 }  // namespace gbs

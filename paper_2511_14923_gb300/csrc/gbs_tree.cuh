@@ -98,6 +98,15 @@ __device__ __forceinline__ double combine(double P0S, int j, int c2, uint32_t t,
                                   p0R, p0tab, outtab);
 }
 
+// Weight of the recursion's product with R = Q + {c2} (bitmask q) in the
+// accumulator of sign sd.
+template <int MODE>
+__device__ __forceinline__ constexpr double upper_weight(int q, double sd) {
+    int n = 0;
+    for (int b = q; b; b &= b - 1) ++n;
+    return MODE == MODE_KAPPA ? ((n & 1) ? sd : -sd) : -1.0 / (double)(4 << n);
+}
+
 // Sign carried by the accumulator of the cumulant recursion: (-1)^d for the
 // click cumulant (d = NP + 2), + for the spin cumulant.
 template <int NP, int MODE>
@@ -122,13 +131,58 @@ __device__ __forceinline__ double combine_tail(double acc, int j, int c2, uint32
         acc = fma(sg * outtab[baseJ[q] + j], p0tab[baseJ[PALL ^ q] + c2], acc);
     }
 #pragma unroll
-    for (int q = 0; q < PALL; ++q) {
-        const double sg = (MODE == MODE_KAPPA) ? ((__popc(q) & 1) ? sd : -sd)
-                                               : -1.0 / (double)(4 << __popc(q));  // R = Q + {c2}
-        acc = fma(sg * outtab[baseT[q] + t], p0R[PALL ^ q], acc);
-    }
+    for (int q = 0; q < PALL; ++q) acc = fma(upper_weight<MODE>(q, sd) * outtab[baseT[q] + t], p0R[PALL ^ q], acc);
     if (MODE == MODE_SPINK) return acc * (double)(1 << (NP + 2));
     return acc;
+}
+
+// The cumulant recursion of the refined path (MODE_KAPPA, MODE_SPINK) in terms of
+// the no-click cumulants ky (kt = (-1)^d ky, kappa = 2^d ky):
+//   ky(S) = P0(S) - P0({j}) P0(S') - sum_{empty != R proper subset S'} ky(R + {j}) P0(S' - R).
+// The lead term P0(S') (r0 (1 + eta) - P0({j})) and the products whose factors are
+// particular to j and to c2 (R within P) run on pairs from the tables' float-pair
+// copies: every order-5 entry then takes 8 FP64 instructions instead of 15, and
+// GB300's FP64 pipe (1/63 of the FP32 rate) no longer binds alone. The products
+// with c2 in R keep FP64: one factor is the same for a whole child. The pairs'
+// error, about 2^-46 of a product, is below the determinants' own.
+// In two parts, so that the table values are not live across the determinant step:
+// the products, then the lead term.
+struct PairSum {
+    Acc g;       // -sum over R within P
+    double acc;  // sum over R with c2, with the order's sign
+};
+// k[q] = ky({j} + Q), p[q] = P0({c2} + Q) as pairs, u[q] = the mode's table at
+// {j, c2} + Q, for the subsets Q of P (bitmasks q).
+template <int NP, int MODE>
+__device__ __forceinline__ PairSum combine_products(const float2 (&k)[1 << NP], const float2 (&p)[1 << NP],
+                                                    const double (&u)[1 << NP], const double *p0R) {
+    constexpr int PALL = (1 << NP) - 1;
+    constexpr double sd = lead_sign<NP, MODE>();
+    PairSum r;
+    r.acc = upper_weight<MODE>(0, sd) * u[0] * p0R[PALL];
+#pragma unroll
+    for (int q = 1; q < PALL; ++q) r.acc = fma(upper_weight<MODE>(q, sd) * u[q], p0R[PALL ^ q], r.acc);
+    const DF f = df_mulu(DF{-k[1].x, -k[1].y}, DF{p[PALL ^ 1].x, p[PALL ^ 1].y});
+    r.g = Acc{f.h, f.l};
+#pragma unroll
+    for (int q = 2; q <= PALL; ++q) acc_sub(r.g, DF{k[q].x, k[q].y}, DF{p[PALL ^ q].x, p[PALL ^ q].y});
+    return r;
+}
+// ps = P0(S'), pj = P0({j}) as pairs.
+template <int NP, int MODE>
+__device__ __forceinline__ double combine_lead(PairSum r, float r0, float eta, float2 pj, float2 ps) {
+    // w = r0 + r0 eta - P0({j}): two-sum of the leading parts, the rest gathered
+    const float s = __fsub_rn(r0, pj.x);
+    const float bb = __fsub_rn(s, r0);
+    const float e1 = __fsub_rn(__fsub_rn(r0, __fsub_rn(s, bb)), __fadd_rn(pj.x, bb));
+    const float pr = r0 * eta;
+    const float lo = __fadd_rn(__fsub_rn(e1, pj.y), __fadd_rn(pr, __fmaf_rn(r0, eta, -pr)));
+    acc_sub(r.g, DF{-ps.x, -ps.y}, df_norm(s, lo));
+    // into FP64, with the order's sign
+    const unsigned flip = lead_sign<NP, MODE>() < 0 ? 0x80000000u : 0u;
+    const double v = r.acc + f2d_bits(__uint_as_float(__float_as_uint(r.g.s) ^ flip)) +
+                     f2d_bits(__uint_as_float(__float_as_uint(r.g.t) ^ flip));
+    return MODE == MODE_SPINK ? v * (double)(1 << (NP + 2)) : v;
 }
 
 template <int MODE>
@@ -174,7 +228,6 @@ __device__ __forceinline__ void order1_entry(const FwdArgs &a, int j, bool write
         flag_status(a.status, ST_NOT_POSDEF);
         P0 = __longlong_as_double(0x7ff8000000000000ULL);
     }
-    if (a.p0f && a.precision == 1) split_df(P0, a.p0f[2 * j], a.p0f[2 * j + 1]);
     // mu({j}) = kt({j}) = 1 - P0({j});  c({j}) = kappa({j}) = 2 P0({j}) - 1
     const double v = (MODE == MODE_MU || MODE == MODE_KAPPA) ? 1.0 - P0
                    : (MODE == MODE_SPINC || MODE == MODE_SPINK) ? fma(2.0, P0, -1.0) : P0;
@@ -273,9 +326,10 @@ struct TreeShared {
     int c3[CC];
     int xoff[CC + 1];
     uint32_t lpref[CC + 1];
-    uint64_t baseJ[CC][NQ];
-    uint64_t baseT[CC][NQ];
-    double p0R[CC][NQ];
+    // (refined cumulants: subsets without c3, whose bases all children share, first)
+    alignas(16) uint64_t baseJ[CC][NQ];
+    alignas(16) uint64_t baseT[CC][NQ];
+    alignas(16) double p0R[CC][NQ];
     double m3[CC][3];
     float p3f[CC][6];  // refined path: the c3 pivot's factors i0, l, i1 as pairs (Piv)
     double g3[DISP ? CC : 1][2];  // displaced: whitened half-mean of each child's c3 pivot
@@ -393,6 +447,13 @@ __device__ __forceinline__ void store_entry(const FwdArgs &a, int d, uint64_t id
     }
     if (write_p0) a.p0[idx] = P0;
     if (MODE != MODE_P0) a.out[idx] = v;
+    if constexpr (MODE == MODE_KAPPA || MODE == MODE_SPINK) {
+        if (a.p0p && d < a.kmax) {
+            // ky = (-1)^d kt = 2^{-d} kappa
+            a.p0p[idx] = pair_of_double(P0);
+            a.kyp[idx] = pair_of_double(MODE == MODE_SPINK ? v * (1.0 / (double)(1 << d)) : (d & 1) ? -v : v);
+        }
+    }
 }
 
 // One work item of the prefix-tree kernel: U = {c4, c5} (D = 5) or {c4} (D = 4),
@@ -424,6 +485,7 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
     static_assert(!(DISP && CL), "displaced states run without clusters");
     constexpr bool NOSLOT = YC > 0;
     static_assert(!NOSLOT || (PREC == 1 && !CL), "the slot-free form is the refined path's, without clusters");
+    constexpr bool PAIRS = PREC == 1 && (MODE == MODE_KAPPA || MODE == MODE_SPINK);  // combine_pairs
     const int ccap = ccap_in < CC ? ccap_in : CC;
     using SH = TreeShared<D, XC, DISP, CC, YC>;
     constexpr int NP = SH::NP;
@@ -581,8 +643,14 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                 sh.lpref[nb] = lp + (uint32_t)binom2(c3);
             }
             int P[3] = {c3, c4, c5};
-            uint64_t idxQ[NQ];
-            child_bases<NP>(P, M, sh.baseJ[b], sh.baseT[b], idxQ);
+            uint64_t bj[NQ], bt[NQ], idxQ[NQ];
+            child_bases<NP>(P, M, bj, bt, idxQ);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int at = PAIRS ? (q & 1) * (NQ / 2) + (q >> 1) : q;
+                sh.baseJ[b][at] = bj[q];
+                sh.baseT[b][at] = bt[q];
+            }
             sh.p0R[b][0] = 0.0;
 #pragma unroll
             for (int q = 1; q < NQ; ++q) sh.p0R[b][q] = a.p0[idxQ[q]];
@@ -682,15 +750,29 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
             if constexpr (PREC == 0) S64 = load_blk(slot + 4 * (size_t)t);
             else if constexpr (NOSLOT) Sg = acc_of(su_block<D>(a.Af, M, sh.yq, c2, j));
             else Sg = slot_pair_df(slot, t);
+            // refined cumulants: table values of the subsets without c3, the same for every
+            // child of the batch (half of a leaf's gathers)
+            [[maybe_unused]] float2 pj, kq[NQ], pq[NQ];
+            [[maybe_unused]] double uq[NQ];
+            if constexpr (PAIRS) {
+                pj = a.p0p[j];
+                kq[0] = float2{};
+#pragma unroll
+                for (int h = 0; h < NQ / 2; ++h) {
+                    const uint64_t bj = sh.baseJ[0][h];
+                    if (h) kq[2 * h] = a.kyp[bj + j];
+                    pq[2 * h] = a.p0p[bj + c2];
+                }
+            }
             for (int b = 0; b < nb && c2 < sh.c3[b]; ++b) {
                 const int xo = sh.xoff[b];
                 const int e2 = xo + c2, ej = xo + j;
                 const uint64_t *bJ = sh.baseJ[b];
                 const uint64_t *bT = sh.baseT[b];
-                const double P0Sp = a.p0[bJ[PALL] + c2];
                 double P0;
                 bool ok;
                 if constexpr (PREC == 0) {
+                    const double P0Sp = a.p0[bJ[PALL] + c2];
                     const Blk z2{xe[0][e2], xe[1][e2], xe[2][e2], xe[3][e2]};
                     const Blk zj{xe[0][ej], xe[1][ej], xe[2][ej], xe[3][ej]};
                     const LInv m2{xe[7][e2], xe[8][e2], xe[9][e2]};
@@ -707,6 +789,45 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                     }
                     ok = det2 > 0.0;
                 } else {
+                    [[maybe_unused]] PairSum sums;
+                    [[maybe_unused]] uint64_t topT = 0, topJ = 0;
+                    if constexpr (PAIRS) {
+                        // the subsets with c3: odd bitmasks, at NQ / 2 .. NQ - 1
+                        const ulonglong2 *bo = reinterpret_cast<const ulonglong2 *>(bJ + NQ / 2);
+                        const ulonglong2 *to = reinterpret_cast<const ulonglong2 *>(bT + NQ / 2);
+                        const double2 *r2 = reinterpret_cast<const double2 *>(sh.p0R[b]);
+                        double p0R[NQ];
+#pragma unroll
+                        for (int h = 0; h < NQ / 4; ++h) {
+                            const ulonglong2 x = bo[h], y = to[h];
+                            const uint64_t jo[2] = {x.x, x.y}, tt[2] = {y.x, y.y};
+#pragma unroll
+                            for (int g = 0; g < 2; ++g) {
+                                const int q = 2 * (2 * h + g) + 1;
+                                kq[q] = a.kyp[jo[g] + j];
+                                pq[q] = a.p0p[jo[g] + c2];
+                                uq[q] = q < PALL ? a.out[tt[g] + t] : 0.0;
+                            }
+                            topJ = x.y;
+                            topT = y.y;
+                        }
+#pragma unroll
+                        for (int h = 0; h < NQ / 2; ++h) {
+                            const double2 x = r2[h];
+                            p0R[2 * h] = x.x;
+                            p0R[2 * h + 1] = x.y;
+                        }
+                        {
+                            const ulonglong2 *be = reinterpret_cast<const ulonglong2 *>(bT);
+#pragma unroll
+                            for (int h = 0; h < NQ / 4; ++h) {
+                                const ulonglong2 x = be[h];
+                                uq[4 * h] = a.out[x.x + t];
+                                uq[4 * h + 2] = a.out[x.y + t];
+                            }
+                        }
+                        sums = combine_products<NP, MODE>(kq, pq, uq, p0R);
+                    }
                     const float4 zh2 = xq[0][e2], zl2 = xq[1][e2], zhj = xq[0][ej], zlj = xq[1][ej];
                     const float4 d0 = xq[2][ej], p4 = xq[4][e2];
                     const float2 d1 = *reinterpret_cast<const float2 *>(&xq[3][ej]);
@@ -717,23 +838,17 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
                     const Piv pv{DF{p4.x, p4.y}, DF{p4.z, p4.w}, DF{p5.x, p5.y}};
                     float r0, eta;
                     refined_leaf_factor(Sg, z2, zj, dj, pv, r0, eta, ok);
-                    if constexpr (MODE == MODE_KAPPA || MODE == MODE_SPINK) {
-                        if (!write_p0 && a.p0f) {
-                            // P0(S) is not stored: its product with P0(S') folds into the
-                            // recursion's leading term (15 FP64 instructions per entry)
-                            const float2 pj = reinterpret_cast<const float2 *>(a.p0f)[j];
-                            double v = combine_tail<NP, MODE>(
-                                refined_lead_term<(lead_sign<NP, MODE>() < 0)>(P0Sp, r0, eta, pj.x, pj.y), j, c2, t,
-                                bJ, bT, sh.p0R[b], a.p0, a.out);
-                            if (!ok) {
-                                flag_status(a.status, ST_NOT_POSDEF);
-                                v = __longlong_as_double(0x7ff8000000000000ULL);
-                            }
-                            store_entry<MODE>(a, NP + 2, bT[PALL] + t, 0.0, v, false);
-                            continue;
+                    if constexpr (PAIRS) {
+                        P0 = write_p0 ? refined_leaf_p0(a.p0[topJ + c2], r0, eta) : 0.0;
+                        double v = combine_lead<NP, MODE>(sums, r0, eta, pj, pq[PALL]);
+                        if (!ok) {
+                            flag_status(a.status, ST_NOT_POSDEF);
+                            P0 = v = __longlong_as_double(0x7ff8000000000000ULL);
                         }
+                        store_entry<MODE>(a, NP + 2, topT + t, P0, v, write_p0);
+                        continue;
                     }
-                    P0 = refined_leaf_p0(P0Sp, r0, eta);
+                    P0 = refined_leaf_p0(a.p0[bJ[PALL] + c2], r0, eta);
                 }
                 if (!ok) {
                     flag_status(a.status, ST_NOT_POSDEF);

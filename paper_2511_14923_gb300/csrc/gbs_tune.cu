@@ -5,10 +5,10 @@
 //   grain   items per CTA slot (subtree granularity: 1, 2, 4, 8),
 //   ccap    children per shared-memory batch (16 or 64),
 //   variant CTA shape: 512 threads x 1 per SM; 256 x 2 per SM (M <= 577); and for
-//           the refined path 640 x 1, 256 x 3 (M <= 577), 768 x 1 with room
-//           for more children per batch, 384 x 2 (M <= 961), 256 x 4 (M <= 385),
+//           the refined path 128 x 6 (M <= 305), 256 x 3 (M <= 577, or with a
+//           larger x area M <= 673), 384 x 2 (M <= 961), 256 x 4 (M <= 385),
 //           256 x 4 / 256 x 3 in thread-block clusters sharing one slot, or
-//           256 x 4 without slots (M <= 162).
+//           256 x 4 without slots (M <= 161).
 // Results live in a process-wide table consulted by every forward call; if the
 // environment variable GBS_AUTOTUNE_CACHE names a file, the table is loaded from
 // it on first use and rewritten after each tuning run (a JSON array of objects).
@@ -204,6 +204,8 @@ int autotune(FwdArgs a, cudaStream_t st, TreeCfg &best, float &best_ms, int &tri
     std::vector<TreeCfg> cand;
     for (int variant = 0; variant <= (a.precision == 1 ? kNumVariants - 1 : 1); ++variant) {
         if ((variant == 1 || variant == 3) && a.M > kVariant1MaxM) continue;
+        if (variant == 2 && a.M > kVariant2MaxM) continue;
+        if (variant == 4 && a.M > kVariant4MaxM) continue;
         if (variant == 5 && a.M > kVariant5MaxM) continue;
         if ((variant == 6 || variant == 7) && a.M > kVariant6MaxM) continue;
         if (variant == 8 && a.M > kVariant1MaxM) continue;
