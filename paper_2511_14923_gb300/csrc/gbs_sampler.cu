@@ -99,7 +99,7 @@ struct Args {
     Tabs o;
     R *W;
     const R *kb;           // kappa(i, n) regrouped for p2_block_kernel, or null (p2_kernel then walks every row itself)
-    float *At;             // tensor-core product: the step's rows, split and tiled (atc_kernel)
+    float *At;             // tensor-core product: the step's rows, split and tiled (operands_kernel)
     const R *hs;           // per-variable half scale s_v / 2, hs[v], v = 1..M
     const R *lead;         // per-variable pairs (kappa'({v}), hs[v]) at lead[2v], lead[2v+1]
     const double *H;       // per-variable log scale ln s_v (the click entropy of mode v - 1)
@@ -392,11 +392,11 @@ static void launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms,
 // 5th-generation tensor cores: tcgen05.mma kind::tf32 with the 3-term split
 // x = hi + lo (hi, lo TF32), Z = Ahi Bhi + Ahi Blo + Alo Bhi accumulated in FP32
 // in tensor memory (the dropped Alo Blo term is ~2^-22 relative). A CTA of 128
-// threads owns 128 rows x 256 samples. W arrives from wtc_kernel already split
+// threads owns 128 rows x 256 samples. W arrives from operands_kernel already split
 // and laid out as the MMA's K-major core matrices (8 rows x 16 bytes, no
 // swizzle), one contiguous block per TC_KC-wide K chunk and sample tile, and
 // is brought in by one TMA bulk copy per chunk; the rows (cumulant segments)
-// arrive the same way from atc_kernel. One elected thread issues the MMAs. A
+// arrive the same way from operands_kernel. One elected thread issues the MMAs. A
 // ring of TC_NS stages, each with a "full" mbarrier (the bulk copies' bytes) and
 // an "empty" one (the MMAs' commit), keeps TC_NS - 1 chunks loading while the
 // MMAs of one run; the ring takes 96 KB of shared memory, so two CTAs share a
@@ -407,13 +407,14 @@ constexpr int TC_M = 128, TC_N = 256, TC_KC = 8;
 constexpr int TC_ACH = TC_M * TC_KC;            // floats of one A copy (hi or lo) of one chunk
 constexpr int TC_BCH = TC_N * TC_KC;            // floats of one B copy of one chunk
 constexpr int TC_AB = TC_M * TC_KC * 4;         // bytes of one A copy per stage (4 KB)
-constexpr int TC_BB = TC_N * TC_KC * 4;         // bytes of one B copy per stage (8 KB)
-constexpr int TC_STAGE = 2 * TC_AB + 2 * TC_BB;  // A hi, A lo, B hi, B lo
-constexpr int TC_NS = 4, TC_NS_DEEP = 8;         // stages of the ring (see launch_ztc)
-constexpr int tc_smem(int ns) { return ns * TC_STAGE + 256; }  // stages, then 2 x ns mbarriers, TMEM slot, flag
-// instruction descriptor: D f32, A and B tf32, both K-major, N = 256, M = 128
-constexpr uint32_t TC_IDESC = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(TC_N >> 3) << 17) |
-                              ((uint32_t)(TC_M >> 4) << 24);
+constexpr int TC_NS = 4, TC_NS_DEEP = 8;         // stages of the ring, of TN samples (see launch_ztc)
+constexpr int TC_NARROW = 64;
+constexpr int tc_stage(int tn) { return 2 * TC_AB + 2 * tn * TC_KC * 4; }  // A hi, A lo, B hi, B lo
+constexpr int tc_smem(int ns, int tn) { return ns * tc_stage(tn) + 256; }  // then 2 x 8 mbarriers, TMEM slot, flag
+// instruction descriptor: D f32, A and B tf32, both K-major, N = n, M = 128
+constexpr uint32_t tc_idesc(int n) {
+    return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -470,10 +471,11 @@ __device__ __forceinline__ void tma_bulk(void *dst, const void *src, uint32_t by
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
+template <int TN>
 __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint32_t acc) {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(d),
-        "l"(a), "l"(b), "r"(TC_IDESC), "r"(acc)
+        "l"(a), "l"(b), "r"(tc_idesc(TN)), "r"(acc)
         : "memory");
 }
 
@@ -500,10 +502,11 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&v)[32]) {
 // float offset ((c nsb + sb) 2 + part) 256 KC + tc_off(s % 256, r % KC) / 4,
 // c = r / KC, sb = s / 256, nsb = S / 256. A thread forms four consecutive r (one 16-byte
 // row of a core matrix) of one sample, so 8 consecutive samples write one
-// 128-byte line. Grid: (samples / ETB, quads of r).
+// 128-byte line. Block (bx, by) of (samples / PREP, ny): quads by, by + ny, ...
+constexpr int PREP = 128;  // threads of the operand kernels
 template <int K>
-__global__ void __launch_bounds__(ETB) wtc_kernel(Args<float> a, int t, int D) {
-    const int s = blockIdx.x * ETB + threadIdx.x;
+__device__ __forceinline__ void w_operand(const Args<float> &a, int t, int D, int bx, int by, int ny) {
+    const int s = bx * PREP + threadIdx.x;
     const int Dp = (D + TC_KC - 1) / TC_KC * TC_KC;
     const int nsb = a.S / TC_N, sb = s / TC_N, sl = s % TC_N;
     Spins<float> sp(a, s), sd(a, s);
@@ -512,7 +515,7 @@ __global__ void __launch_bounds__(ETB) wtc_kernel(Args<float> a, int t, int D) {
     const Grp<float> tb(a, s);
     const uint64_t rowlen = K == 3 ? 0 : cb(t - 2, 2);
     const float *q2 = tb.P2 + (K != 3 && t >= 4 ? cb(t - 2, 3) : 0) * SG;
-    for (int qd = blockIdx.y; qd < Dp / 4; qd += gridDim.y) {
+    for (int qd = by; qd < Dp / 4; qd += ny) {
         const int r0 = 4 * qd;
         float v[4];
         int e = 0, d = 0;
@@ -556,11 +559,11 @@ __global__ void __launch_bounds__(ETB) wtc_kernel(Args<float> a, int t, int D) {
 // The rows of the step product (cumulant segments) split into TF32 hi / lo and
 // laid out like W: row tile rt (128 rows), chunk c (TC_KC inner entries) at
 // float offset (rt nk + c) 2 128 TC_KC, hi then lo, each in the core-matrix layout.
-// Rows beyond `rows` and entries beyond D are zero. Grid: (row tiles, chunks),
-// 128 threads, thread i = row i of the tile.
+// Rows beyond `rows` and entries beyond D are zero. Thread i = row i of tile rt.
 template <int K>
-__global__ void __launch_bounds__(128) atc_kernel(Args<float> a, int t, uint64_t rows, int D) {
-    const int tid = threadIdx.x, rt = blockIdx.x, c = blockIdx.y, nk = gridDim.y;
+__device__ __forceinline__ void a_operand(const Args<float> &a, int t, uint64_t rows, int D, int rt, int c, int nk) {
+    static_assert(PREP == TC_M, "one thread per row of a tile");
+    const int tid = threadIdx.x;
     const uint64_t q = (uint64_t)rt * TC_M + tid;
     uint64_t kb = 0, dst = 0;
     if (q < rows) zrow(K, a.M, t, q, a.off, a.o, kb, dst);
@@ -583,23 +586,38 @@ __global__ void __launch_bounds__(128) atc_kernel(Args<float> a, int t, uint64_t
     }
 }
 
+// Both operands of step t's product in one launch: nw blocks of W (S / PREP per
+// row of blocks), then row tiles x chunks of the rows.
+template <int K>
+__global__ void __launch_bounds__(PREP) operands_kernel(Args<float> a, int t, uint64_t rows, int D, unsigned nw,
+                                                        unsigned nrt, unsigned nk) {
+    const unsigned nx = (unsigned)(a.S / PREP);
+    if (blockIdx.x < nw) {
+        w_operand<K>(a, t, D, (int)(blockIdx.x % nx), (int)(blockIdx.x / nx), (int)(nw / nx));
+    } else {
+        const unsigned q = blockIdx.x - nw;
+        a_operand<K>(a, t, rows, D, (int)(q % nrt), (int)(q / nrt), (int)nk);
+    }
+}
+
 // Z rows of one 128-row tile x 256 samples. Thread 0 streams both operands by
 // TMA bulk copies (A: 128 rows, W: 256 samples, hi and lo, per TC_KC-wide
 // chunk) into a ring of TC_NS stages and issues the MMAs; chunk c-1+TC_NS is
 // loaded into the stage of chunk c-1 once the MMAs of chunk c-1 have completed,
 // while those of chunk c run. All threads then read
 // the accumulator (thread i = row i) and write the rows out.
-template <int K, int NS>
+template <int K, int NS, int TN>
 __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<float> a, int t, uint64_t rows, int D) {
     extern __shared__ __align__(1024) unsigned char smem[];
-    static_assert(NS <= 8, "barrier area");
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + NS * TC_STAGE);
+    constexpr int STAGE = tc_stage(TN), BB = TN * TC_KC * 4;
+    static_assert(NS <= 8 && NS * STAGE >= 4 * 32 * 36 * 4, "barrier area, epilogue tiles");
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + NS * STAGE);
     uint64_t *empty = full + 8;
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + NS * TC_STAGE + 128);
-    int *flag = reinterpret_cast<int *>(smem + NS * TC_STAGE + 192);
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(smem + NS * STAGE + 128);
+    int *flag = reinterpret_cast<int *>(smem + NS * STAGE + 192);
     const int tid = threadIdx.x, warp = tid >> 5;
     const uint64_t m0 = (uint64_t)blockIdx.x * TC_M;
-    const int rt = blockIdx.x, sb = blockIdx.y, s0 = sb * TC_N, nsb = a.S / TC_N;
+    const int rt = blockIdx.x, s0 = (int)blockIdx.y * TN, sb = s0 / TC_N, nsb = a.S / TC_N;
     const int nk = (D + TC_KC - 1) / TC_KC;
     if (tid == 0) {
         for (int i = 0; i < NS; ++i) {
@@ -611,7 +629,7 @@ __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<floa
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tslot)),
-                     "r"(TC_N)
+                     "r"(TN)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -622,13 +640,20 @@ __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<floa
     if (tid == 0) {
         const uint32_t sbase = smem_u32(smem);
         const float *Ab = a.At + (size_t)rt * nk * 2 * TC_ACH;
-        const float *Wb = a.W + (size_t)sb * 2 * TC_BCH;
+        // TN samples of W's 256-sample tile: a contiguous part of its hi and of its lo copy
+        const float *Wb = a.W + (size_t)sb * 2 * TC_BCH + s0 % TC_N * TC_KC;
         auto load = [&](int c) {
             const int st = c % NS;
-            unsigned char *sp = smem + st * TC_STAGE;
-            mbar_expect(&full[st], 2 * TC_AB + 2 * TC_BB);
+            unsigned char *sp = smem + st * STAGE;
+            mbar_expect(&full[st], 2 * TC_AB + 2 * BB);
             tma_bulk(sp, Ab + (size_t)c * 2 * TC_ACH, 2 * TC_AB, &full[st]);
-            tma_bulk(sp + 2 * TC_AB, Wb + (size_t)c * nsb * 2 * TC_BCH, 2 * TC_BB, &full[st]);
+            const float *wc = Wb + (size_t)c * nsb * 2 * TC_BCH;
+            if constexpr (TN == TC_N) {
+                tma_bulk(sp + 2 * TC_AB, wc, 2 * BB, &full[st]);
+            } else {
+                tma_bulk(sp + 2 * TC_AB, wc, BB, &full[st]);
+                tma_bulk(sp + 2 * TC_AB + BB, wc + TC_BCH, BB, &full[st]);
+            }
         };
         // chunk c uses stage c % NS and completes phase (c / NS) & 1 of its
         // barriers; nl chunks loaded, nf of them waited for (full), nc committed,
@@ -649,15 +674,15 @@ __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<floa
             if (!ok) break;
             ++nf;
             tc_fence_after();
-            const uint32_t sbs = sbase + st * TC_STAGE;
+            const uint32_t sbs = sbase + st * STAGE;
 #pragma unroll
             for (int j = 0; j < TC_KC / 8; ++j) {
                 const uint32_t o = j * 256;  // two core matrices per 8-wide slice of K
                 const uint64_t ahi = tc_desc(sbs + o), alo = tc_desc(sbs + TC_AB + o);
-                const uint64_t bhi = tc_desc(sbs + 2 * TC_AB + o), blo = tc_desc(sbs + 2 * TC_AB + TC_BB + o);
-                tc_mma(tmem, ahi, bhi, (c > 0 || j > 0) ? 1u : 0u);
-                tc_mma(tmem, ahi, blo, 1u);
-                tc_mma(tmem, alo, bhi, 1u);
+                const uint64_t bhi = tc_desc(sbs + 2 * TC_AB + o), blo = tc_desc(sbs + 2 * TC_AB + BB + o);
+                tc_mma<TN>(tmem, ahi, bhi, (c > 0 || j > 0) ? 1u : 0u);
+                tc_mma<TN>(tmem, ahi, blo, 1u);
+                tc_mma<TN>(tmem, alo, bhi, 1u);
             }
             tc_commit(&empty[st]);
             ++nc;
@@ -712,7 +737,7 @@ __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<floa
         }
         const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
 #pragma unroll 1
-        for (int cc = 0; cc < TC_N / 32; ++cc) {
+        for (int cc = 0; cc < TN / 32; ++cc) {
             const int sc = s0 + cc * 32;
             const size_t col = (size_t)(sc / SG) * a.gs + sc % SG + c4;  // group block and sample within it
             uint32_t v[32];
@@ -733,24 +758,29 @@ __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<floa
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_N) : "memory");
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TN) : "memory");
 }
 
 // Two CTAs with four stages share a multiprocessor, one's epilogue overlapping the
-// other's MMAs. A launch that leaves at most one CTA for each multiprocessor is
-// bound by its chain of chunks, each waiting for its copies: eight stages (192 KB)
-// keep seven of them in flight. K = 3, M = 1152, 256 samples (9 CTAs of up to 144
-// chunks a step): 33 -> 20 us a step.
+// other's MMAs. A launch that leaves few CTAs is bound by each one's chain of
+// chunks: at one CTA or less per multiprocessor eight stages keep seven chunks'
+// copies in flight; at half of that 64-sample tiles split the MMAs of a chunk over
+// four times the CTAs (the same accumulations, so the same bits). K = 3, M = 1152,
+// 256 samples (9 wide tiles of up to 144 chunks a step): 33 us a step with wide
+// tiles, 26 with narrow ones.
 template <int K>
 static cudaError_t launch_ztc(const Args<float> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
-    const dim3 grid((unsigned)((rows + TC_M - 1) / TC_M), (unsigned)(a.S / TC_N));
-    const bool deep = (uint64_t)grid.x * grid.y <= (uint64_t)sms;
-    const int smem = tc_smem(deep ? TC_NS_DEEP : TC_NS);
-    auto fn = deep ? ztc_kernel<K, TC_NS_DEEP> : ztc_kernel<K, TC_NS>;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    fn<<<grid, 128, smem, st>>>(a, t, rows, D);
-    return cudaSuccess;
+    const unsigned nrt = (unsigned)((rows + TC_M - 1) / TC_M);
+    const uint64_t wide = (uint64_t)nrt * (unsigned)(a.S / TC_N);
+    auto go = [&](auto fn, int ns, int tn) {
+        const int smem = tc_smem(ns, tn);
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess) fn<<<dim3(nrt, (unsigned)(a.S / tn)), 128, smem, st>>>(a, t, rows, D);
+        return e;
+    };
+    if (2 * wide <= (uint64_t)sms) return go(ztc_kernel<K, TC_NS_DEEP, TC_NARROW>, TC_NS_DEEP, TC_NARROW);
+    if (wide <= (uint64_t)sms) return go(ztc_kernel<K, TC_NS_DEEP, TC_N>, TC_NS_DEEP, TC_N);
+    return go(ztc_kernel<K, TC_NS, TC_N>, TC_NS, TC_N);
 }
 
 // ---------------------------------------------------------------- table rows of one step
@@ -1052,7 +1082,7 @@ __device__ __forceinline__ void p2_row_terms(const Grp<R> &t, int e, int d, cons
 constexpr int P2_NB = 8;
 
 template <class R, int VW>
-__global__ void __launch_bounds__(32, 20) p2_block_kernel(Args<R> a, int n0, unsigned npairs) {
+__global__ void __launch_bounds__(32, 16) p2_block_kernel(Args<R> a, int n0, unsigned npairs) {
     const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)threadIdx.x * VW);
     const unsigned r = blockIdx.x;
     int hi, lo;
@@ -1566,9 +1596,6 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
         if (D > 0) {
             bool tc = false;
             if constexpr (sizeof(R) == 4) tc = a.use_tc != 0;
-            if constexpr (sizeof(R) == 4) {
-                if (tc) wtc_kernel<K><<<egrid(S, (uint64_t)((D + TC_KC - 1) / TC_KC * TC_KC / 4)), ETB, 0, st>>>(a, t, D);
-            }
             if (!tc) w_kernel<R, K><<<egrid(S, (uint64_t)D), ETB, 0, st>>>(a, t, D);
             const uint64_t rows = K == 3   ? 1 + (uint64_t)(M - t)
                                   : K == 4 ? 1 + 2 * (uint64_t)(M - t)
@@ -1576,7 +1603,10 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
             if constexpr (sizeof(R) == 4) {
                 if (tc) {
                     const unsigned nrt = (unsigned)((rows + TC_M - 1) / TC_M), nk = (unsigned)((D + TC_KC - 1) / TC_KC);
-                    atc_kernel<K><<<dim3(nrt, nk), 128, 0, st>>>(a, t, rows, D);
+                    // W: about 5000 blocks, each taking its share of the quads
+                    const unsigned nx = (unsigned)(S / PREP), quads = (unsigned)((D + TC_KC - 1) / TC_KC * TC_KC / 4);
+                    const unsigned cap = 5000 / nx < 16 ? 16 : 5000 / nx, nw = nx * (quads < cap ? quads : cap);
+                    operands_kernel<K><<<nw + nrt * nk, PREP, 0, st>>>(a, t, rows, D, nw, nrt, nk);
                     if ((e = launch_ztc<K>(a, t, rows, D, sms, st)) != cudaSuccess) return e;
                 } else {
                     launch_zgemm<R, K>(a, t, rows, D, sms, st);
