@@ -843,39 +843,45 @@ __device__ __forceinline__ double qdiag(const double *r, int M, int k) {
 
 // V = D (S Q S^T) D + I - D^2 with D = diag(sqrt(eta)) (eta repeated for the
 // x and p blocks), Q = diag(e^{-2r}, e^{2r}): a 2M x 2M symmetric product, tiled
-// 32 x 32. Each block computes one tile on or below the diagonal (256 threads,
-// four rows each) and writes it and its mirror; the k dimension advances 32 at
-// a time through shared memory, with the 32 entries of Q of that step computed
-// once per block.
-constexpr int COV_TILE = 32;
+// T x T. Each block computes one tile on or below the diagonal (256 threads, T^2 /
+// 256 rows each) and writes it and its mirror; the k dimension advances 32 at a
+// time through shared memory. The FP64 pipe binds (2 FMAs per clock and
+// multiprocessor), so a matrix that 32-wide tiles would put on a fraction of the
+// multiprocessors takes 16-wide ones: M = 100 leaves 28 wide tiles (87 us) or 91
+// narrow ones (25 us). One chain of FMAs per element either way.
+constexpr int COV_K = 32;
 
+template <int T>
 __global__ void __launch_bounds__(256) covariance_kernel(const double *Ur, const double *Ui, const double *r,
                                                          const double *eta, int M, double *V) {
-    __shared__ double As[COV_TILE][COV_TILE + 1], Bs[COV_TILE][COV_TILE + 1];
+    __shared__ double As[T][COV_K + 1], Bs[T][COV_K + 1];
+    constexpr int RT = 256 / T, NR = T / RT;  // threads per column of the tile, rows per thread
     const int n2 = 2 * M;
     // block -> tile (ta, tb) with tb <= ta
     int ta = (int)((sqrt(8.0 * blockIdx.x + 1.0) - 1.0) * 0.5);
     while ((ta + 1) * (ta + 2) / 2 <= (int)blockIdx.x) ++ta;
     while (ta * (ta + 1) / 2 > (int)blockIdx.x) --ta;
     const int tb = (int)blockIdx.x - ta * (ta + 1) / 2;
-    const int a0 = ta * COV_TILE, b0 = tb * COV_TILE;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    double acc[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int k0 = 0; k0 < n2; k0 += COV_TILE) {
-        const int k = k0 + tx;
+    const int a0 = ta * T, b0 = tb * T;
+    const int lx = threadIdx.x & 31, ly = threadIdx.x >> 5;  // loads: k and row
+    const int tx = threadIdx.x % T, ty = threadIdx.x / T;    // results: column and first row
+    double acc[NR];
+#pragma unroll
+    for (int u = 0; u < NR; ++u) acc[u] = 0.0;
+    for (int k0 = 0; k0 < n2; k0 += COV_K) {
+        const int k = k0 + lx;
         const double q = k < n2 ? qdiag(r, M, k) : 0.0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int row = ty + 8 * u;
-            As[row][tx] = (a0 + row < n2 && k < n2) ? smat(Ur, Ui, M, a0 + row, k) * q : 0.0;
-            Bs[row][tx] = (b0 + row < n2 && k < n2) ? smat(Ur, Ui, M, b0 + row, k) : 0.0;
+        for (int row = ly; row < T; row += 8) {
+            As[row][lx] = (a0 + row < n2 && k < n2) ? smat(Ur, Ui, M, a0 + row, k) * q : 0.0;
+            Bs[row][lx] = (b0 + row < n2 && k < n2) ? smat(Ur, Ui, M, b0 + row, k) : 0.0;
         }
         __syncthreads();
 #pragma unroll 8
-        for (int kk = 0; kk < COV_TILE; ++kk) {
+        for (int kk = 0; kk < COV_K; ++kk) {
             const double bv = Bs[tx][kk];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) acc[u] = fma(As[ty + 8 * u][kk], bv, acc[u]);
+            for (int u = 0; u < NR; ++u) acc[u] = fma(As[ty + RT * u][kk], bv, acc[u]);
         }
         __syncthreads();
     }
@@ -883,8 +889,8 @@ __global__ void __launch_bounds__(256) covariance_kernel(const double *Ur, const
     if (b >= n2) return;
     const double db = sqrt(eta[b < M ? b : b - M]);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int a = a0 + ty + 8 * u;
+    for (int u = 0; u < NR; ++u) {
+        const int a = a0 + ty + RT * u;
         if (a >= n2 || b > a) continue;
         const double da = sqrt(eta[a < M ? a : a - M]);
         double v = da * acc[u] * db;
@@ -955,8 +961,13 @@ __global__ void covariance_bwd_kernel(const double *Ur, const double *Ui, const 
 
 cudaError_t launch_covariance(const double *Ur, const double *Ui, const double *r, const double *eta, int M, double *V,
                               cudaStream_t st) {
-    const int nt = (2 * M + COV_TILE - 1) / COV_TILE;
-    covariance_kernel<<<nt * (nt + 1) / 2, 256, 0, st>>>(Ur, Ui, r, eta, M, V);
+    auto tiles = [&](int t) {
+        const int nt = (2 * M + t - 1) / t;
+        return nt * (nt + 1) / 2;
+    };
+    // four wide tiles for each of 152 multiprocessors: the last wave then costs little
+    if (tiles(32) >= 4 * 152) covariance_kernel<32><<<tiles(32), 256, 0, st>>>(Ur, Ui, r, eta, M, V);
+    else covariance_kernel<16><<<tiles(16), 256, 0, st>>>(Ur, Ui, r, eta, M, V);
     return cudaGetLastError();
 }
 
