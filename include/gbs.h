@@ -134,8 +134,9 @@ int gbs_spin_cumulants(const double *V, int M, int kmax, double *kappa_out, int 
 /* Per-order kernel timing. While enabled (on != 0), every forward call records
    CUDA events on its stream before and after the kernels of each order.
    gbs_timing_read() waits for the events of the most recent call and writes
-   durations in milliseconds: ms_out[0] = packing (V -> 2x2 blocks), ms_out[d] =
-   the kernels of order d (d = 1..GBS_MAX_ORDER; 0 for orders above kmax).
+   durations in milliseconds: ms_out[0] = packing (V -> 2x2 blocks) and orders 1 and
+   2, which share its launch (ms_out[1] and ms_out[2] are then about 0), ms_out[d] =
+   the kernels of order d (d = 3..GBS_MAX_ORDER; 0 for orders above kmax).
    Events are created on first use; timing state is process-wide and not meant
    for concurrent calls from several host threads. Returns GBS_OK or GBS_ERR_CUDA. */
 int gbs_timing(int on);

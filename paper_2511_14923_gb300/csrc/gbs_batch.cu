@@ -8,9 +8,9 @@
 // slot (grain) and children per shared-memory batch. The schedule comes from the
 // batch autotuner's table when this batch shape has been tuned
 // (gbs_batched_autotune), else from a default. gbs_cumulants_batched() then
-// queues a single kernel that runs six phases separated by grid-wide barriers:
-//   0 packing of every instance's (V + I)/2 into 2x2 blocks,
-//   1-3 orders 1..3, one work unit per subset (grid-stride over all instances),
+// queues a single kernel whose phases are separated by grid-wide barriers:
+//   0-2 packing of every instance's (V + I)/2 into 2x2 blocks and orders 1 and 2,
+//   3 order 3, one work unit per block or subset (grid-stride over all instances),
 //   4-5 orders 4 and 5, prefix-tree items of all instances pulled from one
 //       atomic queue per order (largest instances first).
 // The launch reads everything from the workspace, so it can be captured in a
@@ -272,27 +272,25 @@ __global__ void __launch_bounds__(NT, MINB) batched_kernel(char *ws) {
     const uint64_t nthr = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t gtid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
 
-    // phase 0: packing
+    // phases 0-2: packing and orders 1 and 2, which read V alone
     for (uint64_t u = gtid; u < h.total[0]; u += nthr) {
         const int i = find_inst(pref, n, u);
         pack_entry(inst[i].V, inst[i].M, inst[i].A,
                    PREC == 1 ? reinterpret_cast<float *>(inst[i].A + 4 * (size_t)inst[i].M * inst[i].M) : nullptr,
                    (int)(u - pref[i]));
     }
-    grid.sync();
-    // phases 1-3: orders 1..3
     for (uint64_t u = gtid; u < h.total[1]; u += nthr) {
         const int i = find_inst(pref + (n + 1), n, u);
         const FwdArgs a = inst_args(inst[i], status, nullptr, 0, PREC);
         order1_entry<MODE_KAPPA>(a, (int)(u - pref[(n + 1) + i]), 1 < a.kmax);
     }
-    grid.sync();
     for (uint64_t u = gtid; u < h.total[2]; u += nthr) {
         const int i = find_inst(pref + 2 * (n + 1), n, u);
         const FwdArgs a = inst_args(inst[i], status, nullptr, 0, PREC);
         order2_entry<MODE_KAPPA>(a, (uint32_t)(u - pref[2 * (n + 1) + i]), 2 < a.kmax);
     }
     grid.sync();
+    // phase 3: order 3
     for (uint64_t u = gtid; u < h.total[3]; u += nthr) {
         const int i = find_inst(pref + 3 * (n + 1), n, u);
         const FwdArgs a = inst_args(inst[i], status, nullptr, 0, PREC);

@@ -22,10 +22,6 @@ cudaError_t launch_forward_displaced(const FwdArgs &a_in, cudaStream_t st) {
     a.variant = kDefaultCfg.variant;
     a.grain = kDefaultCfg.grain;
     a.ccap = kDefaultCfg.ccap;
-    if (a.ev) cudaEventRecord(a.ev[0], st);
-    cudaError_t e = launch_pack(a, st);
-    if (e != cudaSuccess) return e;
-    if (a.ev) cudaEventRecord(a.ev[1], st);
     return launch_orders<true>(a, st);
 }
 

@@ -26,8 +26,9 @@
 //   that holds j: 2^{d-1} - 1 products per entry instead of one per partition.
 //
 // Kernels
-//   pack_kernel     A = (V+I)/2 as M x M packed 2x2 blocks (xxpp rows k, k+M).
-//   order1/2/3      one thread per subset; the elimination is redone per thread.
+//   front_kernel    A = (V+I)/2 as M x M packed 2x2 blocks (xxpp rows k, k+M), and
+//                   orders 1 and 2, one thread per block or subset.
+//   chunk_kernel    order 3, and order 4 of small and medium tables (gbs_chunk.cuh).
 //   tree_kernel<D>  D = 4, 5: persistent CTAs walk the colex prefix tree. A CTA
 //                   owns U = {c_4, .., c_D} and stores the Schur complement of
 //                   A after eliminating U (modes below c_4) in its scratch slot.
@@ -40,11 +41,6 @@
 #include "gbs_launch.cuh"
 
 namespace gbs {
-
-__global__ void pack_kernel(const double *__restrict__ V, int M, double *__restrict__ A, float *__restrict__ Af) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < M * M) pack_entry(V, M, A, Af, idx);
-}
 
 // ---------------------------------------------------------------- host side
 
@@ -74,19 +70,6 @@ WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm, bool pairs) {
     return w;
 }
 
-cudaError_t launch_pack(const FwdArgs &a, cudaStream_t st) {
-    const int M = a.M;
-    pack_kernel<<<(M * M + FLAT_THREADS - 1) / FLAT_THREADS, FLAT_THREADS, 0, st>>>(
-        a.V, M, a.A, a.precision == 1 ? a.Af : nullptr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_forward(const FwdArgs &a, cudaStream_t st) {
-    if (a.ev) cudaEventRecord(a.ev[0], st);
-    cudaError_t e = launch_pack(a, st);
-    if (e != cudaSuccess) return e;
-    if (a.ev) cudaEventRecord(a.ev[1], st);
-    return launch_orders<false>(a, st);
-}
+cudaError_t launch_forward(const FwdArgs &a, cudaStream_t st) { return launch_orders<false>(a, st); }
 
 }  // namespace gbs

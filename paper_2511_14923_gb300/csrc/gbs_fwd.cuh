@@ -140,8 +140,6 @@ inline int slots_per_sm_for(int M) { return M <= kVariant2MaxM ? 6 : M <= kVaria
 // pairs: with the float-pair tables of refined cumulant calls (kmax >= 4).
 WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm = 0, bool pairs = true);
 
-// Queues the packing of A = (V+I)/2 into 2x2 blocks.
-cudaError_t launch_pack(const FwdArgs &a, cudaStream_t stream);
 // Queues every kernel of one forward call on stream; returns a cudaError_t.
 cudaError_t launch_forward(const FwdArgs &a, cudaStream_t stream);
 // The same for a displaced state (a.mean set, a.precision = 0).

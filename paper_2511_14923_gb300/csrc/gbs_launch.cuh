@@ -15,20 +15,30 @@ constexpr uint32_t kOrder4Pairs = 16384;
 // Shared memory a chunk may take: 227 KB less the kernel's static part.
 constexpr size_t kChunkSmem = 226 * 1024;
 
-// Flat kernels of orders 1-3: one thread per subset of colex rank first + i,
-// i < count (the whole order, or the rank range of a range call's top order).
+// Packing of A, order 1 and order 2 in one launch (none reads what another writes):
+// blocks [0, nb0) pack, [nb0, nb0 + nb1) fill order 1, the rest order 2; one thread
+// per block of A or subset of colex rank first + i, i < count (the whole order, or
+// the rank range of a range call's top order). Three dependent launches of 3-6 us
+// each before; one of about 7 now (call totals below).
+struct Span {
+    uint64_t first, count;
+};
 template <int MODE, bool DISP>
-__global__ void order1_kernel(FwdArgs a, bool write_p0, uint64_t first, uint64_t count) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) order1_entry<MODE, DISP>(a, (int)(first + i), write_p0);
+__global__ void __launch_bounds__(FLAT_THREADS) front_kernel(FwdArgs a, bool wp1, bool wp2, Span s1, Span s2,
+                                                             unsigned nb0, unsigned nb1) {
+    if (blockIdx.x < nb0) {
+        const uint64_t i = (uint64_t)blockIdx.x * FLAT_THREADS + threadIdx.x;
+        if (i < (uint64_t)a.M * a.M) pack_entry(a.V, a.M, a.A, a.precision == 1 ? a.Af : nullptr, (int)i);
+    } else if (blockIdx.x < nb0 + nb1) {
+        const uint64_t i = (uint64_t)(blockIdx.x - nb0) * FLAT_THREADS + threadIdx.x;
+        if (i < s1.count) order1_entry<MODE, DISP>(a, (int)(s1.first + i), wp1);
+    } else {
+        const uint64_t i = (uint64_t)(blockIdx.x - nb0 - nb1) * FLAT_THREADS + threadIdx.x;
+        if (i < s2.count) order2_entry<MODE, DISP>(a, (uint32_t)(s2.first + i), wp2);
+    }
 }
 
-template <int MODE, bool DISP>
-__global__ void order2_kernel(FwdArgs a, bool write_p0, uint64_t first, uint64_t count) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) order2_entry<MODE, DISP>(a, (uint32_t)(first + i), write_p0);
-}
-
+// Flat kernel of order 3: one thread per subset of colex rank first + i, i < count.
 template <int MODE, bool DISP>
 __global__ void order3_kernel(FwdArgs a, bool write_p0, uint64_t first, uint64_t count) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -326,16 +336,15 @@ static cudaError_t launch_mode(const FwdArgs &a, cudaStream_t st) {
     };
     auto grid = [](uint64_t n) { return (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS); };
     cudaError_t e = cudaSuccess;
-    uint64_t f = 0, n = 0;
-    span(1, f, n);
-    if (n) order1_kernel<MODE, DISP><<<grid(n), FLAT_THREADS, 0, st>>>(a, wp(1), f, n);
+    Span s1{0, 0}, s2{0, 0};
+    span(1, s1.first, s1.count);
+    if (a.kmax >= 2) span(2, s2.first, s2.count);
+    const unsigned nb0 = grid((uint64_t)M * M), nb1 = grid(s1.count);
+    mark(0);
+    front_kernel<MODE, DISP><<<nb0 + nb1 + grid(s2.count), FLAT_THREADS, 0, st>>>(a, wp(1), wp(2), s1, s2, nb0, nb1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    mark(1);
     mark(2);
-    if (a.kmax >= 2) {
-        span(2, f, n);
-        if (n) order2_kernel<MODE, DISP><<<grid(n), FLAT_THREADS, 0, st>>>(a, wp(2), f, n);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
     mark(3);
     if (a.kmax >= 3) {
         const bool part = a.top && a.kmax == 3;
@@ -359,7 +368,7 @@ static cudaError_t launch_mode(const FwdArgs &a, cudaStream_t st) {
     return cudaSuccess;
 }
 
-// Queues the per-order kernels (orders 1..kmax) of one forward call after packing.
+// Queues every kernel of one forward call.
 template <bool DISP>
 cudaError_t launch_orders(const FwdArgs &a, cudaStream_t st) {
     switch (a.mode) {

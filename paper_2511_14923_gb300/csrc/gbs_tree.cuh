@@ -190,11 +190,8 @@ __device__ __forceinline__ void store_entry(const FwdArgs &a, int d, uint64_t id
 
 // ---------------------------------------------------------------- small kernels
 
-// Writes block idx = x*M + y of A = (V+I)/2 as 4 doubles, and (if Af is not
-// null) as 4 hi floats then 4 lo floats for the refined path.
-__device__ __forceinline__ void pack_entry(const double *__restrict__ V, int M, double *__restrict__ A,
-                                           float *__restrict__ Af, int idx) {
-    const int x = idx / M, y = idx - x * M;
+// Block (x, y) of A = (V+I)/2 from V.
+__device__ __forceinline__ Blk vblk(const double *__restrict__ V, int M, int x, int y) {
     const size_t n2 = 2 * (size_t)M;
     double a00 = V[x * n2 + y], a01 = V[x * n2 + y + M];
     double a10 = V[(x + M) * n2 + y], a11 = V[(x + M) * n2 + y + M];
@@ -202,7 +199,15 @@ __device__ __forceinline__ void pack_entry(const double *__restrict__ V, int M, 
         a00 += 1.0;
         a11 += 1.0;
     }
-    const Blk b{0.5 * a00, 0.5 * a01, 0.5 * a10, 0.5 * a11};
+    return Blk{0.5 * a00, 0.5 * a01, 0.5 * a10, 0.5 * a11};
+}
+
+// Writes block idx = x*M + y of A = (V+I)/2 as 4 doubles, and (if Af is not
+// null) as 4 hi floats then 4 lo floats for the refined path.
+__device__ __forceinline__ void pack_entry(const double *__restrict__ V, int M, double *__restrict__ A,
+                                           float *__restrict__ Af, int idx) {
+    const int x = idx / M, y = idx - x * M;
+    const Blk b = vblk(V, M, x, y);
     store_blk(A + 4 * (size_t)idx, b);
     if (Af) {
         float4 h, l;
@@ -217,21 +222,31 @@ __device__ __forceinline__ void pack_entry(const double *__restrict__ V, int M, 
 }
 
 
-template <int MODE, bool DISP = false>
-__device__ __forceinline__ void order1_entry(const FwdArgs &a, int j, bool write_p0) {
-    const Sym s = blk_sym(ablk(a.A, a.M, j, j));
+// P0 of one mode from its block of A; NaN (ok = false) unless positive definite.
+template <bool DISP>
+__device__ __forceinline__ double p0_single(const Blk &b, const double *mean, int M, int j, bool &ok) {
+    const Sym s = blk_sym(b);
     const double det = det_sym(s);
     const double rs = rsqrt(det);
     double P0 = rs;
-    if (DISP) P0 *= exp(-quad_inv(s, rs * rs, half_mean(a.mean, a.M, j)));
-    if (!(det > 0.0) || !(s.s00 > 0.0)) {
-        flag_status(a.status, ST_NOT_POSDEF);
-        P0 = __longlong_as_double(0x7ff8000000000000ULL);
-    }
-    // mu({j}) = kt({j}) = 1 - P0({j});  c({j}) = kappa({j}) = 2 P0({j}) - 1
-    const double v = (MODE == MODE_MU || MODE == MODE_KAPPA) ? 1.0 - P0
-                   : (MODE == MODE_SPINC || MODE == MODE_SPINK) ? fma(2.0, P0, -1.0) : P0;
-    store_entry<MODE>(a, 1, (uint64_t)j, P0, v, write_p0);
+    if (DISP) P0 *= exp(-quad_inv(s, rs * rs, half_mean(mean, M, j)));
+    ok = det > 0.0 && s.s00 > 0.0;
+    return ok ? P0 : __longlong_as_double(0x7ff8000000000000ULL);
+}
+// mu({j}) = kt({j}) = 1 - P0({j});  c({j}) = kappa({j}) = 2 P0({j}) - 1
+template <int MODE>
+__device__ __forceinline__ double single_value(double P0) {
+    return (MODE == MODE_MU || MODE == MODE_KAPPA) ? 1.0 - P0 : (MODE == MODE_SPINC || MODE == MODE_SPINK) ? fma(2.0, P0, -1.0) : P0;
+}
+
+// Orders 1 and 2 read V itself (order 2 forms its modes' own P0), so that they can
+// share a launch with the packing.
+template <int MODE, bool DISP = false>
+__device__ __forceinline__ void order1_entry(const FwdArgs &a, int j, bool write_p0) {
+    bool ok;
+    const double P0 = p0_single<DISP>(vblk(a.V, a.M, j, j), a.mean, a.M, j, ok);
+    if (!ok) flag_status(a.status, ST_NOT_POSDEF);
+    store_entry<MODE>(a, 1, (uint64_t)j, P0, single_value<MODE>(P0), write_p0);
 }
 
 
@@ -240,14 +255,16 @@ __device__ __forceinline__ void order2_entry(const FwdArgs &a, uint32_t t, bool 
     const int M = a.M;
     int c2, j;
     pair_decode(t, c2, j);
-    bool ok;
+    bool ok, ok2, okj;
     double detp;
-    const LInv m2 = chol2_inv(blk_sym(ablk(a.A, M, c2, c2)), ok, detp);
-    const Blk w = lmul(m2, ablk(a.A, M, c2, j));
-    const Sym sch = sym_sub_gram(blk_sym(ablk(a.A, M, j, j)), w);
+    const Blk b2 = vblk(a.V, M, c2, c2), bj = vblk(a.V, M, j, j);
+    const double p2 = p0_single<DISP>(b2, a.mean, M, c2, ok2), pj = p0_single<DISP>(bj, a.mean, M, j, okj);
+    const LInv m2 = chol2_inv(blk_sym(b2), ok, detp);
+    const Blk w = lmul(m2, vblk(a.V, M, c2, j));
+    const Sym sch = sym_sub_gram(blk_sym(bj), w);
     const double det2 = det_sym(sch);
     const double rs = rsqrt(det2);
-    double P0 = a.p0[c2] * rs;
+    double P0 = p2 * rs;
     if (DISP) {
         const Vec2 r = sub_wtg(half_mean(a.mean, M, j), w, lvec(m2, half_mean(a.mean, M, c2)));
         P0 *= exp(-quad_inv(sch, rs * rs, r));
@@ -258,11 +275,11 @@ __device__ __forceinline__ void order2_entry(const FwdArgs &a, uint32_t t, bool 
     }
     const uint64_t idx = (uint64_t)M + t;
     double v = P0;
-    if (MODE == MODE_MU) v = a.out[c2] - a.p0[j] + P0;
-    if (MODE == MODE_KAPPA) v = fma(-a.p0[j], a.p0[c2], P0);
+    if (MODE == MODE_MU) v = single_value<MODE>(p2) - pj + P0;
+    if (MODE == MODE_KAPPA) v = fma(-pj, p2, P0);
     // c({j,c2}) = -c({c2}) - 2 (P0({j}) - 2 P0(S));  kappa(S) = 4 (P0(S) - P0({j}) P0({c2}))
-    if (MODE == MODE_SPINC) v = fma(4.0, P0, fma(-2.0, a.p0[j], -a.out[c2]));
-    if (MODE == MODE_SPINK) v = 4.0 * fma(-a.p0[j], a.p0[c2], P0);
+    if (MODE == MODE_SPINC) v = fma(4.0, P0, fma(-2.0, pj, -single_value<MODE>(p2)));
+    if (MODE == MODE_SPINK) v = 4.0 * fma(-pj, p2, P0);
     store_entry<MODE>(a, 2, idx, P0, v, write_p0);
 }
 
