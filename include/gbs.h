@@ -288,8 +288,8 @@ int gbs_sample(const double *kappa, int M, int K, const int *orders, int n_sampl
 /* Times gbs_cumulants for this (M, kmax, precision) under each candidate
    schedule of the prefix-tree kernels -- items per CTA (1, 2, 4, 8), children
    per shared-memory batch (16, 64), CTA shape (512 threads x 1 per SM, 256 x 2
-   per SM when M <= 577; for GBS_FP32_REFINED also 128 x 6 when M <= 305, 256 x 3
-   when M <= 577 or, with a larger shared-memory batch area, M <= 673, 384 x 2 when
+   per SM when M <= 577, 256 x 3 with a larger shared-memory batch area when M <=
+   673; for GBS_FP32_REFINED also 128 x 6 when M <= 305, 256 x 3 when M <= 577, 384 x 2 when
    M <= 961, 256 x 4 when M <= 385, the 256 x 4 and 256 x 3 shapes in
    thread-block clusters whose CTAs share one Schur-complement slot, and 256 x 4
    without slots when M <= 161, forming each Schur-complement block from the
@@ -308,7 +308,7 @@ int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precis
 /* Schedule the forward calls of (M, kmax, precision) run on the current device:
    the one gbs_autotune recorded (or read from GBS_AUTOTUNE_CACHE), else the
    default. schedule_out[3] (host) = {CTA shape (0: 512 threads x 1 per SM,
-   1: 256 x 2, refined only 2: 128 x 6, 3: 256 x 3, 4: 3 with a larger batch area,
+   1: 256 x 2, 4: 256 x 3 with a larger batch area, refined only 2: 128 x 6, 3: 256 x 3,
    5: 384 x 2,
    6: 256 x 4, 7 and 8: 6 and 3 in thread-block clusters, 9: 6 without
    Schur-complement slots), items per CTA slot, children per shared-memory
@@ -338,7 +338,7 @@ size_t gbs_batched_workspace_bytes(const gbs_instance *inst, int n, int precisio
    (CTA shape, items per CTA, children per shared-memory batch). The schedule is
    the one gbs_batched_autotune recorded for a batch with the same multiset of
    (M, kmax) on this device (also read from GBS_AUTOTUNE_CACHE), else a default
-   (128 threads x 6 CTAs per SM for GBS_FP32_REFINED and 256 x 2 for GBS_FP64
+   (128 threads x 6 CTAs per SM for GBS_FP32_REFINED and 256 x 3 for GBS_FP64
    when every M <= 577; 512 x 1 otherwise). inst is a HOST array; the pointers
    in it are device pointers that must stay valid while the plan is used. Copies
    the plan with a host-to-device copy and synchronises cuda_stream: call it
@@ -362,8 +362,8 @@ int gbs_cumulants_batched(int precision, void *workspace, void *cuda_stream);
 /* Batch autotuner (the schedule search of gbs_autotune, for a ragged batch):
    times gbs_cumulants_batched on this batch under candidate schedules -- every
    CTA shape allowed for the precision and the largest M (512 x 1, 256 x 2 when
-   M <= 577; refined also 128 x 6 when M <= 305, 256 x 3 when M <= 577 or, with a
-   larger batch area, M <= 673, 384 x 2
+   M <= 577, 256 x 3 with a larger batch area when M <= 673; refined also 128 x 6
+   when M <= 305, 256 x 3 when M <= 577, 384 x 2
    when M <= 961, and 256 x 4 when M <= 385) at the default
    grain and batch size, then items per CTA slot (1, 2, 4, 8) x children per
    batch (16, 64) for the fastest shape -- records the fastest for this batch

@@ -321,7 +321,7 @@ KernelInfo kinfo() {
 
 bool variant_ok(int precision, int variant, int maxM) {
     if (variant < 0 || variant >= kNumVariants || variant_clustered(variant) || variant == 9) return false;
-    if (precision == 0 && variant >= 2) return false;
+    if (precision == 0 && variant >= 2 && variant != 4) return false;
     if ((variant == 1 || variant == 3) && maxM > kVariant1MaxM) return false;
     if (variant == 2 && maxM > kVariant2MaxM) return false;
     if (variant == 4 && maxM > kVariant4MaxM) return false;
@@ -331,7 +331,10 @@ bool variant_ok(int precision, int variant, int maxM) {
 }
 
 KernelInfo kernel_for(int precision, int variant) {
-    if (precision == 0) return variant == 1 ? kinfo<0, 256, 576, 2>() : kinfo<0, TREE_THREADS, XCAP, 1>();
+    if (precision == 0)
+        return variant == 1   ? kinfo<0, 256, 576, 2>()
+               : variant == 4 ? kinfo<0, 256, kWideXC, 3, kNoSlotCC>()
+                              : kinfo<0, TREE_THREADS, XCAP, 1>();
     switch (variant) {
         case 1: return kinfo<1, 256, 576, 2>();
         case 2: return kinfo<1, 128, kSmallXC, 6, kNoSlotCC>();
@@ -364,12 +367,12 @@ std::mutex g_mu;
 std::map<const void *, Launch> g_launch;
 
 // Default schedule of an untuned batch: the CTA shape the single-instance
-// autotuner picks for large tables on GB300 (128 x 6 refined, 256 x 2 FP64) where
+// autotuner picks for large tables on GB300 (128 x 6 refined, 256 x 3 FP64) where
 // every instance fits it. 48 instances of 16 to 128 modes, refined: 15.0 ms at
 // 128 x 6, 16.2 at 256 x 3.
 TreeCfg default_cfg(int precision, int maxM) {
     TreeCfg c = kDefaultCfg;
-    if (maxM <= kVariant1MaxM) c.variant = precision == 0 ? 1 : maxM <= kVariant2MaxM ? 2 : 3;
+    if (maxM <= kVariant1MaxM) c.variant = precision == 0 ? 4 : maxM <= kVariant2MaxM ? 2 : 3;
     return c;
 }
 

@@ -90,8 +90,8 @@ constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1
 //     item per CTA slot below 128 modes, where a second round of items would wait
 //     for the first, else two; kmax = 4: 256 x 3, two items (M = 144: 0.44 against
 //     0.50 at 128 x 6); larger M 256 x 3, then 384 x 2;
-//   FP64: 256 x 2, one item per CTA slot (M = 111, kmax = 5: 11.2 against 12.3;
-//     M = 50: 0.35 against 0.47); a kmax = 4 table large enough for the prefix tree
+//   FP64: the wide 256 x 3, one item per CTA slot (M = 111, kmax = 5: 10.9 against
+//     11.2 at 256 x 2 and 12.3 at 512 x 1; M = 50: 0.32 against 0.34 and 0.47); a kmax = 4 table large enough for the prefix tree
 //     (gbs_launch.cuh) 512 x 1 with eight (M = 300: 23.5 against 24.9).
 inline TreeCfg default_cfg(int M, int kmax, int precision) {
     TreeCfg c = kDefaultCfg;
@@ -99,8 +99,8 @@ inline TreeCfg default_cfg(int M, int kmax, int precision) {
         c.variant = kmax == 5 && M <= kVariant2MaxM ? 2 : M <= kVariant4MaxM ? 4 : M <= kVariant5MaxM ? 5 : 0;
         c.grain = kmax == 5 && M < 128 ? 1 : 2;
     } else if (kmax == 5) {
-        c.variant = M <= kVariant1MaxM ? 1 : 0;
-        c.grain = c.variant == 1 ? 1 : 2;
+        c.variant = M <= kVariant4MaxM ? 4 : 0;
+        c.grain = c.variant == 4 ? 1 : 2;
     } else {
         c.grain = 8;
     }
@@ -114,9 +114,9 @@ constexpr int kNumVariants = 10;
 // shapes that do not admit M (or the precision) fall back to 512 x 1.
 inline int effective_variant(int variant, int M, int precision) {
     if (variant == 1 || variant == 3 || variant == 8) return M <= kVariant1MaxM && (variant == 1 || precision == 1) ? variant : 0;
+    if (variant == 4) return M <= kVariant4MaxM ? 4 : 0;
     if (precision != 1) return 0;
     if (variant == 2) return M <= kVariant2MaxM ? 2 : 0;
-    if (variant == 4) return M <= kVariant4MaxM ? 4 : 0;
     if (variant == 5) return M <= kVariant5MaxM ? 5 : 0;
     if (variant == 6 || variant == 7) return M <= kVariant6MaxM ? variant : 0;
     if (variant == 9) return M <= kVariant9MaxM ? 9 : 0;

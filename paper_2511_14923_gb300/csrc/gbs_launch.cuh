@@ -241,11 +241,14 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
     if (a.grain <= 0) a.grain = kDefaultCfg.grain;
     if (a.ccap <= 0 || a.ccap > CCAP) a.ccap = kDefaultCfg.ccap;
     if constexpr (DISP) {
-        // displaced states: FP64, one 512-thread CTA per multiprocessor
+        // displaced states: FP64, two 256-thread CTAs per multiprocessor, one of 512
+        // where their x area does not admit M
+        if (a.M <= kVariant1MaxM) return launch_tree_v<D, MODE, 0, 256, 576, 2, true, kNoSlotCC>(a, write_p0, st);
         return launch_tree_v<D, MODE, 0, TREE_THREADS, XCAP, 1, true>(a, write_p0, st);
     } else {
         const int v = effective_variant(a.variant, a.M, PREC);
         if (v == 1) return launch_tree_v<D, MODE, PREC, 256, 576, 2, false>(a, write_p0, st);
+        if (v == 4) return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
         if constexpr (PREC == 1) {
             // 24 warps with 80 registers in 6 CTAs of 4, 3 of 8 (with room for up to 64
             // children a batch, or for more x-entries) or 2 of 12; or 32 warps with 64
@@ -255,7 +258,7 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
             // (its order 4, whose items are small, in the wide 256 x 3 shape: 0.44 against 0.50 ms)
             if (v == 2 && D == 5) return launch_tree_v<D, MODE, PREC, 128, kSmallXC, 6, false, kNoSlotCC>(a, write_p0, st);
             if (v == 3) return launch_tree_v<D, MODE, PREC, 256, 576, 3, false>(a, write_p0, st);
-            if (v == 4 || v == 2) return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
+            if (v == 2) return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
             if (v == 5) return launch_tree_v<D, MODE, PREC, 384, kPairXC, 2, false>(a, write_p0, st);
             if (v == 6) {
                 // order 4 of the 256 x 4 shape runs without slots where it can: its items
@@ -307,11 +310,12 @@ static cudaError_t launch_order3(const FwdArgs &a, bool write_p0, int c_lo, int 
 template <int MODE, int PREC, bool DISP>
 static cudaError_t launch_order4(const FwdArgs &a, bool write_p0, int c_lo, int c_hi, cudaStream_t st) {
     using Shape = ChunkShape<2, PREC, DISP>;
-    const size_t smem = chunk_smem(a.M - 2, kOrder4Pairs, Shape::PX, Shape::PR);
+    const uint32_t L = a.M < 64 ? kOrder4Pairs / 16 : kOrder4Pairs;  // small tables: split the largest prefixes
+    const size_t smem = chunk_smem(a.M - 2, L, Shape::PX, Shape::PR);
     const int below = DISP ? GBS_MAX_MODES + 1 : PREC == 1 ? kOrder4ChunkedR : kOrder4ChunkedZ;
     if (a.M < below && smem <= kChunkSmem) {
         if (c_hi <= 3 || c_hi <= c_lo) return cudaSuccess;
-        return launch_chunk<2, MODE, PREC, DISP>(a, write_p0, c_lo, c_hi, kOrder4Pairs, smem, st);
+        return launch_chunk<2, MODE, PREC, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
     }
     return launch_tree<4, MODE, PREC, DISP>(a, write_p0, st);
 }

@@ -202,7 +202,8 @@ void record_batch_cfg(int sms, const gbs_instance *inst, int n, int precision, c
 
 int autotune(FwdArgs a, cudaStream_t st, TreeCfg &best, float &best_ms, int &tried) {
     std::vector<TreeCfg> cand;
-    for (int variant = 0; variant <= (a.precision == 1 ? kNumVariants - 1 : 1); ++variant) {
+    for (int variant = 0; variant < kNumVariants; ++variant) {
+        if (a.precision == 0 && variant > 1 && variant != 4) continue;
         if ((variant == 1 || variant == 3) && a.M > kVariant1MaxM) continue;
         if (variant == 2 && a.M > kVariant2MaxM) continue;
         if (variant == 4 && a.M > kVariant4MaxM) continue;
