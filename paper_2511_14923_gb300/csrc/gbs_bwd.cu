@@ -48,20 +48,35 @@ __host__ __device__ inline Offsets make_offsets(int M) {
     return o;
 }
 
-// h table, order r (all lower orders done): h(R) = -sum_{T nonempty subset R} P0(T) h(R - T).
-__global__ void h_kernel(int M, int r, Offsets o, const double *__restrict__ p0, double *__restrict__ h) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= binom(M, r)) return;
-    int s[GBS_MAX_ORDER];
-    colex_unrank(i, r, s);
-    const unsigned full = (1u << r) - 1;
-    double acc = 0.0;
-    for (unsigned t = 1; t <= full; ++t) {
-        const unsigned rest = full ^ t;
-        const double hr = rest ? h[sub_index(s, r, rest, o.off)] : 1.0;
-        acc = fma(-p0[sub_index(s, r, t, o.off)], hr, acc);
+// h table of every order below kmax in one launch: h(R) = -sum_{T nonempty subset R}
+// P0(T) h(R - T). A thread forms h of all subsets of its R from their P0 (at most 81
+// products), so no order waits for the one below.
+template <int D>
+__device__ __forceinline__ void h_entry(uint64_t i, const Offsets &o, const double *__restrict__ p0,
+                                        double *__restrict__ h) {
+    int s[D];
+    colex_unrank(i, D, s);
+    double p[1 << D], hh[1 << D];
+    hh[0] = 1.0;
+#pragma unroll
+    for (unsigned m = 1; m < (1u << D); ++m) {
+        p[m] = p0[sub_index(s, D, m, o.off)];
+        double acc = 0.0;
+#pragma unroll
+        for (unsigned t = 1; t <= m; ++t)
+            if ((t & m) == t) acc = fma(-p[t], hh[m ^ t], acc);
+        hh[m] = acc;
     }
-    h[o.off[r] + i] = acc;
+    h[o.off[D] + i] = hh[(1 << D) - 1];
+}
+__global__ void __launch_bounds__(BWD_THREADS) h_kernel(uint64_t n, Offsets o, const double *__restrict__ p0,
+                                                        double *__restrict__ h) {
+    const uint64_t i = (uint64_t)blockIdx.x * BWD_THREADS + threadIdx.x;
+    if (i >= n) return;
+    if (i < o.off[2]) h_entry<1>(i, o, p0, h);
+    else if (i < o.off[3]) h_entry<2>(i - o.off[2], o, p0, h);
+    else if (i < o.off[4]) h_entry<3>(i - o.off[3], o, p0, h);
+    else h_entry<4>(i - o.off[4], o, p0, h);
 }
 
 // grad_V scatter, order d (used for d = 1): -1/4 gP0(T) P0(T) A_T^{-1} into the rows/cols of T,
@@ -245,11 +260,13 @@ __device__ __forceinline__ double gather_walk(int M, const Offsets &o, const int
     return ((BB + R) & 1) ? -t : t;
 }
 
+// gP0 of the order-BB subsets by one block of GATHER_THREADS.
+constexpr int GATHER_THREADS = 1024;
 template <int BB>
-__global__ void __launch_bounds__(1024) gp0_gather_kernel(int M, int kmax, Offsets o, const double *__restrict__ gk,
-                                                          const double *__restrict__ h, double *__restrict__ gp0,
-                                                          int team) {
-    const uint64_t gt = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void gather_block(int M, int kmax, const Offsets &o, const double *__restrict__ gk,
+                                             const double *__restrict__ h, double *__restrict__ gp0, int team,
+                                             unsigned block) {
+    const uint64_t gt = (uint64_t)block * GATHER_THREADS + threadIdx.x;
     const uint64_t unit_b = gt / team;
     const int lane = (int)(gt % team);
     const bool live = unit_b < binom(M, BB);
@@ -300,10 +317,33 @@ __global__ void __launch_bounds__(1024) gp0_gather_kernel(int M, int kmax, Offse
     }
 }
 
-// gP0 for the top order: only R = empty contributes, gP0(B) = g_y(B).
-__global__ void gp0_top_kernel(uint64_t n, double sign, const double *__restrict__ gk, double *__restrict__ gp0) {
-    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) gp0[i] = sign * gk[i];
+// gP0 of every order in one launch: the orders don't read each other, and each by
+// itself leaves much of the GPU waiting for its gathers (M = 100, kmax = 4: 92, 125,
+// 60 and 13 us one after the other, about 270 together). Blocks of order 1 first (the
+// longest walks), then 2, 3, 4; the top order (only R = empty contributes, gP0(B) =
+// g_y(B)) last.
+struct GatherPlan {
+    unsigned end[GBS_MAX_ORDER];  // end[b - 1] = one past the last block of order b < kmax
+    int team[GBS_MAX_ORDER];
+};
+__global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(int M, int kmax, Offsets o,
+                                                                const double *__restrict__ gk,
+                                                                const double *__restrict__ h,
+                                                                double *__restrict__ gp0, GatherPlan pl) {
+    const unsigned b = blockIdx.x;
+    if (b >= pl.end[GBS_MAX_ORDER - 2]) {
+        const uint64_t i = (uint64_t)(b - pl.end[GBS_MAX_ORDER - 2]) * GATHER_THREADS + threadIdx.x;
+        const double sign = (kmax & 1) ? -1.0 : 1.0;
+        if (i < binom(M, kmax)) gp0[o.off[kmax] + i] = sign * gk[o.off[kmax] + i];
+    } else if (b < pl.end[0]) {
+        gather_block<1>(M, kmax, o, gk, h, gp0, pl.team[0], b);
+    } else if (b < pl.end[1]) {
+        gather_block<2>(M, kmax, o, gk, h, gp0, pl.team[1], b - pl.end[0]);
+    } else if (b < pl.end[2]) {
+        gather_block<3>(M, kmax, o, gk, h, gp0, pl.team[2], b - pl.end[1]);
+    } else {
+        gather_block<4>(M, kmax, o, gk, h, gp0, pl.team[3], b - pl.end[2]);
+    }
 }
 
 // A_{T'}^{-1} for every order-DP subset T' (rows x of T', then p of T'), packed
@@ -762,31 +802,32 @@ cudaError_t launch_backward(const BwdArgs &a, cudaStream_t st) {
     if ((e = launch_forward(f, st)) != cudaSuccess) return e;
     mark(1);
     // 2. h table, orders 1..kmax-1
-    for (int r = 1; r < K; ++r) {
-        const uint64_t n = binom(M, r);
-        h_kernel<<<(unsigned)((n + BWD_THREADS - 1) / BWD_THREADS), BWD_THREADS, 0, st>>>(M, r, o, a.p0, a.h);
+    const uint64_t nh = o.off[K];  // subsets of order below K
+    if (nh) {
+        h_kernel<<<(unsigned)((nh + BWD_THREADS - 1) / BWD_THREADS), BWD_THREADS, 0, st>>>(nh, o, a.p0, a.h);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     mark(2);
     // 3. gP0 by gathering over supersets (one team of threads per subset B)
-    for (int b = 1; b <= K; ++b) {
-        const uint64_t n = binom(M, b);
-        if (b == K) {
-            gp0_top_kernel<<<(unsigned)((n + BWD_THREADS - 1) / BWD_THREADS), BWD_THREADS, 0, st>>>(
-                n, (K & 1) ? -1.0 : 1.0, a.gk + o.off[K], a.gp0 + o.off[K]);
-        } else {
-            // team size: about four units per lane, at most one block per B
-            uint64_t units = 0;
-            for (int q = 0; q < K - b; ++q) units += binom(M - b, q);
-            int team = 1;
-            while (team < 1024 && 4 * (uint64_t)team < units) team *= 2;
-            const int nt = team > 32 ? team : 256;  // a team wider than a warp fills its block
-            const unsigned gl = (unsigned)((n * team + nt - 1) / nt);
-            if (b == 1) gp0_gather_kernel<1><<<gl, nt, 0, st>>>(M, K, o, a.gk, a.h, a.gp0, team);
-            else if (b == 2) gp0_gather_kernel<2><<<gl, nt, 0, st>>>(M, K, o, a.gk, a.h, a.gp0, team);
-            else if (b == 3) gp0_gather_kernel<3><<<gl, nt, 0, st>>>(M, K, o, a.gk, a.h, a.gp0, team);
-            else gp0_gather_kernel<4><<<gl, nt, 0, st>>>(M, K, o, a.gk, a.h, a.gp0, team);
+    {
+        GatherPlan pl{};
+        unsigned blocks = 0;
+        for (int b = 1; b < GBS_MAX_ORDER; ++b) {
+            pl.team[b - 1] = 1;
+            if (b < K) {
+                // team size: about four units per lane, at most one block per B
+                uint64_t units = 0;
+                for (int q = 0; q < K - b; ++q) units += binom(M - b, q);
+                int team = 1;
+                while (team < GATHER_THREADS && 4 * (uint64_t)team < units) team *= 2;
+                if (team > 32) team = GATHER_THREADS;  // a team wider than a warp is a whole block
+                pl.team[b - 1] = team;
+                blocks += (unsigned)((binom(M, b) * team + GATHER_THREADS - 1) / GATHER_THREADS);
+            }
+            pl.end[b - 1] = blocks;
         }
+        blocks += (unsigned)((binom(M, K) + GATHER_THREADS - 1) / GATHER_THREADS);
+        gather_kernel<<<blocks, GATHER_THREADS, 0, st>>>(M, K, o, a.gk, a.h, a.gp0, pl);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     mark(3);
