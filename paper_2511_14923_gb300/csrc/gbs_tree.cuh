@@ -5,6 +5,8 @@
 #pragma once
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "gbs.h"
 #include "gbs_common.cuh"
 #include "gbs_fwd.cuh"
@@ -16,6 +18,17 @@ constexpr int FLAT_THREADS = 256;
 constexpr int TREE_THREADS = 512;
 constexpr int XCAP = 1152;  // per-batch x-entries in shared memory (>= GBS_MAX_MODES)
 constexpr int CCAP = kMaxChildren;  // per-batch children
+
+// x * 2^K by its exponent on the integer pipe (GB300 issues 2 FP64 instructions per
+// clock and multiprocessor): exact where x and the result are normal numbers; zero,
+// infinity, NaN and what lies within 2^|K| of the range's ends come back as they are.
+template <int K>
+__device__ __forceinline__ double mul_pow2(double x) {
+    const unsigned h = (unsigned)__double2hiint(x), e = (h >> 20) & 0x7ffu;
+    constexpr unsigned lo = K < 0 ? 1 - K : 1, hi = K < 0 ? 0x7ff : 0x7ff - K;
+    const unsigned g = e - lo < hi - lo ? h + (unsigned)(K * (1 << 20)) : h;
+    return __hiloint2double((int)g, __double2loint(x));
+}
 
 // ---------------------------------------------------------------- shared combine step
 
@@ -98,13 +111,22 @@ __device__ __forceinline__ double combine(double P0S, int j, int c2, uint32_t t,
                                   p0R, p0tab, outtab);
 }
 
-// Weight of the recursion's product with R = Q + {c2} (bitmask q) in the
-// accumulator of sign sd.
-template <int MODE>
-__device__ __forceinline__ constexpr double upper_weight(int q, double sd) {
-    int n = 0;
-    for (int b = q; b; b &= b - 1) ++n;
-    return MODE == MODE_KAPPA ? ((n & 1) ? sd : -sd) : -1.0 / (double)(4 << n);
+// The recursion's weights for the table value of R + {j}, n = |R| (R within P, or
+// R = Q + {c2} with n = |Q| + 1): (-1)^n of the order's sign for the click cumulant,
+// -2^{-(n+1)} for the spin cumulant (an exponent, no FP64 instruction).
+template <int MODE, int N>
+__device__ __forceinline__ double weighted(double x, double sd) {
+    if constexpr (MODE == MODE_SPINK) return -mul_pow2<-(N + 1)>(x);
+    else return (N & 1) ? -sd * x : sd * x;
+}
+__host__ __device__ constexpr int bits_of(int q) { return q ? (q & 1) + bits_of(q >> 1) : 0; }
+// f(integral constant q) for q = Q0 .. Q1 - 1
+template <int Q0, int Q1, class F>
+__device__ __forceinline__ void for_subsets(F f) {
+    if constexpr (Q0 < Q1) {
+        f(std::integral_constant<int, Q0>{});
+        for_subsets<Q0 + 1, Q1>(f);
+    }
 }
 
 // Sign carried by the accumulator of the cumulant recursion: (-1)^d for the
@@ -124,15 +146,13 @@ __device__ __forceinline__ double combine_tail(double acc, int j, int c2, uint32
                                                const double *__restrict__ p0tab, const double *__restrict__ outtab) {
     constexpr int PALL = (1 << NP) - 1;
     constexpr double sd = lead_sign<NP, MODE>();
-#pragma unroll
-    for (int q = 1; q <= PALL; ++q) {
-        const double sg = (MODE == MODE_KAPPA) ? ((__popc(q) & 1) ? -sd : sd)
-                                               : -1.0 / (double)(2 << __popc(q));  // -2^{-(|R|+1)}, R = Q
-        acc = fma(sg * outtab[baseJ[q] + j], p0tab[baseJ[PALL ^ q] + c2], acc);
-    }
-#pragma unroll
-    for (int q = 0; q < PALL; ++q) acc = fma(upper_weight<MODE>(q, sd) * outtab[baseT[q] + t], p0R[PALL ^ q], acc);
-    if (MODE == MODE_SPINK) return acc * (double)(1 << (NP + 2));
+    for_subsets<1, PALL + 1>([&](auto q) {
+        acc = fma(weighted<MODE, bits_of(q())>(outtab[baseJ[q()] + j], sd), p0tab[baseJ[PALL ^ q()] + c2], acc);
+    });
+    for_subsets<0, PALL>([&](auto q) {
+        acc = fma(weighted<MODE, bits_of(q()) + 1>(outtab[baseT[q()] + t], sd), p0R[PALL ^ q()], acc);
+    });
+    if constexpr (MODE == MODE_SPINK) return mul_pow2<NP + 2>(acc);
     return acc;
 }
 
@@ -159,9 +179,8 @@ __device__ __forceinline__ PairSum combine_products(const float2 (&k)[1 << NP], 
     constexpr int PALL = (1 << NP) - 1;
     constexpr double sd = lead_sign<NP, MODE>();
     PairSum r;
-    r.acc = upper_weight<MODE>(0, sd) * u[0] * p0R[PALL];
-#pragma unroll
-    for (int q = 1; q < PALL; ++q) r.acc = fma(upper_weight<MODE>(q, sd) * u[q], p0R[PALL ^ q], r.acc);
+    r.acc = weighted<MODE, 1>(u[0], sd) * p0R[PALL];
+    for_subsets<1, PALL>([&](auto q) { r.acc = fma(weighted<MODE, bits_of(q()) + 1>(u[q()], sd), p0R[PALL ^ q()], r.acc); });
     const DF f = df_mulu(DF{-k[1].x, -k[1].y}, DF{p[PALL ^ 1].x, p[PALL ^ 1].y});
     r.g = Acc{f.h, f.l};
 #pragma unroll
@@ -182,7 +201,8 @@ __device__ __forceinline__ double combine_lead(PairSum r, float r0, float eta, f
     const unsigned flip = lead_sign<NP, MODE>() < 0 ? 0x80000000u : 0u;
     const double v = r.acc + f2d_bits(__uint_as_float(__float_as_uint(r.g.s) ^ flip)) +
                      f2d_bits(__uint_as_float(__float_as_uint(r.g.t) ^ flip));
-    return MODE == MODE_SPINK ? v * (double)(1 << (NP + 2)) : v;
+    if constexpr (MODE == MODE_SPINK) return mul_pow2<NP + 2>(v);
+    return v;
 }
 
 template <int MODE>
