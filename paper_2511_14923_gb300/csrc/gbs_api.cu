@@ -256,13 +256,11 @@ int gbs_timing_read_backward(float *ms_out) {
 int gbs_stream_status(const void *workspace, void *cuda_stream) {
     if (!workspace) return fail(GBS_ERR_INVALID_ARG, "NULL workspace");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // the copy follows the stream's work and, into pageable memory, returns when it is
-    // done: one wait instead of a synchronisation and a copy of their own
-    unsigned s = 0;
-    cudaError_t e = cudaMemcpyAsync(&s, workspace, sizeof s, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "reading the status word: %s", cudaGetErrorString(e));
-    e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "cudaStreamSynchronize: %s", cudaGetErrorString(e));
+    unsigned s = 0;
+    e = cudaMemcpy(&s, workspace, sizeof s, cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "reading the status word: %s", cudaGetErrorString(e));
     return gbs_status_code(s);
 }
 
