@@ -138,7 +138,7 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
     a.slots = L.slots;
     a.sms = sms;
     a.ev = nullptr;
-    const gbs::TreeCfg cfg = gbs::tuned_cfg(sms, M, kmax, precision);
+    const gbs::TreeCfg cfg = gbs::tuned_cfg(sms, M, kmax, precision, mode);
     a.grain = cfg.grain;
     a.ccap = cfg.ccap;
     a.variant = cfg.variant;
@@ -308,7 +308,7 @@ int gbs_cumulants_backward(const double *V, int M, int kmax, const double *grad_
     a.mode = gbs::MODE_P0;
     a.precision = GBS_FP32_REFINED;  // the P0 recomputation (launch_backward)
     {
-        const gbs::TreeCfg cfg = gbs::tuned_cfg(sms, M, kmax, GBS_FP32_REFINED);
+        const gbs::TreeCfg cfg = gbs::tuned_cfg(sms, M, kmax, GBS_FP32_REFINED, gbs::MODE_P0);
         a.grain = cfg.grain;
         a.ccap = cfg.ccap;
         a.variant = cfg.variant;

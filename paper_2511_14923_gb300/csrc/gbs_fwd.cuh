@@ -38,11 +38,10 @@ struct FwdArgs {
     uint64_t top_base;
     int c_lo, c_hi;
     // prefix-tree schedule (autotuned): items per CTA slot, children per shared-
-    // memory batch, CTA shape (0: 512 threads x 1 per SM; 1: 256 x 2; refined path
-    // only: 2: 128 x 6 with a 304-entry x area, 3: 256 x 3, 4: 256 x 3 with a 672-entry
-    // x area, 5: 384 x 2
-    // with a 960-entry x area, 6: 256 x 4 with a 384-entry x area, 7: 6 in clusters
-    // of 4, 8: 3 in clusters of 3, 9: 6 without Schur-complement slots)
+    // memory batch, CTA shape (0: 512 threads x 1 per SM; 1: 256 x 2; 4: 256 x 3 with a
+    // 672-entry x area; refined path only: 2: 128 x 6 with a 304-entry x area, 3: 256 x
+    // 3, 5: 384 x 2 with a 960-entry x area, 6: 256 x 4 with a 384-entry x area, 7: 6 in
+    // clusters of 4, 8: 3 in clusters of 3, 9: 6 without Schur-complement slots)
     int grain, ccap, variant;
 };
 
@@ -89,14 +88,22 @@ constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1
 //     10.7 at 256 x 3 and 17.7 at 512 x 1; M = 77: 0.64 against 0.66 and 1.2), one
 //     item per CTA slot below 128 modes, where a second round of items would wait
 //     for the first, else two; kmax = 4: 256 x 3, two items (M = 144: 0.44 against
-//     0.50 at 128 x 6); larger M 256 x 3, then 384 x 2;
+//     0.50 at 128 x 6), but 256 x 4 for the tables without gathers on pairs (P0, M =
+//     100: 85 us against 105; M = 77, kmax = 5: 363 against 370 the call); larger M
+//     256 x 3, then 384 x 2;
 //   FP64: the wide 256 x 3, one item per CTA slot (M = 111, kmax = 5: 10.9 against
-//     11.2 at 256 x 2 and 12.3 at 512 x 1; M = 50: 0.32 against 0.34 and 0.47); a kmax = 4 table large enough for the prefix tree
-//     (gbs_launch.cuh) 512 x 1 with eight (M = 300: 23.5 against 24.9).
-inline TreeCfg default_cfg(int M, int kmax, int precision) {
+//     11.2 at 256 x 2 and 12.3 at 512 x 1; M = 50: 0.32 against 0.34 and 0.47); a
+//     kmax = 4 table large enough for the prefix tree (gbs_launch.cuh) 512 x 1 with
+//     eight (M = 300: 23.5 against 24.9).
+inline TreeCfg default_cfg(int M, int kmax, int precision, int mode) {
     TreeCfg c = kDefaultCfg;
     if (precision == 1) {
-        c.variant = kmax == 5 && M <= kVariant2MaxM ? 2 : M <= kVariant4MaxM ? 4 : M <= kVariant5MaxM ? 5 : 0;
+        const bool cumulants = mode == MODE_KAPPA || mode == MODE_SPINK;
+        c.variant = kmax == 5 && M <= kVariant2MaxM                ? 2
+                    : kmax == 4 && !cumulants && M <= kVariant6MaxM ? 6
+                    : M <= kVariant4MaxM                            ? 4
+                    : M <= kVariant5MaxM                            ? 5
+                                                                    : 0;
         c.grain = kmax == 5 && M < 128 ? 1 : 2;
     } else if (kmax == 5) {
         c.variant = M <= kVariant4MaxM ? 4 : 0;

@@ -254,13 +254,15 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
             // children a batch, or for more x-entries) or 2 of 12; or 32 warps with 64
             // registers in 4 CTAs. Order 5 runs fastest in the smallest CTAs, whose
             // batches wait least at their barriers (M = 144: 128 x 6 10.6 ms, 256 x 3
-            // 10.7, 256 x 4 11.6, the shared gathers spilling at 64 registers)
-            // (its order 4, whose items are small, in the wide 256 x 3 shape: 0.44 against 0.50 ms)
+            // 10.7, 256 x 4 11.6, the shared gathers spilling at 64 registers). Order 4
+            // of that shape, whose items are small, runs in the wide 256 x 3 one (0.44
+            // against 0.50 ms), or in 256 x 4 where it has no such gathers.
             if (v == 2 && D == 5) return launch_tree_v<D, MODE, PREC, 128, kSmallXC, 6, false, kNoSlotCC>(a, write_p0, st);
+            if (v == 2 && (MODE == MODE_KAPPA || MODE == MODE_SPINK))
+                return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
             if (v == 3) return launch_tree_v<D, MODE, PREC, 256, 576, 3, false>(a, write_p0, st);
-            if (v == 2) return launch_tree_v<D, MODE, PREC, 256, kWideXC, 3, false, kNoSlotCC>(a, write_p0, st);
             if (v == 5) return launch_tree_v<D, MODE, PREC, 384, kPairXC, 2, false>(a, write_p0, st);
-            if (v == 6) {
+            if (v == 6 || v == 2) {
                 // order 4 of the 256 x 4 shape runs without slots where it can: its items
                 // are small (one U = {c4} split into many stride classes), so rebuilding
                 // the slot per item cost more than forming the blocks in place (same bits)

@@ -175,11 +175,11 @@ int device_cc() {
 
 }  // namespace
 
-TreeCfg tuned_cfg(int sms, int M, int kmax, int precision) {
+TreeCfg tuned_cfg(int sms, int M, int kmax, int precision, int mode) {
     std::lock_guard<std::mutex> lock(g_mu);
     load_locked();
     auto it = g_table.find(Key{device_cc(), sms, M, kmax, precision});
-    return it == g_table.end() ? default_cfg(M, kmax, precision) : it->second.cfg;
+    return it == g_table.end() ? default_cfg(M, kmax, precision, mode) : it->second.cfg;
 }
 
 bool tuned_batch_cfg(int sms, const gbs_instance *inst, int n, int precision, TreeCfg &cfg) {
