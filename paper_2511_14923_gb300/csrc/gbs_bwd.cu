@@ -319,7 +319,7 @@ __device__ __forceinline__ void gather_block(int M, int kmax, const Offsets &o, 
 
 // gP0 of every order in one launch: the orders don't read each other, and each by
 // itself leaves much of the GPU waiting for its gathers (M = 100, kmax = 4: 92, 125,
-// 60 and 13 us one after the other, about 270 together). Blocks of order 1 first (the
+// 60 and 13 us one after the other, 226 together). Blocks of order 1 first (the
 // longest walks), then 2, 3, 4; the top order (only R = empty contributes, gP0(B) =
 // g_y(B)) last.
 struct GatherPlan {
@@ -889,7 +889,7 @@ __device__ __forceinline__ double qdiag(const double *r, int M, int k) {
 // time through shared memory. The FP64 pipe binds (2 FMAs per clock and
 // multiprocessor), so a matrix that 32-wide tiles would put on a fraction of the
 // multiprocessors takes 16-wide ones: M = 100 leaves 28 wide tiles (87 us) or 91
-// narrow ones (25 us). One chain of FMAs per element either way.
+// narrow ones (37 us). One chain of FMAs per element either way.
 constexpr int COV_K = 32;
 
 template <int T>

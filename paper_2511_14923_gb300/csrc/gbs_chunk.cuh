@@ -48,6 +48,8 @@ __global__ void __launch_bounds__(CHUNK_THREADS, DISP ? 4 : 6)
     constexpr int NQ = 1 << NP, PALL = NQ - 1;
     extern __shared__ __align__(16) double shc[];
     __shared__ ChunkPrefix<NP> pre;
+    await_previous();
+    if (NP + 2 < a.kmax) release_next();
     const int M = a.M;
     // prefixes with the largest top element first
     int P[3] = {0, 0, 0};
@@ -292,8 +294,8 @@ static cudaError_t launch_chunk(const FwdArgs &a, bool write_p0, int c_lo, int c
     const int hi = c_hi - 1, lo = c_lo > NP + 1 ? c_lo : NP + 1;  // largest and smallest top element
     const int c3 = hi - (NP - 1);
     const uint64_t prefixes = NP == 1 ? (uint64_t)(hi - lo + 1) : binom2(hi + 1) - binom2(lo);
-    fn<<<dim3((unsigned)prefixes, (unsigned)((binom2(c3) + L - 1) / L)), CHUNK_THREADS, smem, st>>>(a, write_p0, hi, L);
-    return cudaGetLastError();
+    return launch_next(!a.ev, fn, dim3((unsigned)prefixes, (unsigned)((binom2(c3) + L - 1) / L)), CHUNK_THREADS, smem, st, a,
+                       write_p0, hi, L);
 }
 
 }  // namespace gbs

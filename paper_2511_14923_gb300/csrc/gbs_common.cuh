@@ -194,6 +194,36 @@ __device__ __forceinline__ void flag_status(unsigned *status, unsigned bits) {
     if (status) atomicOr(status, bits);
 }
 
+// Chains of dependent kernels. A kernel queued by launch_next may start while the one
+// before it in the stream still runs, and awaits that one's end (its writes visible)
+// before it reads or writes global memory: every thread calls await_previous first.
+// A kernel whose successor is queued so calls release_next after that, which lets the
+// successor's CTAs take the places left as soon as all of its own have one, so the
+// 2-3 us from one kernel's last block to the next one's first are spent waiting in
+// place. Since each kernel awaits its predecessor, the end of one is the end of all
+// before it; the last kernel of a call releases nothing, so whatever the caller queues
+// next starts as after any kernel. Both are no-ops in an ordinary launch.
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Queues fn after the kernel queued before it in st, as above (chained), or as an
+// ordinary launch.
+template <class... P, class... Q>
+inline cudaError_t launch_next(bool chained, void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                               Q... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+}
+
 // Host-side fault injection, for tests of the error paths: true when the
 // environment variable GBS_FAULT_INJECT lists `site` (comma-separated names).
 // Sites: "forward_memset" (the forward calls' first runtime call is treated as

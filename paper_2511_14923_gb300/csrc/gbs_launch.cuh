@@ -19,13 +19,19 @@ constexpr size_t kChunkSmem = 226 * 1024;
 // blocks [0, nb0) pack, [nb0, nb0 + nb1) fill order 1, the rest order 2; one thread
 // per block of A or subset of colex rank first + i, i < count (the whole order, or
 // the rank range of a range call's top order). Three dependent launches of 3-6 us
-// each before; one of about 7 now (call totals below).
+// each before; one of about 7 now.
 struct Span {
     uint64_t first, count;
 };
+// Orders 3 and 4 by chunks are chained to what is before them (launch_next): M = 50,
+// kmax = 4 65.1 -> 58.9 us, M = 97 displaced 564 -> 560. The persistent prefix-tree
+// kernels are not: their CTAs, in place early, keep the split of shared memory and
+// first-level cache of the kernel before for their whole run (M = 144, kmax = 5,
+// refined 10.57 -> 10.76 ms chained).
 template <int MODE, bool DISP>
 __global__ void __launch_bounds__(FLAT_THREADS) front_kernel(FwdArgs a, bool wp1, bool wp2, Span s1, Span s2,
                                                              unsigned nb0, unsigned nb1) {
+    if (a.kmax >= 3) release_next();  // itself queued after the memset of the counters
     if (blockIdx.x < nb0) {
         const uint64_t i = (uint64_t)blockIdx.x * FLAT_THREADS + threadIdx.x;
         if (i < (uint64_t)a.M * a.M) pack_entry(a.V, a.M, a.A, a.precision == 1 ? a.Af : nullptr, (int)i);
@@ -41,6 +47,7 @@ __global__ void __launch_bounds__(FLAT_THREADS) front_kernel(FwdArgs a, bool wp1
 // Flat kernel of order 3: one thread per subset of colex rank first + i, i < count.
 template <int MODE, bool DISP>
 __global__ void order3_kernel(FwdArgs a, bool write_p0, uint64_t first, uint64_t count) {
+    await_previous();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) order3_entry<MODE, DISP>(a, first + i, write_p0);
 }
@@ -296,9 +303,8 @@ static cudaError_t launch_order3(const FwdArgs &a, bool write_p0, int c_lo, int 
     using Shape = ChunkShape<1, 0, DISP>;
     const size_t smem = chunk_smem(c_hi - 1, L, Shape::PX, Shape::PR);
     if (smem <= kChunkSmem) return launch_chunk<1, MODE, 0, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
-    order3_kernel<MODE, DISP><<<(unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS), FLAT_THREADS, 0, st>>>(a, write_p0,
-                                                                                                 first, n);
-    return cudaGetLastError();
+    return launch_next(!a.ev, order3_kernel<MODE, DISP>, (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS), FLAT_THREADS, 0,
+                       st, a, write_p0, first, n);
 }
 
 // Order 4, top elements in [c_lo, c_hi): by chunks below kOrder4ChunkedZ / R

@@ -240,6 +240,8 @@ constexpr int ETB = 64;  // threads per block of the per-(entry, sample) kernels
 
 template <class R, int K>
 __global__ void __launch_bounds__(ETB) w_kernel(Args<R> a, int t, int D) {
+    await_previous();
+    if constexpr (K == 3) release_next();
     const int s = blockIdx.x * ETB + threadIdx.x;
     const size_t S = (size_t)a.S;
     // this block's share of r = 0 .. D-1, walked in order
@@ -288,6 +290,8 @@ __global__ void __launch_bounds__(ETB) w_kernel(Args<R> a, int t, int D) {
 // tile is chosen by the CTAs it leaves (launch_zgemm).
 template <class R, int K, int T>
 __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t rows, int D) {
+    await_previous();
+    if constexpr (K == 3) release_next();
     constexpr int BT = 16 * T, BK = T == 1 ? 16 : 8;
     constexpr int E = BT * BK / 256;  // elements of each operand per thread per stage
     __shared__ __align__(16) R As[2][BK][BT];
@@ -374,17 +378,19 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
 // the 64-wide FP64 tiles used before left 56-80 CTAs for 152 multiprocessors at
 // the heaviest steps: 179 ms a call, 31 ms being the pipe's.
 template <class R, int K>
-static void launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
+static cudaError_t launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
     auto ctas = [&](int bt) { return (rows + bt - 1) / bt * (uint64_t)(a.S / bt); };
     auto grid = [&](int bt) { return dim3((unsigned)((rows + bt - 1) / bt), (unsigned)(a.S / bt)); };
+    cudaError_t e;
     if constexpr (sizeof(R) == 4) {
-        if (ctas(128) >= 2 * (uint64_t)sms) zgemm_kernel<R, K, 8><<<grid(128), 256, 0, st>>>(a, t, rows, D);
-        else if (ctas(64) >= 2 * (uint64_t)sms) zgemm_kernel<R, K, 4><<<grid(64), 256, 0, st>>>(a, t, rows, D);
-        else zgemm_kernel<R, K, 2><<<grid(32), 256, 0, st>>>(a, t, rows, D);
+        if (ctas(128) >= 2 * (uint64_t)sms) e = launch_next(K == 3, zgemm_kernel<R, K, 8>, grid(128), 256, 0, st, a, t, rows, D);
+        else if (ctas(64) >= 2 * (uint64_t)sms) e = launch_next(K == 3, zgemm_kernel<R, K, 4>, grid(64), 256, 0, st, a, t, rows, D);
+        else e = launch_next(K == 3, zgemm_kernel<R, K, 2>, grid(32), 256, 0, st, a, t, rows, D);
     } else {
-        if (ctas(32) >= 8 * (uint64_t)sms) zgemm_kernel<R, K, 2><<<grid(32), 256, 0, st>>>(a, t, rows, D);
-        else zgemm_kernel<R, K, 1><<<grid(16), 256, 0, st>>>(a, t, rows, D);
+        if (ctas(32) >= 8 * (uint64_t)sms) e = launch_next(K == 3, zgemm_kernel<R, K, 2>, grid(32), 256, 0, st, a, t, rows, D);
+        else e = launch_next(K == 3, zgemm_kernel<R, K, 1>, grid(16), 256, 0, st, a, t, rows, D);
     }
+    return e;
 }
 
 // ---------------------------------------------------------------- step product on the tensor cores
@@ -591,6 +597,8 @@ __device__ __forceinline__ void a_operand(const Args<float> &a, int t, uint64_t 
 template <int K>
 __global__ void __launch_bounds__(PREP) operands_kernel(Args<float> a, int t, uint64_t rows, int D, unsigned nw,
                                                         unsigned nrt, unsigned nk) {
+    await_previous();
+    if constexpr (K == 3) release_next();
     const unsigned nx = (unsigned)(a.S / PREP);
     if (blockIdx.x < nw) {
         w_operand<K>(a, t, D, (int)(blockIdx.x % nx), (int)(blockIdx.x / nx), (int)(nw / nx));
@@ -608,6 +616,8 @@ __global__ void __launch_bounds__(PREP) operands_kernel(Args<float> a, int t, ui
 // the accumulator (thread i = row i) and write the rows out.
 template <int K, int NS, int TN>
 __global__ void __launch_bounds__(128, NS == TC_NS ? 2 : 1) ztc_kernel(Args<float> a, int t, uint64_t rows, int D) {
+    await_previous();
+    if constexpr (K == 3) release_next();
     extern __shared__ __align__(1024) unsigned char smem[];
     constexpr int STAGE = tc_stage(TN), BB = TN * TC_KC * 4;
     static_assert(NS <= 8 && NS * STAGE >= 4 * 32 * 36 * 4, "barrier area, epilogue tiles");
@@ -775,8 +785,8 @@ static cudaError_t launch_ztc(const Args<float> &a, int t, uint64_t rows, int D,
     auto go = [&](auto fn, int ns, int tn) {
         const int smem = tc_smem(ns, tn);
         const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess) fn<<<dim3(nrt, (unsigned)(a.S / tn)), 128, smem, st>>>(a, t, rows, D);
-        return e;
+        if (e != cudaSuccess) return e;
+        return launch_next(K == 3, fn, dim3(nrt, (unsigned)(a.S / tn)), 128, (size_t)smem, st, a, t, rows, D);
     };
     if (2 * wide <= (uint64_t)sms) return go(ztc_kernel<K, TC_NS_DEEP, TC_NARROW>, TC_NS_DEEP, TC_NARROW);
     if (wide <= (uint64_t)sms) return go(ztc_kernel<K, TC_NS_DEEP, TC_N>, TC_NS_DEEP, TC_N);
@@ -923,6 +933,8 @@ constexpr int BIAS_W = 16;
 
 template <class R, int K>
 __global__ void __launch_bounds__(32 * BIAS_W) bias_kernel(Args<R> a, int n) {
+    await_previous();
+    if constexpr (K == 3) release_next();
     constexpr int TI = 256 / sizeof(R);  // i per tile
     constexpr int PER = TI / BIAS_W;     // per thread
     __shared__ R cs[2][TI][32], vs[2][TI][32];
@@ -1337,6 +1349,8 @@ __device__ __forceinline__ void p1_row_k45(const Args<R> &a, const Grp<R> &t, in
 // read rows below n only): the p1 warps first, the p+ warps by falling length.
 template <class R, int K, int VW, int U, int WPB>
 __global__ void __launch_bounds__(32 * WPB, 32 / WPB) rows_kernel(Args<R> a, int n) {
+    await_previous();
+    if (K == 3 && n < a.M) release_next();
     const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
     const int item = (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
     if (item < n - 1) {
@@ -1560,6 +1574,12 @@ static dim3 egrid(int S, uint64_t entries) {
     return dim3((unsigned)bx, (unsigned)by);
 }
 
+// Steps of K = 3 are chains of four kernels of 6 to 110 us; chained (launch_next) their
+// gaps go: M = 1152, 256 samples 191.8 -> 184.9 ms a call. At K = 5 (1.6 ms a step, M =
+// 144, 8192 samples) chaining every kernel was 0.6 % slower, 222.9 -> 224.2 ms: blocks
+// in place early keep the kernel before's split of shared memory and first-level cache,
+// which the table walk reads through. K = 4 and 5 stay with ordinary launches.
+//
 // The kernels of step t after its products: VW samples per lane, U loads of a
 // chain ahead, WPB warps per block. Two samples per lane in FP32 and one in FP64,
 // eight loads ahead, two warps: the fastest or within 2 % of it at every size tried
@@ -1570,18 +1590,22 @@ static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
     constexpr int VW = sizeof(R) == 4 ? 2 : 1, U = 8, WPB = 2, NT = 32 * WPB;
     const unsigned gy = (unsigned)(a.S / (32 * VW));
     auto grid = [&](int warps) { return dim3((unsigned)((warps + WPB - 1) / WPB), gy); };
-    if (K == 5 && t > 3) yv_kernel<R, VW, U, WPB><<<grid(t - 3), NT, 0, st>>>(a, t);
-    bias_kernel<R, K><<<(unsigned)(a.S / 32), 32 * BIAS_W, 0, st>>>(a, t);
-    if (K >= 4 && a.opp >= 3 && t > 1) pvv_kernel<R, VW, U, WPB><<<grid(t - 1), NT, 0, st>>>(a, t);
+    cudaError_t e = cudaSuccess;
+    auto next = [&](auto fn, dim3 g, int nt, auto... args) {
+        if (e == cudaSuccess) e = launch_next(K == 3, fn, g, nt, 0, st, a, args...);
+    };
+    if (K == 5 && t > 3) next(yv_kernel<R, VW, U, WPB>, grid(t - 3), NT, t);
+    next(bias_kernel<R, K>, (unsigned)(a.S / 32), 32 * BIAS_W, t);
+    if (K >= 4 && a.opp >= 3 && t > 1) next(pvv_kernel<R, VW, U, WPB>, grid(t - 1), NT, t);
     if (K >= 4 && t > 2) {  // before the p1 rows: fills T
         constexpr int VP = sizeof(R) == 4 ? 4 : 2;
         const unsigned gs = (unsigned)(a.S / (32 * VP)), npairs = (unsigned)cb(a.M - 1, 2);
-        if (a.kb && (t - 1) % P2_NB == 0 && t > 3)  // pairs e < t
-            p2_block_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
-        p2_kernel<R, VP><<<dim3((unsigned)cb(t - 1, 2), gs), 32, 0, st>>>(a, t, npairs);
+        const dim3 pairs((unsigned)cb(t - 1, 2), gs);  // e < t
+        if (a.kb && (t - 1) % P2_NB == 0 && t > 3) next(p2_block_kernel<R, VP>, pairs, 32, t, npairs);
+        next(p2_kernel<R, VP>, pairs, 32, t, npairs);
     }
-    rows_kernel<R, K, VW, U, WPB><<<grid(2 * t - 1), NT, 0, st>>>(a, t);
-    return cudaGetLastError();
+    next(rows_kernel<R, K, VW, U, WPB>, grid(2 * t - 1), NT, t);
+    return e;
 }
 
 template <class R, int K>
@@ -1596,7 +1620,8 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
         if (D > 0) {
             bool tc = false;
             if constexpr (sizeof(R) == 4) tc = a.use_tc != 0;
-            if (!tc) w_kernel<R, K><<<egrid(S, (uint64_t)D), ETB, 0, st>>>(a, t, D);
+            if (!tc) e = launch_next(K == 3, w_kernel<R, K>, egrid(S, (uint64_t)D), ETB, 0, st, a, t, D);
+            if (e != cudaSuccess) return e;
             const uint64_t rows = K == 3   ? 1 + (uint64_t)(M - t)
                                   : K == 4 ? 1 + 2 * (uint64_t)(M - t)
                                            : 1 + 2 * (uint64_t)(M - t) + cb(M - t, 2);
@@ -1606,14 +1631,15 @@ static cudaError_t run_chunk(Args<R> a, double *prob, int sms, cudaStream_t st) 
                     // W: about 5000 blocks, each taking its share of the quads
                     const unsigned nx = (unsigned)(S / PREP), quads = (unsigned)((D + TC_KC - 1) / TC_KC * TC_KC / 4);
                     const unsigned cap = 5000 / nx < 16 ? 16 : 5000 / nx, nw = nx * (quads < cap ? quads : cap);
-                    operands_kernel<K><<<nw + nrt * nk, PREP, 0, st>>>(a, t, rows, D, nw, nrt, nk);
-                    if ((e = launch_ztc<K>(a, t, rows, D, sms, st)) != cudaSuccess) return e;
+                    e = launch_next(K == 3, operands_kernel<K>, nw + nrt * nk, PREP, 0, st, a, t, rows, D, nw, nrt, nk);
+                    if (e == cudaSuccess) e = launch_ztc<K>(a, t, rows, D, sms, st);
                 } else {
-                    launch_zgemm<R, K>(a, t, rows, D, sms, st);
+                    e = launch_zgemm<R, K>(a, t, rows, D, sms, st);
                 }
             } else {
-                launch_zgemm<R, K>(a, t, rows, D, sms, st);
+                e = launch_zgemm<R, K>(a, t, rows, D, sms, st);
             }
+            if (e != cudaSuccess) return e;
         }
         e = step_rows<R, K>(a, t, st);
         if (e != cudaSuccess) return e;
