@@ -47,34 +47,24 @@ WORKLOAD = ("M=144 kmax=5 click-cumulant table: 72 squeezers r~U[0.8,1.6] on mod
             "eta_i~U[0.3,0.5], seed 20251116")
 DTYPE = {"fp64": "f64", "fp32r": "f32 determinant steps refined to f64 accuracy; f64 sums"}
 
-# Executed thread instructions per table entry of each prefix-tree kernel (ncu
-# SASS counters sm__sass_thread_inst_executed_op_{dfma,dadd,dmul,fp32}_pred_on,
+# Executed thread instructions per table entry of the order-4 and order-5 kernels
+# (ncu SASS counters sm__sass_thread_inst_executed_op_{dfma,dadd,dmul,fp32}_pred_on,
 # one counter per capture, divided by the launch's entries; the M=144 kmax=5
-# cumulant call with the tuned schedules pinned: refined 256 x 4, grain 2, 64
-# children; FP64 256 x 2, grain 4, 16 children). They include the amortised
+# cumulant call with the default schedules: refined order 5 in 128 x 6, order 4 in
+# 256 x 3; FP64 order 5 in 256 x 3, order 4 by chunks). They include the amortised
 # per-item Schur-complement build and per-child eliminations. None = not captured
 # for the kernel as it stands.
 OPS_PER_ENTRY = {
-    ("fp32r", 5): {"dfma": 15.021, "dadd": 0.014, "dmul": 0.019, "fp32": 418.24},
-    ("fp32r", 4): {"dfma": 8.013, "dadd": 0.021, "dmul": 1.022, "fp32": 427.87},
-    ("fp64", 5): {"dfma": 36.149, "dadd": 0.001, "dmul": 8.406, "fp32": 4.592},
-    ("fp64", 4): {"dfma": 33.458, "dadd": 0.013, "dmul": 8.375, "fp32": 13.474},
-}
-# The same counts for the slot-free refined form (order 4 of the 256 x 4 shape at
-# grain 2, and order 5 of the slot-free shape): ncu's DFMA and FP32 counters of
-# those kernels; their FP64 arithmetic is the slot kernels', so DADD and DMUL are
-# taken from the rows above.
-OPS_PER_ENTRY_NOSLOT = {
-    ("fp32r", 5): {"dfma": 15.021, "dadd": 0.014, "dmul": 0.019, "fp32": 477.89},
-    ("fp32r", 4): {"dfma": 8.022, "dadd": 0.021, "dmul": 1.022, "fp32": 452.21},
+    ("fp32r", 5): {"dfma": 6.016, "dadd": 2.009, "dmul": 1.014, "fp32": 356.86},
+    ("fp32r", 4): {"dfma": 3.013, "dadd": 4.026, "dmul": 2.026, "fp32": 343.26},
+    ("fp64", 5): {"dfma": 36.138, "dadd": 0.001, "dmul": 8.406, "fp32": 4.417},
+    ("fp64", 4): {"dfma": 35.888, "dadd": 0.030, "dmul": 8.461, "fp32": 13.032},
 }
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of the
 # order-5 kernel at M=144, by precision and CTA shape (gbs_schedule's variant:
-# 6 = 256 x 4 with Schur-complement slots, 9 = 256 x 4 without, 1 = 256 x 2),
-# from ncu captures of the tree kernels with that schedule pinned (mean of the
-# warm-up and timed launches); a shape not listed has no figure (None).
-TRAFFIC_BYTES = {("fp32r", 6): 5.7475e9 + 4.3202e9, ("fp32r", 9): 2.2075e9 + 3.8513e9,
-                 ("fp64", 1): 3.4121e9 + 4.2817e9}
+# 2 = 128 x 6, 4 = 256 x 3), from ncu captures of the calls above; a shape not
+# listed has no figure (None).
+TRAFFIC_BYTES = {("fp32r", 2): 7.447e9 + 4.4696e9, ("fp64", 4): 4.333e9 + 4.3353e9}
 NOMINAL_FP64_FMA_PER_CLK_PER_SM = 2
 NOMINAL_FP32_FMA_PER_CLK_PER_SM = 128
 HBM_FALLBACK_GBS = 6800.0
@@ -188,8 +178,8 @@ def tree_roofline(prec, M, d, kmax, ms, peaks, sms, sm_mhz, hbm):
                     "frac": alg / (ms * 1e-3) / 1e9 / hbm[0]}}
     ops = OPS_PER_ENTRY.get((prec, d))
     v = gbs.schedule(M, kmax, prec)["variant"]
-    if prec == "fp32r" and (v == 9 or (v == 6 and d == 4 and M <= 161)):
-        ops = OPS_PER_ENTRY_NOSLOT.get((prec, d))  # the slot-free form (order 4 of the 256 x 4 shape too)
+    if prec == "fp32r" and (v == 9 or (v in (6, 7) and d == 4)):
+        ops = None  # the slot-free forms rebuild blocks that the counted kernels read
     if ops:
         out.update(pipe_fracs(ops, n, ms, peaks, sms, sm_mhz))
     traffic = order5_traffic(prec, M) if d == 5 else None
@@ -429,7 +419,7 @@ def run_batch(precision, steps, warmup, autotune, peaks, sms, sm_mhz):
                       "l2": "43 GB of outputs per step, far above L2"},
            "schedule": b.schedule(), "autotune_best_ms": b.tune_ms, "gpu_launches": steps,
            "per_instance_fp64": {"ms_per_step": ms_single, "value": N / (ms_single * 1e-3),
-                                 "launches": 6 * len(insts)},
+                                 "launches": sum(1 + max(0, x.kmax - 2) for x in insts)},
            "roofline": roof, "clocks": clk.summary()}
     del b, Vs
     torch.cuda.empty_cache()
@@ -523,7 +513,7 @@ def run_fit(steps, warmup, peaks):
 
 # FP64 pipe instructions (DFMA + DADD + DMUL) and FP32 instructions per entry of
 # the displaced-state order-5 kernel at M=144 (ncu SASS counters); None = not captured.
-DISP_OPS_PER_ENTRY = {"dfma": 56.324, "dadd": 1.001, "dmul": 16.480, "fp32": 5.058}
+DISP_OPS_PER_ENTRY = {"dfma": 56.324, "dadd": 1.001, "dmul": 16.480, "fp32": 5.575}
 
 
 def run_displaced(steps, warmup, peaks, sms, sm_mhz):
@@ -885,7 +875,7 @@ def main():
                 "wall_s_timed": res[head][2],
                 "roofline": headline_roofline(head, M, kmax, res[head][1], peaks, sms, sm_mhz, hbm),
                 "pipe_peaks_measured": peaks, "hbm_peak": {"gbs": hbm[0], "source": hbm[1]},
-                "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 6 * args.steps, "clocks": clocks}
+                "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 4 * args.steps, "clocks": clocks}  # orders 1-2, 3, 4, 5
         for p in precs[1:]:
             line[f"{p}_path"] = {"value": replica_value(N, args.steps, world, tot[p]), "unit": "subsets/s",
                                  "ms_per_step": tot[p] / args.steps, "dtype": DTYPE[p],
