@@ -431,9 +431,9 @@ def run_batch(precision, steps, warmup, autotune, peaks, sms, sm_mhz):
 # FP64 flops (FMA = 2), FP64-pipe instructions, FP32 instructions; None = not
 # captured (or stale after a kernel change).
 FIT_PHASE_COUNTS = {
-    "p0_recompute": {"fp64_flops": 34599015, "fp64_instr": 22408520, "fp32_instr": 1701487776},
-    "h_table": {"fp64_flops": 2293700, "fp64_instr": 1146850, "fp32_instr": 3758700},
-    "gp0_gather": {"fp64_flops": 118296845, "fp64_instr": 62419595, "fp32_instr": 9289756},
+    "p0_recompute": {"fp64_flops": 21461133, "fp64_instr": 13767002, "fp32_instr": 1145365972},
+    "h_table": {"fp64_flops": 5047450, "fp64_instr": 3097150, "fp32_instr": 3758700},
+    "gp0_gather": {"fp64_flops": 118298125, "fp64_instr": 62420875, "fp32_instr": 17132462},
     "gv_scatter": {"fp64_flops": 220049841, "fp64_instr": 179690437, "fp32_instr": 8485702640},
 }
 
