@@ -12,10 +12,10 @@
 //   P0(S) / P0(S') = det(Sch_j)^{-1/2} = r0 (1 + eta),
 // r0 the FP32 reciprocal square root and eta its residual's correction (eta also
 // carries the low part of the determinant: one step of refinement to FP64
-// accuracy). About 230 FP32 instructions a leaf; an FP32 Cholesky step with its
-// residual by error-free transformations and the second-order expansion of
-// log det(I + G), the form before, took 375 and lost more in the expansion's FP32
-// terms (P0 relative error 2.0e-13 at most at M = 144, 6.6e-14 now).
+// accuracy). Bound by FP32 issue, about 240 instructions a leaf. The block's three
+// sums are normalised before the determinant (9 of them; M = 144, kmax = 5: 10.56 ->
+// 10.72 ms the call): without that, P0 of two-mode squeezed pairs was off by 1.0e-10
+// at r = 3, with it by 1.6e-12 (M = 8 to 66, relative, largest).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -180,7 +180,10 @@ __device__ __forceinline__ void refined_leaf_factor(ABlk S, const DFBlk &z2, con
     acc_sub_row(S, z2.a00, z2.a01, zj.a00, zj.a01);
     acc_sub_row(S, z2.a10, z2.a11, zj.a10, zj.a11);
     const ASym sch = acc_sub_gram(d, pivot_rows(S, pv));
-    const DF a{sch.s00.s, sch.s00.t}, b{sch.s01.s, sch.s01.t}, c{sch.s11.s, sch.s11.t};
+    // normalised first: where the elimination cancels (j's two-mode squeezed partner in
+    // the prefix) the remainders are not small beside the leading parts, and the
+    // products below drop what is of second order in them
+    const DF a = acc_norm(sch.s00), b = acc_norm(sch.s01), c = acc_norm(sch.s11);
     // det = a c - b^2 (a c >= b^2: the fast two-sum is exact)
     const DF p = df_mulu(a, c);
     const float q = b.h * b.h;
