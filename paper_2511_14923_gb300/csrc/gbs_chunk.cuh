@@ -13,6 +13,8 @@
 namespace gbs {
 
 constexpr int CHUNK_THREADS = 128;
+// Dynamic shared memory a chunk may take: 227 KB less the kernel's static part.
+constexpr size_t kChunkSmem = 226 * 1024;
 
 // Shared memory: doubles per mode x <= max c2 and per row c2 of the chunk.
 template <int NP, int PREC, bool DISP>
@@ -287,8 +289,11 @@ template <int NP, int MODE, int PREC, bool DISP>
 static cudaError_t launch_chunk(const FwdArgs &a, bool write_p0, int c_lo, int c_hi, uint32_t L, size_t smem,
                                 cudaStream_t st) {
     auto fn = chunk_kernel<NP, MODE, PREC, DISP>;
-    if (smem > 40 * 1024) {  // the static part takes a little of the 48 KB that need no opt-in
-        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the static part takes a little of the 48 KB that need no opt-in. The limit belongs
+    // to the kernel, not to this call: every call sets the same one, so that no host
+    // thread lowers it between another's two calls
+    if (smem > 40 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChunkSmem);
         if (e != cudaSuccess) return e;
     }
     const int hi = c_hi - 1, lo = c_lo > NP + 1 ? c_lo : NP + 1;  // largest and smallest top element

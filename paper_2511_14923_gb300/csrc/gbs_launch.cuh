@@ -12,8 +12,6 @@ namespace gbs {
 // chunk: one chunk a prefix up to 182 modes.
 constexpr int kOrder4ChunkedZ = 224, kOrder4ChunkedR = 64;
 constexpr uint32_t kOrder4Pairs = 16384;
-// Shared memory a chunk may take: 227 KB less the kernel's static part.
-constexpr size_t kChunkSmem = 226 * 1024;
 
 // Packing of A, order 1 and order 2 in one launch (none reads what another writes):
 // blocks [0, nb0) pack, [nb0, nb0 + nb1) fill order 1, the rest order 2; one thread
