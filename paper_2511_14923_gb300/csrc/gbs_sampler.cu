@@ -233,6 +233,16 @@ __device__ __forceinline__ void zrow(int K, int M, int t, uint64_t q, const uint
     }
 }
 
+// Blocks with the samples on the slow grid axis: y, and z beyond the 65535 blocks y
+// may have (FP64 batches of 2^21, 32 samples a block). The number of blocks, a
+// multiple of 4 (S is one of 128), halves evenly.
+static dim3 sample_grid(unsigned x, unsigned blocks) {
+    unsigned z = 1;
+    for (; blocks > 65535; blocks /= 2) z *= 2;
+    return dim3(x, blocks, z);
+}
+__device__ __forceinline__ int sample_block() { return (int)(blockIdx.z * gridDim.y + blockIdx.y); }
+
 // W_t[r][s], the inner operand of the step-t product: K = 5, pair r = (e, d) of
 // bits below t, chi_e chi_d P2~[t-1][e][d]; K = 3, d = r + 1, chi_d P1~[t-1][d].
 // Grid: (samples / ETB, entries); the entry index is uniform in a block.
@@ -300,7 +310,7 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
     __shared__ uint64_t dst[BT];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const uint64_t m0 = (uint64_t)blockIdx.x * BT;
-    const int s0 = blockIdx.y * BT;
+    const int s0 = sample_block() * BT;
     for (int m = tid; m < BT; m += 256) {
         const uint64_t q = m0 + m;
         if (q < rows) zrow(K, a.M, t, q, a.off, a.o, kb[m], dst[m]);
@@ -380,7 +390,7 @@ __global__ void __launch_bounds__(256) zgemm_kernel(Args<R> a, int t, uint64_t r
 template <class R, int K>
 static cudaError_t launch_zgemm(const Args<R> &a, int t, uint64_t rows, int D, int sms, cudaStream_t st) {
     auto ctas = [&](int bt) { return (rows + bt - 1) / bt * (uint64_t)(a.S / bt); };
-    auto grid = [&](int bt) { return dim3((unsigned)((rows + bt - 1) / bt), (unsigned)(a.S / bt)); };
+    auto grid = [&](int bt) { return sample_grid((unsigned)((rows + bt - 1) / bt), (unsigned)(a.S / bt)); };
     cudaError_t e;
     if constexpr (sizeof(R) == 4) {
         if (ctas(128) >= 2 * (uint64_t)sms) e = launch_next(K == 3, zgemm_kernel<R, K, 8>, grid(128), 256, 0, st, a, t, rows, D);
@@ -902,7 +912,7 @@ template <class R, int VW, int U, int WPB>
 __global__ void __launch_bounds__(32 * WPB) yv_kernel(Args<R> a, int n) {
     const int i = 3 + (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
     if (i >= n) return;
-    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    const Grp<R> t(a, sample_block() * (32 * VW) + (int)(threadIdx.x & 31) * VW);
     Lanes<R, VW> y = ldl<R, VW>(t.Z + i_z(i, n) * SG);
     const R *z5 = t.Z5 + i_z5(0, i, n) * SG, *q = t.Pp + (size_t)c2u(i - 1) * SG;  // Z5_j(i, n) and Pp~[i-1][j+1] at j
     struct Three {
@@ -1032,7 +1042,7 @@ template <class R, int VW, int U, int WPB>
 __global__ void __launch_bounds__(32 * WPB) pvv_kernel(Args<R> a, int n) {
     const int j = 1 + (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
     if (j >= n) return;
-    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    const Grp<R> t(a, sample_block() * (32 * VW) + (int)(threadIdx.x & 31) * VW);
     const R *k3n = a.kap + a.off[3] + cb(n - 1, 3) + (j - 1);  // kappa(j, i, n) at C(i-1, 2)
     Lanes<R, VW> v;
 #pragma unroll
@@ -1351,7 +1361,7 @@ template <class R, int K, int VW, int U, int WPB>
 __global__ void __launch_bounds__(32 * WPB, 32 / WPB) rows_kernel(Args<R> a, int n) {
     await_previous();
     if (K == 3 && n < a.M) release_next();
-    const Grp<R> t(a, (int)blockIdx.y * (32 * VW) + (int)(threadIdx.x & 31) * VW);
+    const Grp<R> t(a, sample_block() * (32 * VW) + (int)(threadIdx.x & 31) * VW);
     const int item = (int)blockIdx.x * WPB + (int)(threadIdx.x >> 5);
     if (item < n - 1) {
         if constexpr (K == 3) p1_row_k3<R, VW, U>(a, t, n, 1 + item);
@@ -1589,7 +1599,7 @@ template <class R, int K>
 static cudaError_t step_rows(const Args<R> &a, int t, cudaStream_t st) {
     constexpr int VW = sizeof(R) == 4 ? 2 : 1, U = 8, WPB = 2, NT = 32 * WPB;
     const unsigned gy = (unsigned)(a.S / (32 * VW));
-    auto grid = [&](int warps) { return dim3((unsigned)((warps + WPB - 1) / WPB), gy); };
+    auto grid = [&](int warps) { return sample_grid((unsigned)((warps + WPB - 1) / WPB), gy); };
     cudaError_t e = cudaSuccess;
     auto next = [&](auto fn, dim3 g, int nt, auto... args) {
         if (e == cudaSuccess) e = launch_next(K == 3, fn, g, nt, 0, st, a, args...);
