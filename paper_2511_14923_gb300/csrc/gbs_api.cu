@@ -27,6 +27,9 @@ cudaEvent_t g_bev[5];
 bool g_bev_ready = false;
 
 int fail(int code, const char *fmt, ...) {
+    // a failed runtime call is reported here: not once more by the next call's check
+    // of its launches (or by the caller's own)
+    if (code == GBS_ERR_CUDA) cudaGetLastError();
     va_list ap;
     va_start(ap, fmt);
     vsnprintf(g_err, sizeof g_err, fmt, ap);
@@ -152,7 +155,9 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
         a.ev = g_ev;
         g_timing_used = true;
     }
-    e = mean ? gbs::launch_forward_displaced(a, st) : gbs::launch_forward(a, st);
+    e = gbs::fault_injected("forward_launch") ? cudaSetDevice(-1)
+        : mean                                ? gbs::launch_forward_displaced(a, st)
+                                              : gbs::launch_forward(a, st);
     if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));
     return ok();
 }

@@ -227,7 +227,8 @@ inline cudaError_t launch_next(bool chained, void (*fn)(P...), dim3 grid, dim3 b
 // Host-side fault injection, for tests of the error paths: true when the
 // environment variable GBS_FAULT_INJECT lists `site` (comma-separated names).
 // Sites: "forward_memset" (the forward calls' first runtime call is treated as
-// failed, GBS_ERR_CUDA), "sampler_no_loads" (the sampler's tensor-core step
+// failed, GBS_ERR_CUDA), "forward_launch" (a runtime call that the host refuses, a
+// device index of -1, in the place of their launches), "sampler_no_loads" (the sampler's tensor-core step
 // product issues no copies and gives up its first wait quickly, so the call
 // reports GBS_ERR_TIMEOUT with nothing in flight). Nothing faults on the GPU.
 inline bool fault_injected(const char *site) {
