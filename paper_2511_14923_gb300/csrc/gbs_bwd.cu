@@ -260,8 +260,14 @@ __device__ __forceinline__ double gather_walk(int M, const Offsets &o, const int
     return ((BB + R) & 1) ? -t : t;
 }
 
-// gP0 of the order-BB subsets by one block of GATHER_THREADS.
-constexpr int GATHER_THREADS = 1024;
+// gP0 of the order-BB subsets by one block of GATHER_THREADS: GATHER_THREADS / team
+// of them. (A whole block for every team wider than a warp would leave most of it
+// without units: a team is sized for four a lane, 64 lanes at 129 to 256 of them. M =
+// 144, kmax = 4 3.50 -> 0.84 ms, kmax = 5 195 -> 51.) A block holds its places until
+// its longest walk ends: 512 threads against 1024 M = 100, kmax = 4 227 -> 204 us,
+// kmax = 5 9.13 -> 8.01 ms; 256, whose teams are too narrow for order 1, M = 30 and 48,
+// kmax = 5 53 -> 74 and 254 -> 332 us.
+constexpr int GATHER_THREADS = 512;
 template <int BB>
 __device__ __forceinline__ void gather_block(int M, int kmax, const Offsets &o, const double *__restrict__ gk,
                                              const double *__restrict__ h, double *__restrict__ gp0, int team,
@@ -305,13 +311,14 @@ __device__ __forceinline__ void gather_block(int M, int kmax, const Offsets &o, 
     for (int off = w / 2; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off, w);
     if (team <= 32) {
         if (live && lane == 0) gp0[o.off[BB] + unit_b] = acc;
-    } else {  // one team per block
-        __shared__ double red[32];
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    } else {  // several warps a team
+        __shared__ double red[GATHER_THREADS / 32];
+        const int warp = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0) red[warp] = acc;
         __syncthreads();
-        if (threadIdx.x == 0 && live) {
+        if (lane == 0 && live) {
             double tot = 0.0;
-            for (int k = 0; k < team / 32; ++k) tot += red[k];
+            for (int k = 0; k < team / 32; ++k) tot += red[warp + k];
             gp0[o.off[BB] + unit_b] = tot;
         }
     }
@@ -319,17 +326,16 @@ __device__ __forceinline__ void gather_block(int M, int kmax, const Offsets &o, 
 
 // gP0 of every order in one launch: the orders don't read each other, and each by
 // itself leaves much of the GPU waiting for its gathers (M = 100, kmax = 4: 92, 125,
-// 60 and 13 us one after the other, 226 together). Blocks of order 1 first (the
+// 60 and 13 us one after the other, 204 together). Blocks of order 1 first (the
 // longest walks), then 2, 3, 4; the top order (only R = empty contributes, gP0(B) =
 // g_y(B)) last.
 struct GatherPlan {
     unsigned end[GBS_MAX_ORDER];  // end[b - 1] = one past the last block of order b < kmax
     int team[GBS_MAX_ORDER];
 };
-__global__ void __launch_bounds__(GATHER_THREADS) gather_kernel(int M, int kmax, Offsets o,
-                                                                const double *__restrict__ gk,
-                                                                const double *__restrict__ h,
-                                                                double *__restrict__ gp0, GatherPlan pl) {
+__global__ void __launch_bounds__(GATHER_THREADS, 1024 / GATHER_THREADS)
+    gather_kernel(int M, int kmax, Offsets o, const double *__restrict__ gk, const double *__restrict__ h,
+                  double *__restrict__ gp0, GatherPlan pl) {
     const unsigned b = blockIdx.x;
     if (b >= pl.end[GBS_MAX_ORDER - 2]) {
         const uint64_t i = (uint64_t)(b - pl.end[GBS_MAX_ORDER - 2]) * GATHER_THREADS + threadIdx.x;
@@ -820,7 +826,6 @@ cudaError_t launch_backward(const BwdArgs &a, cudaStream_t st) {
                 for (int q = 0; q < K - b; ++q) units += binom(M - b, q);
                 int team = 1;
                 while (team < GATHER_THREADS && 4 * (uint64_t)team < units) team *= 2;
-                if (team > 32) team = GATHER_THREADS;  // a team wider than a warp is a whole block
                 pl.team[b - 1] = team;
                 blocks += (unsigned)((binom(M, b) * team + GATHER_THREADS - 1) / GATHER_THREADS);
             }
