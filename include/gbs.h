@@ -96,7 +96,10 @@ uint64_t gbs_rank(const int *modes, int d);
 int gbs_unrank(uint64_t r, int d, int *modes_out);
 
 /* Workspace bytes needed by any compute call with these (M, kmax, precision) on
-   the current CUDA device; 0 if the arguments are invalid. */
+   the current CUDA device; 0 if the arguments are invalid. GBS_FP32_REFINED with
+   kmax >= 4 takes 16 bytes more for each entry of the orders below kmax, which the
+   cumulant tables read; given a workspace of the GBS_FP64 size, a refined cumulant
+   call fills its table by the FP64 kernels (the other refined calls need no more). */
 size_t gbs_workspace_bytes(int M, int kmax, int precision);
 
 /* Message for the most recent failing call on this host thread ("" if none). */

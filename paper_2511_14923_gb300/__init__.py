@@ -196,15 +196,17 @@ class Workspace:
         return int(lib().gbs_stream_status(ctypes.c_void_p(self.ptr), ctypes.c_void_p(st.cuda_stream)))
 
 
-def _workspace_for(workspace, M: int, kmax: int, precision: str, device) -> Workspace:
+def _workspace_for(workspace, M: int, kmax: int, precision: str, device, least: str | None = None) -> Workspace:
     """The caller's Workspace after checking that it sits on the inputs' device and
-    is large enough for (M, kmax, precision), or a new one."""
+    is large enough for (M, kmax, precision), or a new one. least: the precision whose
+    size is enough for a caller's workspace, if not that one."""
     if workspace is None:
         return Workspace(M, kmax, precision, device=device)
     if not isinstance(workspace, Workspace):
         raise TypeError("workspace must be a Workspace")
     if workspace.buf.device != torch.device(device):
         raise ValueError(f"workspace is on {workspace.buf.device}, the inputs on {device}")
+    precision = least or precision
     need = workspace_bytes(M, kmax, precision)
     if workspace.nbytes < need:
         raise GbsError(5, f"workspace holds {workspace.nbytes} bytes, (M={M}, kmax={kmax}, {precision}) needs {need}")
@@ -257,7 +259,7 @@ def _forward(fname: str, V: torch.Tensor, kmax: int, precision: str, out, worksp
     elif out.numel() != n or out.dtype != torch.float64 or not out.is_cuda or not out.is_contiguous():
         raise ValueError(f"out must be a contiguous CUDA float64 tensor of {n} entries")
     _on(out, V.device, "out")
-    ws = _workspace_for(workspace, M, kmax, precision, V.device)
+    ws = _workspace_for(workspace, M, kmax, precision, V.device, least="fp64")
     st = torch.cuda.current_stream(V.device)
     f = getattr(lib(), fname)
     _check(f(ctypes.c_void_p(V.data_ptr()), M, kmax, ctypes.c_void_p(out.data_ptr()), PRECISIONS[precision],
@@ -350,7 +352,8 @@ def table_range(V, kmax, c_lo, c_hi, table="kappa", precision="fp64", out=None, 
     elif out.numel() < n or out.dtype != torch.float64 or not out.is_cuda or not out.is_contiguous():
         raise ValueError(f"out must be a contiguous CUDA float64 tensor of at least {n} entries")
     _on(out, V.device, "out")
-    nb = int(lib().gbs_range_workspace_bytes(M, kmax, PRECISIONS[precision]))
+    # (a caller's workspace may have the FP64 size, as for whole tables)
+    nb = int(lib().gbs_range_workspace_bytes(M, kmax, PRECISIONS[precision if workspace is None else "fp64"]))
     if nb == 0:
         raise GbsError(1, f"invalid (M={M}, kmax={kmax}, precision={precision})")
     ws = _workspace_tensor(workspace, nb, V.device)

@@ -70,8 +70,14 @@ size_t range_total(const gbs::WsLayout &L, int M, int kmax) {
     return L.total + ((sizeof(double) * (size_t)gbs::order_offset(M, kmax) + 255) & ~(size_t)255);
 }
 
-int check_common(const double *V, int M, int kmax, const void *out, int precision, void *ws, size_t ws_bytes,
-                 gbs::WsLayout &L, int &sms, bool range = false) {
+// True for the calls that keep the lower orders as float pairs as well (gbs_tree.cuh).
+bool uses_pairs(int mode, int kmax, int precision) {
+    return precision == GBS_FP32_REFINED && kmax >= 4 && (mode == gbs::MODE_KAPPA || mode == gbs::MODE_SPINK);
+}
+
+// least: accept a workspace without room for the float pairs too (L then has none).
+int check_common(const double *V, int M, int kmax, const void *out, int precision, int mode, void *ws,
+                 size_t ws_bytes, gbs::WsLayout &L, int &sms, bool range, bool least) {
     if (!valid_mk(M, kmax)) return fail(GBS_ERR_INVALID_ARG, "%s", gbs::shape_message(M, kmax).c_str());
     if (precision != GBS_FP64 && precision != GBS_FP32_REFINED)
         return fail(GBS_ERR_INVALID_ARG, "precision must be GBS_FP64 (0) or GBS_FP32_REFINED (1); got %d", precision);
@@ -83,10 +89,14 @@ int check_common(const double *V, int M, int kmax, const void *out, int precisio
         return fail(GBS_ERR_INVALID_ARG, "V, output and workspace must be CUDA device (or managed) memory");
     sms = device_sms();
     if (sms <= 0) return fail(GBS_ERR_CUDA, "no CUDA device is current");
-    L = gbs::ws_layout(M, kmax, sms);
-    const size_t need = range ? range_total(L, M, kmax) : L.total;
-    if (ws_bytes < need)
-        return fail(GBS_ERR_WORKSPACE, "workspace too small: %zu bytes given, %zu needed", ws_bytes, need);
+    bool pairs = uses_pairs(mode, kmax, precision);
+    auto need = [&] {
+        L = gbs::ws_layout(M, kmax, sms, 0, pairs);
+        return range ? range_total(L, M, kmax) : L.total;
+    };
+    if (ws_bytes < need() && pairs && least) pairs = false;
+    if (ws_bytes < need())
+        return fail(GBS_ERR_WORKSPACE, "workspace too small: %zu bytes given, %zu needed", ws_bytes, need());
     return GBS_OK;
 }
 
@@ -103,8 +113,10 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
     if (range.on() && (range.c_lo < 0 || range.c_lo > range.c_hi || range.c_hi > M))
         return fail(GBS_ERR_INVALID_ARG, "need 0 <= c_lo <= c_hi <= M; got c_lo=%d c_hi=%d M=%d", range.c_lo,
                     range.c_hi, M);
-    int rc = check_common(V, M, kmax, out, precision, ws, ws_bytes, L, sms, range.on());
+    int rc = check_common(V, M, kmax, out, precision, mode, ws, ws_bytes, L, sms, range.on(), true);
     if (rc != GBS_OK) return rc;
+    // a workspace of the FP64 size: the table by the FP64 kernels, which need no pairs
+    if (uses_pairs(mode, kmax, precision) && L.p0p_off == L.total) precision = GBS_FP64;
     if (mean && (((uintptr_t)mean & 7) || !is_device_ptr(mean)))
         return fail(GBS_ERR_INVALID_ARG, "mean must be 8-byte aligned CUDA device (or managed) memory");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -122,7 +134,7 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
     a.precision = precision;
     a.A = reinterpret_cast<double *>(w + L.A_off);
     a.Af = reinterpret_cast<float *>(a.A + 4 * (size_t)M * M);
-    if (precision == GBS_FP32_REFINED && kmax >= 4 && (mode == gbs::MODE_KAPPA || mode == gbs::MODE_SPINK)) {
+    if (uses_pairs(mode, kmax, precision)) {
         a.p0p = reinterpret_cast<float2 *>(w + L.p0p_off);
         a.kyp = reinterpret_cast<float2 *>(w + L.kyp_off);
     }
@@ -220,7 +232,7 @@ int gbs_unrank(uint64_t r, int d, int *modes_out) {
 size_t gbs_workspace_bytes(int M, int kmax, int precision) {
     if (!valid_mk(M, kmax) || (precision != GBS_FP64 && precision != GBS_FP32_REFINED)) return 0;
     const int sms = device_sms();
-    return gbs::ws_layout(M, kmax, sms > 0 ? sms : 1).total;
+    return gbs::ws_layout(M, kmax, sms > 0 ? sms : 1, 0, precision == GBS_FP32_REFINED).total;
 }
 
 const char *gbs_last_error(void) { return g_err; }
@@ -464,7 +476,7 @@ int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precis
                  size_t ws_bytes, void *cuda_stream, float *best_ms_out) {
     gbs::WsLayout L;
     int sms = 0;
-    int rc = check_common(V, M, kmax, kappa_out, precision, workspace, ws_bytes, L, sms);
+    int rc = check_common(V, M, kmax, kappa_out, precision, gbs::MODE_KAPPA, workspace, ws_bytes, L, sms, false, false);
     if (rc != GBS_OK) return rc;
     char *w = static_cast<char *>(workspace);
     gbs::FwdArgs a{};
@@ -475,7 +487,7 @@ int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precis
     a.precision = precision;
     a.A = reinterpret_cast<double *>(w + L.A_off);
     a.Af = reinterpret_cast<float *>(a.A + 4 * (size_t)M * M);
-    if (precision == GBS_FP32_REFINED && kmax >= 4) {
+    if (uses_pairs(a.mode, kmax, precision)) {
         a.p0p = reinterpret_cast<float2 *>(w + L.p0p_off);
         a.kyp = reinterpret_cast<float2 *>(w + L.kyp_off);
     }
@@ -540,7 +552,7 @@ int gbs_spin_cumulants(const double *V, int M, int kmax, double *kappa_out, int 
 size_t gbs_range_workspace_bytes(int M, int kmax, int precision) {
     if (!valid_mk(M, kmax) || (precision != GBS_FP64 && precision != GBS_FP32_REFINED)) return 0;
     const int sms = device_sms();
-    return range_total(gbs::ws_layout(M, kmax, sms > 0 ? sms : 1), M, kmax);
+    return range_total(gbs::ws_layout(M, kmax, sms > 0 ? sms : 1, 0, precision == GBS_FP32_REFINED), M, kmax);
 }
 
 uint64_t gbs_range_entries(int M, int kmax, int c_lo, int c_hi) {

@@ -62,7 +62,7 @@ WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm, bool pairs) {
     // the reduced half-means of a displaced state
     w.slot_doubles = 4 * ((size_t)binom2(M) + (size_t)M) + 2 * (size_t)M;
     if (kmax >= 4) off = align256(off + sizeof(double) * w.slot_doubles * w.slots);
-    w.p0p_off = off;  // any precision: one workspace serves both
+    w.p0p_off = off;  // last, so that the layout without them is the first part of the other
     if (pairs && kmax >= 4) off = align256(off + sizeof(float2) * (size_t)np0);
     w.kyp_off = off;
     if (pairs && kmax >= 4) off = align256(off + sizeof(float2) * (size_t)np0);

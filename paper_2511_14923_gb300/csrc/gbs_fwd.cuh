@@ -145,7 +145,7 @@ inline int slots_per_sm_for(int M) { return M <= kVariant2MaxM ? 6 : M <= kVaria
 // Reserves slots_per_sm scratch slots per multiprocessor (0 = slots_per_sm_for(M);
 // with one, only one CTA per multiprocessor runs).
 // pairs: with the float-pair tables of refined cumulant calls (kmax >= 4).
-WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm = 0, bool pairs = true);
+WsLayout ws_layout(int M, int kmax, int sms, int slots_per_sm, bool pairs);
 
 // Queues every kernel of one forward call on stream; returns a cudaError_t.
 cudaError_t launch_forward(const FwdArgs &a, cudaStream_t stream);
