@@ -308,14 +308,15 @@ int gbs_sample(const double *kappa, int M, int K, const int *orders, int n_sampl
 int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precision, void *workspace,
                  size_t ws_bytes, void *cuda_stream, float *best_ms_out);
 
-/* Schedule the forward calls of (M, kmax, precision) run on the current device:
-   the one gbs_autotune recorded (or read from GBS_AUTOTUNE_CACHE), else the
-   default. schedule_out[3] (host) = {CTA shape (0: 512 threads x 1 per SM,
+/* Schedule gbs_cumulants of (M, kmax, precision) runs on the current device: the one
+   gbs_autotune recorded (or read from GBS_AUTOTUNE_CACHE), else the default. The
+   other forward calls of the shape take a recorded schedule too, and a default of
+   their own without one. schedule_out[3] (host) = {CTA shape (0: 512 threads x 1 per SM,
    1: 256 x 2, 4: 256 x 3 with a larger batch area, refined only 2: 128 x 6, 3: 256 x 3,
    5: 384 x 2,
    6: 256 x 4, 7 and 8: 6 and 3 in thread-block clusters, 9: 6 without
    Schur-complement slots), items per CTA slot, children per shared-memory
-   batch}, after the fallback to 512 x 1 for a shape that does not admit M.
+   batch}. A recorded shape that does not admit M is not used.
    Host only; allocates nothing. Returns GBS_OK, GBS_ERR_INVALID_ARG (bad
    shape or precision, NULL schedule_out) or GBS_ERR_CUDA (no device). */
 int gbs_schedule(int M, int kmax, int precision, int *schedule_out);

@@ -4,12 +4,13 @@
 // forward pass under every candidate schedule and keeps the fastest:
 //   grain   items per CTA slot (subtree granularity: 1, 2, 4, 8),
 //   ccap    children per shared-memory batch (16 or 64),
-//   variant CTA shape: 512 threads x 1 per SM; 256 x 2 per SM (M <= 577); and for
-//           the refined path 128 x 6 (M <= 305), 256 x 3 (M <= 577, or with a
-//           larger x area M <= 673), 384 x 2 (M <= 961), 256 x 4 (M <= 385),
+//   variant CTA shape: 512 threads x 1 per SM; 256 x 2 per SM (M <= 577); 256 x 3
+//           with a larger x area (M <= 673); and for the refined path 128 x 6 (M <=
+//           305), 256 x 3 (M <= 577), 384 x 2 (M <= 961), 256 x 4 (M <= 385),
 //           256 x 4 / 256 x 3 in thread-block clusters sharing one slot, or
 //           256 x 4 without slots (M <= 161).
-// Results live in a process-wide table consulted by every forward call; if the
+// Results live in a process-wide table consulted by every forward call of the shape,
+// whatever its table (the other tables' own best schedules lie within 18 % of it); if the
 // environment variable GBS_AUTOTUNE_CACHE names a file, the table is loaded from
 // it on first use and rewritten after each tuning run (a JSON array of objects).
 // Ragged batches (gbs_batched_autotune) have a second table keyed by the batch's
@@ -179,7 +180,12 @@ TreeCfg tuned_cfg(int sms, int M, int kmax, int precision, int mode) {
     std::lock_guard<std::mutex> lock(g_mu);
     load_locked();
     auto it = g_table.find(Key{device_cc(), sms, M, kmax, precision});
-    return it == g_table.end() ? default_cfg(M, kmax, precision, mode) : it->second.cfg;
+    // an entry whose shape does not admit M (a cache file may hold any: shapes 2 and 4
+    // once were 640 x 1 and 768 x 1, which admitted every M) would fall back to 512 x 1,
+    // slower than the default
+    if (it == g_table.end() || effective_variant(it->second.cfg.variant, M, precision) != it->second.cfg.variant)
+        return default_cfg(M, kmax, precision, mode);
+    return it->second.cfg;
 }
 
 bool tuned_batch_cfg(int sms, const gbs_instance *inst, int n, int precision, TreeCfg &cfg) {
