@@ -453,7 +453,9 @@ int gbs_covariance(const double *U_re, const double *U_im, const double *r, cons
     for (const void *p : ptrs)
         if (!p || ((uintptr_t)p & 7) || !is_device_ptr(p))
             return fail(GBS_ERR_INVALID_ARG, "all arrays must be non-NULL, 8-byte aligned device memory");
-    cudaError_t e = gbs::launch_covariance(U_re, U_im, r, eta, M, V_out, static_cast<cudaStream_t>(cuda_stream));
+    const int sms = device_sms();
+    if (sms <= 0) return fail(GBS_ERR_CUDA, "no CUDA device is current");
+    cudaError_t e = gbs::launch_covariance(U_re, U_im, r, eta, M, V_out, sms, static_cast<cudaStream_t>(cuda_stream));
     if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));
     return ok();
 }

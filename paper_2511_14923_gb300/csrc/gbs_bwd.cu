@@ -1006,13 +1006,13 @@ __global__ void covariance_bwd_kernel(const double *Ur, const double *Ui, const 
 }
 
 cudaError_t launch_covariance(const double *Ur, const double *Ui, const double *r, const double *eta, int M, double *V,
-                              cudaStream_t st) {
+                              int sms, cudaStream_t st) {
     auto tiles = [&](int t) {
         const int nt = (2 * M + t - 1) / t;
         return nt * (nt + 1) / 2;
     };
-    // four wide tiles for each of 152 multiprocessors: the last wave then costs little
-    if (tiles(32) >= 4 * 152) covariance_kernel<32><<<tiles(32), 256, 0, st>>>(Ur, Ui, r, eta, M, V);
+    // four wide tiles for each multiprocessor: the last wave then costs little
+    if (tiles(32) >= 4 * sms) covariance_kernel<32><<<tiles(32), 256, 0, st>>>(Ur, Ui, r, eta, M, V);
     else covariance_kernel<16><<<tiles(16), 256, 0, st>>>(Ur, Ui, r, eta, M, V);
     return cudaGetLastError();
 }

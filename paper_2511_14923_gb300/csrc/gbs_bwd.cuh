@@ -24,7 +24,7 @@ struct BwdArgs {
 
 cudaError_t launch_backward(const BwdArgs &a, cudaStream_t st);
 cudaError_t launch_covariance(const double *Ur, const double *Ui, const double *r, const double *eta, int M, double *V,
-                              cudaStream_t st);
+                              int sms, cudaStream_t st);
 cudaError_t launch_covariance_bwd(const double *Ur, const double *Ui, const double *r, const double *eta, int M,
                                   const double *V, const double *G, double *dr, double *deta, cudaStream_t st);
 
