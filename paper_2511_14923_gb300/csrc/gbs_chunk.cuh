@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(CHUNK_THREADS, DISP ? 4 : 6)
 // Shared-memory bytes of chunks of L pairs below the top mode c3 = top: PX doubles
 // per mode up to the chunk's largest c2, PR per row of it. A chunk that starts at
 // c2 = 1 touches about sqrt(2 L) rows; one that ends in the upper half has few.
-inline size_t chunk_smem(int top, uint32_t L, int px, int pr) {
+constexpr size_t chunk_smem(int top, uint32_t L, int px, int pr) {
     size_t rows = 2;
     while (rows * (rows - 1) / 2 < L && rows < (size_t)top) ++rows;
     rows += 2;

@@ -21,7 +21,7 @@ struct FwdArgs {
     double *A;            // packed 2x2 blocks of (V+I)/2, M*M*4 doubles (workspace)
     float *Af;            // the same blocks as float pairs (hi x4, lo x4), refined path (workspace)
     // refined cumulant calls with kmax >= 4: the lower orders' P0 and no-click cumulants
-    // ky (gbs_tree.cuh, combine_pairs) as float pairs (workspace; null otherwise)
+    // ky (gbs_tree.cuh, combine_products) as float pairs (workspace; null otherwise)
     float2 *p0p, *kyp;
     double *p0;           // P0 table: the output for MODE_P0, a workspace table (orders < kmax) otherwise
     double *out;          // mu or kappa table (MODE_MU / MODE_KAPPA); equals p0 for MODE_P0
@@ -47,7 +47,7 @@ struct FwdArgs {
 
 // Valid (M, kmax) of a forward table: orders 4 and 5 run the prefix-tree kernels
 // (shared-memory x-entries sized for GBS_MAX_MODES); tables with kmax <= 3 run
-// one thread per subset and take up to GBS_MAX_MODES_K3 modes.
+// order 3 by chunks and take up to GBS_MAX_MODES_K3 modes.
 inline bool valid_mk(int M, int kmax) {
     return M >= 1 && kmax >= 1 && kmax <= 5 && kmax <= M && M <= (kmax <= 3 ? 4096 : 1024);
 }
@@ -78,7 +78,8 @@ constexpr int kVariant5MaxM = kPairXC + 1;
 constexpr int kQuadXC = 384;
 constexpr int kVariant6MaxM = kQuadXC + 1;
 // Children per batch the shapes with small or wide x areas have room for. The
-// slot-free 256-thread x 4 refined variant: the elimination rows Y(x), x < c4 <= M - 2, it keeps in shared memory.
+// slot-free 256-thread x 4 refined variant: the elimination rows Y(x), x < c4 <= M - 2,
+// it keeps in shared memory.
 constexpr int kNoSlotCC = 24;
 constexpr int kNoSlotYC = 160;
 constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1

@@ -16,8 +16,8 @@ constexpr uint32_t kOrder4Pairs = 16384;
 // Packing of A, order 1 and order 2 in one launch (none reads what another writes):
 // blocks [0, nb0) pack, [nb0, nb0 + nb1) fill order 1, the rest order 2; one thread
 // per block of A or subset of colex rank first + i, i < count (the whole order, or
-// the rank range of a range call's top order). Three dependent launches of 3-6 us
-// each before; one of about 7 now.
+// the rank range of a range call's top order). Bound by the launch: about 7 us for all
+// three, 3-6 us each as launches that wait for each other.
 struct Span {
     uint64_t first, count;
 };
@@ -42,12 +42,13 @@ __global__ void __launch_bounds__(FLAT_THREADS) front_kernel(FwdArgs a, bool wp1
     }
 }
 
-// Flat kernel of order 3: one thread per subset of colex rank first + i, i < count.
-template <int MODE, bool DISP>
+// Flat kernel of order 3 for displaced states whose modes do not fit a chunk's shared
+// memory (M > 3213): one thread per subset of colex rank first + i, i < count.
+template <int MODE>
 __global__ void order3_kernel(FwdArgs a, bool write_p0, uint64_t first, uint64_t count) {
     await_previous();
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < count) order3_entry<MODE, DISP>(a, first + i, write_p0);
+    if (i < count) order3_entry<MODE, true>(a, first + i, write_p0);
 }
 
 template <int D, int MODE, int PREC, int NT, int XC, int MINB, bool DISP, int CC = CCAP, int YC = 0>
@@ -290,24 +291,30 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
 // c3, up to 12 operations for each of c2 modes, is then below 5 % of the leaves').
 // kt, FP64: M = 1152 43.4 -> 14.7 ms (36 FP64 instructions an entry: the FP64
 // pipe's own 14.6), M = 200 0.248 -> 0.112, M = 20 26.0 -> 23.5 us, against one
-// thread per subset redoing the elimination. That kernel is left for displaced
-// states whose modes do not fit shared memory.
+// thread per subset redoing the elimination (order3_kernel, left for displaced
+// states whose modes do not fit shared memory).
 template <int MODE, bool DISP>
 static cudaError_t launch_order3(const FwdArgs &a, bool write_p0, int c_lo, int c_hi, cudaStream_t st) {
-    const uint64_t first = binom(c_lo, 3), n = binom(c_hi, 3) - first;
+    [[maybe_unused]] const uint64_t first = binom(c_lo, 3);
+    const uint64_t n = binom(c_hi, 3) - first;
     if (n == 0) return cudaSuccess;
     const uint64_t want = (n / ((uint64_t)a.sms * 16) + 255) / 256 * 256;
     const uint32_t L = want < 256 ? 256 : want > 8192 ? 8192 : (uint32_t)want;
     using Shape = ChunkShape<1, 0, DISP>;
     const size_t smem = chunk_smem(c_hi - 1, L, Shape::PX, Shape::PR);
-    if (smem <= kChunkSmem) return launch_chunk<1, MODE, 0, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
-    return launch_next(!a.ev, order3_kernel<MODE, DISP>, (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS), FLAT_THREADS, 0,
-                       st, a, write_p0, first, n);
+    if constexpr (DISP) {
+        if (smem > kChunkSmem)
+            return launch_next(!a.ev, order3_kernel<MODE>, (unsigned)((n + FLAT_THREADS - 1) / FLAT_THREADS),
+                               FLAT_THREADS, 0, st, a, write_p0, first, n);
+    } else {
+        static_assert(chunk_smem(GBS_MAX_MODES_K3 - 1, 8192, Shape::PX, Shape::PR) <= kChunkSmem, "zero-mean: any M fits");
+    }
+    return launch_chunk<1, MODE, 0, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
 }
 
 // Order 4, top elements in [c_lo, c_hi): by chunks below kOrder4ChunkedZ / R
 // modes (FP64, refined) and, for displaced states, wherever the modes fit shared
-// memory; else by the prefix tree. A chunk forms its leaves' blocks from the
+// memory (they always do: 108 KB at M = 1024); else by the prefix tree. A chunk forms its leaves' blocks from the
 // prefix's pivot rows (8 FP64 or 48 pair operations more a leaf) and needs no
 // slot, queue or batches. kt, us, tree at its best schedule / chunks:
 //   FP64       M = 20 52.7 / 36.4  50 77.7 / 75  100 434 / 391  144 1526 / 1460  300 23500 / 25800
@@ -318,12 +325,12 @@ static cudaError_t launch_order4(const FwdArgs &a, bool write_p0, int c_lo, int 
     using Shape = ChunkShape<2, PREC, DISP>;
     const uint32_t L = a.M < 64 ? kOrder4Pairs / 16 : kOrder4Pairs;  // small tables: split the largest prefixes
     const size_t smem = chunk_smem(a.M - 2, L, Shape::PX, Shape::PR);
-    const int below = DISP ? GBS_MAX_MODES + 1 : PREC == 1 ? kOrder4ChunkedR : kOrder4ChunkedZ;
-    if (a.M < below && smem <= kChunkSmem) {
-        if (c_hi <= 3 || c_hi <= c_lo) return cudaSuccess;
-        return launch_chunk<2, MODE, PREC, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
-    }
-    return launch_tree<4, MODE, PREC, DISP>(a, write_p0, st);
+    constexpr int below = DISP ? GBS_MAX_MODES + 1 : PREC == 1 ? kOrder4ChunkedR : kOrder4ChunkedZ;
+    static_assert(chunk_smem(below - 3, kOrder4Pairs, Shape::PX, Shape::PR) <= kChunkSmem, "the largest chunk fits");
+    if constexpr (!DISP)
+        if (a.M >= below) return launch_tree<4, MODE, PREC, DISP>(a, write_p0, st);
+    if (c_hi <= 3 || c_hi <= c_lo) return cudaSuccess;
+    return launch_chunk<2, MODE, PREC, DISP>(a, write_p0, c_lo, c_hi, L, smem, st);
 }
 
 template <int MODE, bool DISP>

@@ -100,7 +100,6 @@ struct Args {
     R *W;
     const R *kb;           // kappa(i, n) regrouped for p2_block_kernel, or null (p2_kernel then walks every row itself)
     float *At;             // tensor-core product: the step's rows, split and tiled (operands_kernel)
-    const R *hs;           // per-variable half scale s_v / 2, hs[v], v = 1..M
     const R *lead;         // per-variable pairs (kappa'({v}), hs[v]) at lead[2v], lead[2v+1]
     const double *H;       // per-variable log scale ln s_v (the click entropy of mode v - 1)
     unsigned *status;      // status word (ST_* bits), first bytes of the workspace
@@ -176,12 +175,6 @@ __device__ __forceinline__ typename Pair2<R>::T lead(const Args<R> &a, int n) {
 // kappa of the sorted variable set (v_1 < .. < v_d), 1-based.
 template <class R>
 __device__ __forceinline__ R k1(const Args<R> &a, int n) { return a.kap[a.off[1] + (n - 1)]; }
-template <class R>
-__device__ __forceinline__ R k2(const Args<R> &a, int i, int n) { return a.kap[a.off[2] + cb(n - 1, 2) + (i - 1)]; }
-template <class R>
-__device__ __forceinline__ R k3(const Args<R> &a, int j, int i, int n) {
-    return a.kap[a.off[3] + cb(n - 1, 3) + cb(i - 1, 2) + (j - 1)];
-}
 
 // Pair rank -> (hi, lo), hi > lo >= 0 (colex: rank = C(hi, 2) + lo). The root
 // estimate is taken in FP32 (GB300's FP64 pipe is narrow and every lane of the
@@ -434,7 +427,7 @@ constexpr uint32_t tc_idesc(int n) {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// byte offset of element (row r, inner k) of an operand copy with 32-wide K
+// byte offset of element (row r, inner k) of an operand copy of one chunk
 __device__ __forceinline__ uint32_t tc_off(int r, int k) {
     const int core = (r >> 3) * (TC_KC / 4) + (k >> 2);  // core matrix: 8-row group, then 4-wide K slice
     return (uint32_t)((core * 8 + (r & 7)) * 16 + (k & 3) * 4);
@@ -1539,10 +1532,10 @@ SamplerLayout sampler_layout(int M, int K, int S, int precision) {
     size_t off = 256;  // status word first (read by gbs_stream_status)
     L.tab = off;       // S is a multiple of SG: whole groups
     off = a256(off + sampler_tabs(M, K).entries * Ss * es);
-    // W: plain [r][S], or for the tensor-core product hi / lo copies of 32-padded chunks
+    // W: plain [r][S], or for the tensor-core product hi / lo copies of TC_KC-wide chunks
     L.W = off;
     off = a256(off + 2 * ((K >= 4 ? cb(M - 1, 2) : (size_t)M) + 32) * Ss * es);
-    // tensor-core product rows: max over the steps of (row tiles x chunks) x 8192 floats
+    // tensor-core product rows: max over the steps of (row tiles x chunks) x 2 TC_ACH floats
     size_t at = 0;
     if (precision != 0)
         for (int t = 1; t <= M; ++t) {
@@ -1713,7 +1706,6 @@ static cudaError_t run_all(const SamplerCall &c, cudaStream_t st) {
             a.kb = kb;
         }
         a.kap = kf;
-        a.hs = hs;
         a.lead = ldp;
         a.H = H;
     }

@@ -362,7 +362,6 @@ struct TreeShared {
     // children of the current batch
     int c3[CC];
     int xoff[CC + 1];
-    uint32_t lpref[CC + 1];
     // (refined cumulants: subsets without c3, whose bases all children share, first)
     alignas(16) uint64_t baseJ[CC][NQ];
     alignas(16) uint64_t baseT[CC][NQ];
@@ -522,7 +521,7 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
     static_assert(!(DISP && CL), "displaced states run without clusters");
     constexpr bool NOSLOT = YC > 0;
     static_assert(!NOSLOT || (PREC == 1 && !CL), "the slot-free form is the refined path's, without clusters");
-    constexpr bool PAIRS = PREC == 1 && (MODE == MODE_KAPPA || MODE == MODE_SPINK);  // combine_pairs
+    constexpr bool PAIRS = PREC == 1 && (MODE == MODE_KAPPA || MODE == MODE_SPINK);  // combine_products
     const int ccap = ccap_in < CC ? ccap_in : CC;
     using SH = TreeShared<D, XC, DISP, CC, YC>;
     constexpr int NP = SH::NP;
@@ -666,19 +665,13 @@ __device__ __forceinline__ void tree_item(const FwdArgs &a, TreeShared<D, XC, DI
             const int b = tid;
             const int c3 = cfirst - (k0 + b) * nc;
             int xo = 0;
-            uint32_t lp = 0;
             for (int q = 0; q < b; ++q) {
                 const int cq = cfirst - (k0 + q) * nc;
                 xo += cq;
-                lp += (uint32_t)binom2(cq);
             }
             sh.c3[b] = c3;
             sh.xoff[b] = xo;
-            sh.lpref[b] = lp;
-            if (b == nb - 1) {
-                sh.xoff[nb] = xo + c3;
-                sh.lpref[nb] = lp + (uint32_t)binom2(c3);
-            }
+            if (b == nb - 1) sh.xoff[nb] = xo + c3;
             int P[3] = {c3, c4, c5};
             uint64_t bj[NQ], bt[NQ], idxQ[NQ];
             child_bases<NP>(P, M, bj, bt, idxQ);
