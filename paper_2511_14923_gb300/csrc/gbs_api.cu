@@ -121,7 +121,8 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
         return fail(GBS_ERR_INVALID_ARG, "mean must be 8-byte aligned CUDA device (or managed) memory");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     char *w = static_cast<char *>(ws);
-    if (gbs::fault_injected("forward_memset"))
+    const char *const faults = gbs::fault_sites();
+    if (gbs::fault_injected("forward_memset", faults))
         return fail(GBS_ERR_CUDA, "cudaMemsetAsync: injected failure (GBS_FAULT_INJECT=forward_memset)");
     cudaError_t e = cudaMemsetAsync(w + L.status_off, 0, 256, st);
     if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
@@ -167,9 +168,9 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
         a.ev = g_ev;
         g_timing_used = true;
     }
-    e = gbs::fault_injected("forward_launch") ? cudaSetDevice(-1)
-        : mean                                ? gbs::launch_forward_displaced(a, st)
-                                              : gbs::launch_forward(a, st);
+    e = gbs::fault_injected("forward_launch", faults) ? cudaSetDevice(-1)
+        : mean                                        ? gbs::launch_forward_displaced(a, st)
+                                                      : gbs::launch_forward(a, st);
     if (e != cudaSuccess) return fail(GBS_ERR_CUDA, "kernel launch: %s", cudaGetErrorString(e));
     return ok();
 }

@@ -231,8 +231,8 @@ inline cudaError_t launch_next(bool chained, void (*fn)(P...), dim3 grid, dim3 b
 // device index of -1, in the place of their launches), "sampler_no_loads" (the sampler's tensor-core step
 // product issues no copies and gives up its first wait quickly, so the call
 // reports GBS_ERR_TIMEOUT with nothing in flight). Nothing faults on the GPU.
-inline bool fault_injected(const char *site) {
-    const char *env = getenv("GBS_FAULT_INJECT");
+inline const char *fault_sites() { return getenv("GBS_FAULT_INJECT"); }
+inline bool fault_injected(const char *site, const char *env = fault_sites()) {
     if (!env || !*env) return false;
     const size_t n = strlen(site);
     for (const char *p = env; (p = strstr(p, site)) != nullptr; p += n)
