@@ -45,7 +45,8 @@ sys.path.insert(0, ROOT)
 METRIC = "subsets/s and wall time for the order-≤5 M=144 cumulant table, mixed vs FP64 GPU"
 WORKLOAD = ("M=144 kmax=5 click-cumulant table: 72 squeezers r~U[0.8,1.6] on modes 0-71, Haar U(144), "
             "eta_i~U[0.3,0.5], seed 20251116")
-DTYPE = {"fp64": "f64", "fp32r": "f32 determinant steps refined to f64 accuracy; f64 sums"}
+DTYPE = {"fp64": "f64", "fp32r": "f32 pairs (about 46 bits) in the determinant steps below the prefix and in half of the "
+                  "recursion's products; f64 prefix and sums"}
 
 # Executed thread instructions per table entry of the order-4 and order-5 kernels
 # (ncu SASS counters sm__sass_thread_inst_executed_op_{dfma,dadd,dmul,fp32}_pred_on,
@@ -55,8 +56,8 @@ DTYPE = {"fp64": "f64", "fp32r": "f32 determinant steps refined to f64 accuracy;
 # per-item Schur-complement build and per-child eliminations. None = not captured
 # for the kernel as it stands.
 OPS_PER_ENTRY = {
-    ("fp32r", 5): {"dfma": 6.016, "dadd": 2.009, "dmul": 1.014, "fp32": 356.86},
-    ("fp32r", 4): {"dfma": 3.013, "dadd": 4.026, "dmul": 2.026, "fp32": 343.26},
+    ("fp32r", 5): {"dfma": 6.016, "dadd": 2.009, "dmul": 1.014, "fp32": 365.85},
+    ("fp32r", 4): {"dfma": 3.013, "dadd": 4.026, "dmul": 2.026, "fp32": 352.26},
     ("fp64", 5): {"dfma": 36.138, "dadd": 0.001, "dmul": 8.406, "fp32": 4.417},
     ("fp64", 4): {"dfma": 35.888, "dadd": 0.030, "dmul": 8.461, "fp32": 13.032},
 }
@@ -64,7 +65,7 @@ OPS_PER_ENTRY = {
 # order-5 kernel at M=144, by precision and CTA shape (gbs_schedule's variant:
 # 2 = 128 x 6, 4 = 256 x 3), from ncu captures of the calls above; a shape not
 # listed has no figure (None).
-TRAFFIC_BYTES = {("fp32r", 2): 7.447e9 + 4.4696e9, ("fp64", 4): 4.333e9 + 4.3353e9}
+TRAFFIC_BYTES = {("fp32r", 2): 7.525e9 + 4.4731e9, ("fp64", 4): 4.318e9 + 4.3419e9}
 NOMINAL_FP64_FMA_PER_CLK_PER_SM = 2
 NOMINAL_FP32_FMA_PER_CLK_PER_SM = 128
 HBM_FALLBACK_GBS = 6800.0
@@ -431,9 +432,9 @@ def run_batch(precision, steps, warmup, autotune, peaks, sms, sm_mhz):
 # FP64 flops (FMA = 2), FP64-pipe instructions, FP32 instructions; None = not
 # captured (or stale after a kernel change).
 FIT_PHASE_COUNTS = {
-    "p0_recompute": {"fp64_flops": 21461133, "fp64_instr": 13767002, "fp32_instr": 1145365972},
+    "p0_recompute": {"fp64_flops": 21312819, "fp64_instr": 13643882, "fp32_instr": 1118730413},
     "h_table": {"fp64_flops": 5047450, "fp64_instr": 3097150, "fp32_instr": 3758700},
-    "gp0_gather": {"fp64_flops": 118298125, "fp64_instr": 62420875, "fp32_instr": 17132462},
+    "gp0_gather": {"fp64_flops": 118040525, "fp64_instr": 62163275, "fp32_instr": 17081262},
     "gv_scatter": {"fp64_flops": 220049841, "fp64_instr": 179690437, "fp32_instr": 8485702640},
 }
 

@@ -368,8 +368,8 @@ std::map<const void *, Launch> g_launch;
 
 // Default schedule of an untuned batch: the CTA shape the single-instance
 // autotuner picks for large tables on GB300 (128 x 6 refined, 256 x 3 FP64) where
-// every instance fits it. 48 instances of 16 to 128 modes, refined: 15.0 ms at
-// 128 x 6, 16.2 at 256 x 3.
+// every instance fits it. 48 instances of 16 to 128 modes, refined: 15.1 ms at
+// 128 x 6, 8 % more at 256 x 3.
 TreeCfg default_cfg(int precision, int maxM) {
     TreeCfg c = kDefaultCfg;
     if (maxM <= kVariant1MaxM) c.variant = precision == 0 ? 4 : maxM <= kVariant2MaxM ? 2 : 3;

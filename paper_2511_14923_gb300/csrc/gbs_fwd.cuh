@@ -85,12 +85,12 @@ constexpr int kNoSlotYC = 160;
 constexpr int kVariant9MaxM = kNoSlotYC + 1;  // order 4 reaches c4 = M - 1
 // Schedule of an untuned forward call, from sweeps of shape x grain (kt, M = 20 to
 // 300, kmax = 4 and 5; the tuner still finds the last percents):
-//   refined, kmax = 5: 128 x 6 where its x area admits M (M = 144: 10.6 ms against
-//     10.7 at 256 x 3 and 17.7 at 512 x 1; M = 77: 0.64 against 0.66 and 1.2), one
+//   refined, kmax = 5: 128 x 6 where its x area admits M (M = 144: 10.76 ms against
+//     10.81 at 256 x 3 and 14.3 at 512 x 1; M = 77: 0.64 against 0.66 and 1.05), one
 //     item per CTA slot below 128 modes, where a second round of items would wait
 //     for the first, else two; kmax = 4: 256 x 3, two items (M = 144: 0.44 against
 //     0.50 at 128 x 6), but 256 x 4 for the tables without gathers on pairs (P0, M =
-//     100: 85 us against 105; M = 77, kmax = 5: 363 against 370 the call); larger M
+//     100, kmax = 4: 124 us the call against 140); larger M
 //     256 x 3, then 384 x 2;
 //   FP64: the wide 256 x 3, one item per CTA slot (M = 111, kmax = 5: 10.9 against
 //     11.2 at 256 x 2 and 12.3 at 512 x 1; M = 50: 0.32 against 0.34 and 0.47); a

@@ -259,8 +259,8 @@ static cudaError_t launch_tree(const FwdArgs &a_in, bool write_p0, cudaStream_t 
             // 24 warps with 80 registers in 6 CTAs of 4, 3 of 8 (with room for up to 64
             // children a batch, or for more x-entries) or 2 of 12; or 32 warps with 64
             // registers in 4 CTAs. Order 5 runs fastest in the smallest CTAs, whose
-            // batches wait least at their barriers (M = 144: 128 x 6 10.6 ms, 256 x 3
-            // 10.7, 256 x 4 11.6, the shared gathers spilling at 64 registers). Order 4
+            // batches wait least at their barriers (M = 144: 128 x 6 10.76 ms, 256 x 3
+            // 10.81, 256 x 4 12.0, the shared gathers spilling at 64 registers). Order 4
             // of that shape, whose items are small, runs in the wide 256 x 3 one (0.44
             // against 0.50 ms), or in 256 x 4 where it has no such gathers.
             if (v == 2 && D == 5) return launch_tree_v<D, MODE, PREC, 128, kSmallXC, 6, false, kNoSlotCC>(a, write_p0, st);
