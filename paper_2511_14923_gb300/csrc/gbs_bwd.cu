@@ -1021,8 +1021,10 @@ cudaError_t launch_covariance_bwd(const double *Ur, const double *Ui, const doub
                                   const double *V, const double *G, double *dr, double *deta, cudaStream_t st) {
     const size_t smem = sizeof(double) * 4 * (size_t)M;
     if (smem > 48 * 1024) {
+        // the limit is the kernel's: every call sets the one for the largest M, so that no
+        // host thread lowers it between another's two calls
         const cudaError_t e = cudaFuncSetAttribute(covariance_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
+                                                   (int)(sizeof(double) * 4 * GBS_MAX_MODES_K3));
         if (e != cudaSuccess) return e;
     }
     covariance_bwd_kernel<<<M, 256, smem, st>>>(Ur, Ui, r, eta, M, V, G, dr, deta);
