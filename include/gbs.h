@@ -106,7 +106,8 @@ int gbs_unrank(uint64_t r, int d, int *modes_out);
    the current CUDA device; 0 if the arguments are invalid. GBS_FP32_REFINED with
    kmax >= 4 takes 16 bytes more for each entry of the orders below kmax, which the
    cumulant tables read; given a workspace of the GBS_FP64 size, a refined cumulant
-   call fills its table by the FP64 kernels (the other refined calls need no more). */
+   call fills its table by the FP64 kernels, and gbs_autotune tunes those (the other
+   refined calls need no more). */
 size_t gbs_workspace_bytes(int M, int kmax, int precision);
 
 /* Message for the most recent failing call on this host thread ("" if none). */

@@ -601,7 +601,7 @@ def autotune(V, kmax, precision="fp32r", workspace=None) -> float:
     """Tune the prefix-tree schedule for this shape (see gbs_autotune); returns the best ms."""
     V, M = _prep(V)
     out = torch.empty(table_size(M, kmax), dtype=torch.float64, device=V.device)
-    ws = _workspace_for(workspace, M, kmax, precision, V.device)
+    ws = _workspace_for(workspace, M, kmax, precision, V.device, least="fp64")
     st = torch.cuda.current_stream(V.device)
     ms = ctypes.c_float(0.0)
     _check(lib().gbs_autotune(_vp(V), M, kmax, _vp(out), PRECISIONS[precision], ctypes.c_void_p(ws.ptr), ws.nbytes,

@@ -75,9 +75,10 @@ bool uses_pairs(int mode, int kmax, int precision) {
     return precision == GBS_FP32_REFINED && kmax >= 4 && (mode == gbs::MODE_KAPPA || mode == gbs::MODE_SPINK);
 }
 
-// least: accept a workspace without room for the float pairs too (L then has none).
-int check_common(const double *V, int M, int kmax, const void *out, int precision, int mode, void *ws,
-                 size_t ws_bytes, gbs::WsLayout &L, int &sms, bool range, bool least) {
+// A workspace of the FP64 size serves a refined call too: one that would use the float
+// pairs becomes an FP64 call (precision), by the FP64 kernels, which need none.
+int check_common(const double *V, int M, int kmax, const void *out, int &precision, int mode, void *ws,
+                 size_t ws_bytes, gbs::WsLayout &L, int &sms, bool range) {
     if (!valid_mk(M, kmax)) return fail(GBS_ERR_INVALID_ARG, "%s", gbs::shape_message(M, kmax).c_str());
     if (precision != GBS_FP64 && precision != GBS_FP32_REFINED)
         return fail(GBS_ERR_INVALID_ARG, "precision must be GBS_FP64 (0) or GBS_FP32_REFINED (1); got %d", precision);
@@ -94,7 +95,10 @@ int check_common(const double *V, int M, int kmax, const void *out, int precisio
         L = gbs::ws_layout(M, kmax, sms, 0, pairs);
         return range ? range_total(L, M, kmax) : L.total;
     };
-    if (ws_bytes < need() && pairs && least) pairs = false;
+    if (pairs && ws_bytes < need()) {
+        pairs = false;
+        precision = GBS_FP64;
+    }
     if (ws_bytes < need())
         return fail(GBS_ERR_WORKSPACE, "workspace too small: %zu bytes given, %zu needed", ws_bytes, need());
     return GBS_OK;
@@ -113,10 +117,8 @@ int run_forward(int mode, const double *V, int M, int kmax, double *out, int pre
     if (range.on() && (range.c_lo < 0 || range.c_lo > range.c_hi || range.c_hi > M))
         return fail(GBS_ERR_INVALID_ARG, "need 0 <= c_lo <= c_hi <= M; got c_lo=%d c_hi=%d M=%d", range.c_lo,
                     range.c_hi, M);
-    int rc = check_common(V, M, kmax, out, precision, mode, ws, ws_bytes, L, sms, range.on(), true);
+    int rc = check_common(V, M, kmax, out, precision, mode, ws, ws_bytes, L, sms, range.on());
     if (rc != GBS_OK) return rc;
-    // a workspace of the FP64 size: the table by the FP64 kernels, which need no pairs
-    if (uses_pairs(mode, kmax, precision) && L.p0p_off == L.total) precision = GBS_FP64;
     if (mean && (((uintptr_t)mean & 7) || !is_device_ptr(mean)))
         return fail(GBS_ERR_INVALID_ARG, "mean must be 8-byte aligned CUDA device (or managed) memory");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -479,7 +481,7 @@ int gbs_autotune(const double *V, int M, int kmax, double *kappa_out, int precis
                  size_t ws_bytes, void *cuda_stream, float *best_ms_out) {
     gbs::WsLayout L;
     int sms = 0;
-    int rc = check_common(V, M, kmax, kappa_out, precision, gbs::MODE_KAPPA, workspace, ws_bytes, L, sms, false, false);
+    int rc = check_common(V, M, kmax, kappa_out, precision, gbs::MODE_KAPPA, workspace, ws_bytes, L, sms, false);
     if (rc != GBS_OK) return rc;
     char *w = static_cast<char *>(workspace);
     gbs::FwdArgs a{};

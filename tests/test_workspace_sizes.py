@@ -48,6 +48,8 @@ def test_fp64_sized_workspace_serves_refined_calls(kmax):
         want = f(V, kmax, prec)
         assert torch.equal(got, want)
         assert torch.equal(part, want[first:])
+    assert gbs.autotune(V, kmax, "fp32r", workspace=ws) > 0
+    assert torch.equal(gbs.cumulants(V, kmax, "fp32r", workspace=ws), gbs.cumulants(V, kmax, "fp64" if kmax >= 4 else "fp32r"))
     with pytest.raises(gbs.GbsError):
         small = gbs.Workspace(M - 1, kmax, "fp32r")
         small.nbytes = ws.nbytes - 1
